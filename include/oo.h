@@ -281,7 +281,8 @@ oo_status oo_stencil_noalloc_check(oo_ctx *ctx);
  * results, so tuning changes speed only.  Outputs the chosen variant and,
  * if ms_per_variant is not NULL, the mean sweep time of each variant
  * (OO_STENCIL_VARIANTS entries).  Without tuning a grid uses the default
- * rule (variant 1 when K - 1 > 64, else 4), which is the tuner's choice at
+ * rule (variant 1, or 4 where 64-wide tiles pad the rows much less than
+ * 128-wide ones), which is the tuner's choice at
  * the benchmarked sizes.  Synchronous.                                     */
 enum { OO_STENCIL_VARIANTS = 5 };
 oo_status oo_tune_stencil(oo_ctx *ctx, int I, int J, int K, int *variant, double *ms_per_variant);
@@ -311,7 +312,7 @@ oo_status oo_inject_wait_timeout(oo_ctx *ctx, int what);
 /* Context options (per context, never read from the process environment):
  *   OO_OPT_JACOBI_FUSED     -1 (default) fuse all iterations of the all-GPU
  *                           iteration nests into one cooperative launch for
- *                           grids of at most 2^20 points; 0 never; 1
+ *                           grids of at most 1.8 M interior points; 0 never; 1
  *                           whenever the placement and copies allow it.
  *   OO_OPT_STENCIL_VARIANT  -1 (default) the oo_tune_stencil choice for the
  *                           grid, else the default rule; 0 ..

@@ -18,14 +18,14 @@
 //
 // N2 is a persistent, warp-specialised kernel.  One producer thread streams
 // tiles with TMA (cp.async.bulk.tensor) into shared memory: for every plane i
-// of a work unit, the twelve coefficient tiles (TK x TJ) and one p tile with
+// of a run, the twelve coefficient tiles (TK x TJ) and one p tile with
 // a one-point halo in j and a 4-float-aligned halo in k.  Consumer warps
-// march i through the unit with the three p planes i-1, i, i+1 resident in a
+// march i through the run with the three p planes i-1, i, i+1 resident in a
 // ring, compute the update in float-float arithmetic (error-free sums and
 // FMA products, about 44 significant bits, rounded once at the store), and
-// accumulate ss^2 in float-float per thread and in FP64 per warp and unit.
-// Every unit's partial residuals go to scratch; the last CTA to finish sums
-// them in unit order, so the residual is deterministic.  Five tile variants
+// accumulate ss^2 in float-float per thread and run, then in FP64 per warp.
+// Every warp's partial residual goes to scratch; the last CTA to finish sums
+// them in a fixed order, so the residual is deterministic.  Five tile variants
 // (tile shape, consumer warps, points per thread, CTAs per SM) compute the
 // same values; a rule by row length picks one unless a plan is given one
 // (the autotuner, oo_tune_stencil).  Every mbarrier wait is bounded; a wait that runs out
@@ -266,6 +266,50 @@ __global__ void bc_k_kernel(float *p, int rows, int K, int pitch) {
     }
 }
 
+// N4 and N5 in one launch on the array a stencil sweep writes, for runs in
+// which p and wrk2 exchange roles (launch_bc_faces): items are the float4
+// chunks of the i / j face rows, then the two ends of every interior row.
+// Bound by launch latency (3 us alone), so it is launched to run beside the
+// sweep, whose interior stores it does not touch; it ends only after the
+// sweep has (griddepcontrol.wait), so what follows it follows both.
+__global__ void bc_faces_kernel(float *p, int I, int J, int K, int pitch) {
+    const unsigned chunks = (unsigned)(K + 3) / 4u;
+    const unsigned face_rows = 2u * J + 2u * (I - 2);
+    const size_t n_chunks = (size_t)face_rows * chunks, total = n_chunks + (size_t)(I - 2) * (J - 2);
+    const size_t step = (size_t)gridDim.x * blockDim.x;
+    asm volatile("griddepcontrol.launch_dependents;");  // the next sweep may set itself up
+    const float g0 = dirichlet_dev(0, K), g1 = dirichlet_dev(K - 1, K);
+    for (size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x; x < total; x += step) {
+        if (x >= n_chunks) {
+            const unsigned r = (unsigned)(x - n_chunks);
+            float *row = p + ((size_t)(1 + r / (J - 2)) * J + 1 + r % (J - 2)) * pitch;
+            row[0] = g0;
+            row[K - 1] = g1;
+            continue;
+        }
+        const unsigned c = (unsigned)(x % chunks), r = (unsigned)(x / chunks);
+        int i, j;
+        if (r < 2u * J) {
+            i = (r < (unsigned)J) ? 0 : I - 1;
+            j = (int)(r % (unsigned)J);
+        } else {
+            const unsigned q = r - 2u * J;
+            i = 1 + (int)(q / 2u);
+            j = (q % 2u) ? J - 1 : 0;
+        }
+        const size_t off = ((size_t)i * J + j) * pitch + 4u * c;
+        const int k = 4 * (int)c;
+        if (k + 3 < K) {
+            reinterpret_cast<float4 *>(p + off)[0] =
+                make_float4(dirichlet_dev(k, K), dirichlet_dev(k + 1, K), dirichlet_dev(k + 2, K),
+                            dirichlet_dev(k + 3, K));
+        } else {
+            for (int e = 0; e < 4 && k + e < K; ++e) p[off + e] = dirichlet_dev(k + e, K);
+        }
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 int grid_for(size_t work, int threads, int max_blocks) {
     const size_t b = (work + threads - 1) / threads;
     return (int)std::max<size_t>(1, std::min<size_t>(b, (size_t)max_blocks));
@@ -320,152 +364,296 @@ void launch_bc_k(const JacobiDims &d, float *p, cudaStream_t s) {
     OO_CUDA_TRY(cudaGetLastError());
 }
 
+void launch_bc_faces(const JacobiDims &d, float *p, cudaStream_t s) {
+    const size_t work = (size_t)(2 * d.J + 2 * (d.I - 2)) * ((d.K + 3) / 4) + (size_t)(d.I - 2) * (d.J - 2);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid_for(work, 256, sm_count()));
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    OO_CUDA_TRY(cudaLaunchKernelEx(&cfg, bc_faces_kernel, p, d.I, d.J, d.K, d.pitch));
+}
+
 // ======================================================= fused iterations
 // All iterations of the all-GPU iteration nests (N2 stencil, N3 copy-back,
 // N4 / N5 boundary) in one cooperative launch, for grids small enough that
-// launch latency, not HBM, bounds the separate kernels.  Per iteration:
-// the stencil over the interior (each thread a strided set of points, the
-// same float-float arithmetic as the tiled kernel, term by term), a grid
-// barrier, block 0 sums the per-block FP64 residual partials in block
-// order, every point of p is rewritten (interior = wrk2, faces = g(k), i.e.
-// N3, N4 and N5), a second grid barrier.  Barrier waits are bounded: a wait
-// that runs out sets the error word and every block leaves at its next
-// barrier.
+// launches, not HBM, bound the separate kernels.
+//
+// What bounds it: at 33 x 33 x 65 an SM holds 400 points, less than one per
+// thread, so an iteration is one point's chain (about 280 float-float
+// instructions, 19 loads) plus one exchange between SMs.  So:
+//   - CTA b (one per SM) owns the same contiguous range of interior points
+//     in every iteration; their coefficients are read once and stay in its
+//     shared memory (12 x 4 bytes a point, the points beyond it read theirs
+//     from L2);
+//   - p and wrk2 exchange roles from one iteration to the next instead of
+//     being copied: both hold g(k) on the faces from the setup nest, the
+//     stencil writes the interior, so the array written is p after N3, N4
+//     and N5;
+//   - a CTA waits for the CTAs that own points its own points touch
+//     (index distance up to one plane, one row and one point), not for the
+//     grid: each CTA publishes the number of iterations it has finished, and
+//     that a neighbour has finished iteration t says both that its new
+//     values are there and that it no longer reads the array iteration
+//     t + 1 overwrites;
+//   - one warp publishes and waits, another sums the residual while the
+//     sixteen others compute: FP64 adds run at 1/59 of the FP32 rate, and
+//     512 threads reducing in FP64 take as long as the stencil itself.
+// Two grid barriers, a copy pass and the coefficients from L2 in every
+// iteration took 14.2 us at 33 x 33 x 65; this takes 3.4 us, of which about
+// 3 are the exchange (a single CTA's worth of points takes 3.2).
+// Waits are bounded: one that runs out sets the error word and every CTA
+// leaves at its next wait.
 namespace {
+
+constexpr int kFusedThreads = 512;               // compute threads; two more warps serve them
+constexpr int kFusedLine = 32;                   // words between two CTAs' words
+constexpr int kFusedChunk = 64;                  // iterations between residual sums
+constexpr size_t kFusedSmem = 216 * 1024;        // coefficients of up to 4608 points of a CTA
 
 struct FusedArgs {
     const float *coef[NCOEF];
-    float *p, *wrk2;
+    float *p, *wrk2;        // even iterations read p and write wrk2, odd ones the reverse
     double *res;
-    double *partials;       // gridDim.x
-    unsigned *ctl;          // [0] arrivals, [1] generation, [2] error
+    double *partials;       // 2 chunks x kFusedChunk iterations x gridDim.x
+    unsigned *err;          // error word
+    unsigned *done;         // per CTA (and one line never written): iterations finished
+    unsigned *summed;       // per CTA, in the same lines: chunks whose partials are written
     int I, J, K, pitch, iters;
+    int cap;                // points whose coefficients fit the shared memory
     float omega;
-    unsigned barrier_extra;  // fault injection: arrivals awaited beyond the grid (0 in normal runs)
+    unsigned wait_extra;    // fault injection: CTAs awaited beyond the grid (0 in normal runs)
 };
 
-__device__ __forceinline__ bool fused_grid_barrier(unsigned *ctl, unsigned extra) {
-    __syncthreads();
-    __shared__ int ok_s;
-    if (threadIdx.x == 0) {
-        volatile unsigned *gen = ctl + 1, *err = ctl + 2;
-        const unsigned g = *gen;
-        __threadfence();
-        if (atomicAdd(ctl, 1u) == gridDim.x - 1 + extra) {
-            atomicExch(ctl, 0u);
-            __threadfence();
-            atomicAdd(ctl + 1, 1u);
-        } else {
-            const long long t0 = clock64();
-            while (*gen == g) {
-                if (*err) break;
+template <int THREADS>
+__device__ __forceinline__ void bar_named(int id) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(THREADS) : "memory");
+}
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+// publish: what this thread has seen and written is visible to who reads v
+__device__ __forceinline__ void st_release(unsigned *p, unsigned v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// One warp waits (bounded) until the words of CTAs [lo, hi] have all reached
+// `want`; false if a wait ran out, here or elsewhere.  A CTA's words have a
+// 128-byte line of their own: with all of them in a few lines the polls of
+// 152 CTAs held up the stores they waited for (33 x 33 x 65: 6.8 us an
+// iteration, 3.5 us so).
+__device__ __forceinline__ bool fused_wait(const unsigned *words, int lo, int hi, unsigned want, unsigned *err) {
+    bool ok = true;
+    for (int c = lo + (int)(threadIdx.x & 31); c <= hi; c += 32) {
+        const unsigned *word = words + (size_t)c * kFusedLine;
+        if ((int)(ld_relaxed(word) - want) >= 0) continue;
+        const long long t0 = clock64();
+        for (unsigned n = 1; ok && (int)(ld_relaxed(word) - want) < 0; ++n)
+            if (n % 64 == 0) {
+                if (ld_relaxed(err)) ok = false;
                 if (clock64() - t0 > kWaitLimitCycles) {
-                    atomicOr(ctl + 2, 1u);
-                    break;
+                    atomicOr(err, 1u);
+                    ok = false;
+                }
+            }
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    fence_gpu();  // what the awaited CTAs wrote is read after this
+    return ok;
+}
+
+__global__ void __launch_bounds__(kFusedThreads + 64, 1) jacobi_fused_kernel(FusedArgs a) {
+    extern __shared__ float coef_s[];            // [NCOEF][cap]
+    __shared__ float2 ss_s[2][kFusedThreads];    // each thread's residual, of an even / odd iteration
+    __shared__ int ok_s;
+    constexpr int kAll = kFusedThreads + 64, kSync = kFusedThreads + 32;
+    const int J = a.J, Ji = J - 2, Ki = a.K - 2;
+    const long long nint = (long long)(a.I - 2) * Ji * Ki;
+    const int G = gridDim.x, b = blockIdx.x;
+    const long long q0 = nint * b / G;
+    const int n = (int)(nint * (b + 1) / G - q0);
+    const size_t sj = a.pitch, si = (size_t)J * a.pitch;
+    const int lane = threadIdx.x & 31;
+
+    // Barrier 1: iteration `it` of this CTA is stored (every warp).  Barrier 2:
+    // the neighbours' is too, or ok_s is false (all but the residual warp).
+    // After a failure barrier 1 is passed once more, where the residual warp
+    // reads ok_s.
+    if (threadIdx.x >= kSync) {
+        // ------------------------------------------------ residual warp
+        bool ok = true;
+        for (int it = 0; it < a.iters; ++it) {
+            bar_named<kAll>(1);
+            if (it > 0 && !ok_s) return;
+            if (!ok) continue;
+            double v = 0.0;
+#pragma unroll 4
+            for (int t = lane; t < kFusedThreads; t += 32) {
+                const float2 s = ss_s[it & 1][t];
+                v += (double)s.x + (double)s.y;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            const int chunk = it / kFusedChunk, at = it % kFusedChunk;
+            double *part = a.partials + (size_t)(chunk & 1) * kFusedChunk * G;
+            if (lane == 0) part[(size_t)at * G + b] = v;
+            if (at == kFusedChunk - 1 || it == a.iters - 1) {
+                // every CTA's partials of the chunk: CTA b sums iterations b,
+                // b + G, ... of it.  The other chunk's buffer is free again
+                // when every CTA has come this far.
+                if (lane == 0) st_release(a.summed + b * kFusedLine, chunk + 1);
+                ok = fused_wait(a.summed, 0, G - 1, chunk + 1, a.err);
+                for (int x = b; ok && x <= at; x += G) {
+                    double sum = 0.0;
+                    for (int c = lane; c < G; c += 32) sum += __ldcg(part + (size_t)x * G + c);
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                    if (lane == 0) a.res[(size_t)chunk * kFusedChunk + x] = sum;
                 }
             }
         }
-        __threadfence();
-        ok_s = *err == 0;
+        return;
     }
-    __syncthreads();
-    return ok_s != 0;
+    if (threadIdx.x >= kFusedThreads) {
+        // ------------------------------------------------ exchange warp
+        const long long D = (long long)Ji * Ki + Ki + 1;  // how far a point's update reaches
+        auto owner = [&](long long q) { return (int)(((q + 1) * G - 1) / nint); };
+        const int lo = owner(max(0ll, q0 - D)), hi = owner(min(nint - 1, q0 + n - 1 + D));
+        for (int it = 0; it < a.iters; ++it) {
+            bar_named<kAll>(1);
+            if (lane == 0) st_release(a.done + b * kFusedLine, it + 1);
+            const bool ok = fused_wait(a.done, lo, it == 0 ? hi + (int)a.wait_extra : hi, it + 1, a.err);
+            if (lane == 0) ok_s = ok;
+            bar_named<kSync>(2);
+            if (!ok) {
+                if (it + 1 < a.iters) bar_named<kAll>(1);
+                return;
+            }
+        }
+        return;
+    }
+
+    // ----------------------------------------------------- compute warps
+    // this thread's points q0 + tid, + 512, ...: (i, j, k) of the first, and
+    // the step to the next as (di, dj, dk)
+    const int tid = threadIdx.x;
+    const long long first = min(nint - 1, q0 + tid);
+    const int k_first = 1 + (int)(first % Ki), j_first = 1 + (int)(first / Ki % Ji), i_first = 1 + (int)(first / Ki / Ji);
+    const int dk = kFusedThreads % Ki, dj = kFusedThreads / Ki % Ji, di = kFusedThreads / Ki / Ji;
+    auto advance = [&](int &i, int &j, int &k) {
+        k += dk;
+        if (k > Ki) {
+            k -= Ki;
+            ++j;
+        }
+        j += dj;
+        if (j > Ji) {
+            j -= Ji;
+            ++i;
+        }
+        i += di;
+    };
+    {
+        int i = i_first, j = j_first, k = k_first;
+        for (int q = tid; q < min(n, a.cap); q += kFusedThreads) {
+            const size_t c = (size_t)i * si + (size_t)j * sj + k;
+#pragma unroll
+            for (int x = 0; x < NCOEF; ++x) coef_s[x * a.cap + q] = a.coef[x][c];
+            advance(i, j, k);
+        }
+    }
+    for (int it = 0; it < a.iters; ++it) {
+        const float *src = it & 1 ? a.wrk2 : a.p;
+        float *dst = it & 1 ? a.p : a.wrk2;
+        float RH = 0.0f, RL = 0.0f;
+        int i = i_first, j = j_first, k = k_first;
+        for (int q = tid; q < n; q += kFusedThreads) {
+            const size_t c = (size_t)i * si + (size_t)j * sj + k;
+            PWin W, C, E;
+            load_pwin<true>(src, c - si, sj, false, W);
+            load_pwin<true>(src, c, sj, true, C);
+            load_pwin<true>(src, c + si, sj, false, E);
+            float cf[NCOEF];
+            if (q < a.cap) {
+#pragma unroll
+                for (int x = 0; x < NCOEF; ++x) cf[x] = coef_s[x * a.cap + q];
+            } else {
+#pragma unroll
+                for (int x = 0; x < NCOEF; ++x) cf[x] = __ldg(a.coef[x] + c);
+            }
+            dst[c] = stencil_point_core(cf, W, C, E, a.omega, RH, RL);
+            advance(i, j, k);
+        }
+        ss_s[it & 1][tid] = make_float2(RH, RL);
+        bar_named<kAll>(1);
+        bar_named<kSync>(2);
+        if (!ok_s) {
+            if (it + 1 < a.iters) bar_named<kAll>(1);
+            return;
+        }
+    }
 }
 
-__global__ void __launch_bounds__(512, 1) jacobi_fused_kernel(FusedArgs a) {
-    __shared__ double red[16];
-    const int I = a.I, J = a.J, K = a.K, Ji = J - 2, Ki = K - 2;
-    const int nint = (I - 2) * Ji * Ki, nall = I * J * K;
-    const int stride = gridDim.x * blockDim.x, tid0 = blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t sj = a.pitch, si = (size_t)J * a.pitch;
-    const float omega = a.omega;
-    for (int it = 0; it < a.iters; ++it) {
-        // ---- N2: stencil on the interior
-        float RH = 0.0f, RL = 0.0f;
-        for (int x = tid0; x < nint; x += stride) {
-            const int k = 1 + x % Ki, r = x / Ki, j = 1 + r % Ji, i = 1 + r / Ji;
-            stencil_point_ff(a.coef, a.p, (size_t)i * si + (size_t)j * sj + k, si, sj, omega, a.wrk2, RH, RL);
-        }
-        double v = (double)RH + (double)RL;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double b = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += red[w];
-            a.partials[blockIdx.x] = b;
-        }
-        if (!fused_grid_barrier(a.ctl, a.barrier_extra)) return;
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            double sum = 0.0;
-            for (int b = 0; b < (int)gridDim.x; ++b) sum += __ldcg(&a.partials[b]);
-            a.res[it] = sum;
-        }
-        // ---- N3 copy-back (interior), N4 / N5 faces = g(k)
-        for (int x = tid0; x < nall; x += stride) {
-            const int k = x % K, r = x / K, j = r % J, i = r / J;
-            const size_t c = (size_t)i * si + (size_t)j * sj + k;
-            const bool interior = i >= 1 && i <= I - 2 && j >= 1 && j <= J - 2 && k >= 1 && k <= K - 2;
-            a.p[c] = interior ? __ldcg(&a.wrk2[c]) : dirichlet_dev(k, K);
-        }
-        if (!fused_grid_barrier(a.ctl, a.barrier_extra)) return;
-    }
-}
+// control block: a line with the error word, one per CTA and one more, then the partials
+size_t fused_words_bytes() { return (size_t)(sm_count() + 2) * kFusedLine * 4; }
 
 }  // namespace
 
-size_t jacobi_fused_ctl_bytes() { return 256 + (size_t)sm_count() * 8; }
+size_t jacobi_fused_ctl_bytes() { return fused_words_bytes() + (size_t)2 * kFusedChunk * sm_count() * 8; }
 
 bool jacobi_fused_eligible(const JacobiDims &d, int option) {
     if (option == 0) return false;
     const long long nall = (long long)d.I * d.J * d.K;
     if (option == 1) return nall < (1ll << 31);
-    // measured (all iteration nests, 100 iterations): fused 0.74 vs 1.17 ms at
-    // 33 x 33 x 65, 2.73 vs 2.87 ms at 65 x 65 x 129, but 5.36 vs 4.83 ms at
-    // 97 x 97 x 193, where the tiled kernels' bandwidth wins
-    return nall <= (1ll << 20);
+    // Interior points up to which one launch wins over two per iteration
+    // (us an iteration, 100 iterations): 8.4 against 16.0 at 65 x 65 x 129
+    // (0.5 M), 19.5 against 26.7 at 60 x 250 x 97 (1.4 M), 24.1 against 28.3
+    // at 97 x 97 x 193 (1.7 M), 30.4 against 29.9 at 129^3 (2.0 M), where
+    // most coefficients no longer fit the shared memories.
+    return (long long)(d.I - 2) * (d.J - 2) * (d.K - 2) <= 1800000;
 }
 
-void launch_jacobi_fused(const JacobiDims &d, const float *const coef[NCOEF], float *p, float *wrk2, float omega,
-                         int iters, double *res_dev, void *ctl, cudaStream_t s, bool inject_timeout) {
+float *launch_jacobi_fused(const JacobiDims &d, const float *const coef[NCOEF], float *p, float *wrk2, float omega,
+                           int iters, double *res_dev, void *ctl, cudaStream_t s, bool inject_timeout) {
     OO_REQUIRE((long long)d.I * d.J * d.K < (1ll << 31), OO_EINVAL, "grid too large for the fused iterations");
-    if (iters <= 0) return;
-    // one 512-thread block per SM: every grid barrier is sm_count() arrivals
-    // on one counter (thousands of small blocks made the barriers the cost)
-    static std::atomic<int> fits{-1};
-    if (fits.load() < 0) {
-        int b = 0;
-        OO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, jacobi_fused_kernel, 512, 0));
-        fits.store(b >= 1 ? 1 : 0);
-    }
-    OO_REQUIRE(fits.load() == 1, OO_ECUDA, "fused Jacobi kernel does not fit an SM");
-    const long long nall = (long long)d.I * d.J * d.K;
-    const int grid = (int)std::max<long long>(1, std::min<long long>(sm_count(), (nall + 511) / 512));
+    if (iters <= 0) return p;
+    static std::atomic<uint64_t> attr{0};
+    set_smem_limit_once((const void *)jacobi_fused_kernel, kFusedSmem, attr);
+    // one CTA per SM, at least half a point per thread (fewer CTAs, fewer to wait for)
+    const long long nint = (long long)(d.I - 2) * (d.J - 2) * (d.K - 2);
+    const int grid = (int)std::max<long long>(1, std::min<long long>(sm_count(), (nint + 255) / 256));
+    const long long per_cta = (nint + grid - 1) / grid;
     FusedArgs a{};
     for (int q = 0; q < NCOEF; ++q) a.coef[q] = coef[q];
     a.p = p;
     a.wrk2 = wrk2;
     a.res = res_dev;
-    a.ctl = static_cast<unsigned *>(ctl);
-    a.partials = reinterpret_cast<double *>(static_cast<char *>(ctl) + 256);
+    a.err = static_cast<unsigned *>(ctl);
+    a.done = a.err + kFusedLine;
+    a.summed = a.done + 1;
+    a.partials = reinterpret_cast<double *>(static_cast<char *>(ctl) + fused_words_bytes());
     a.I = d.I;
     a.J = d.J;
     a.K = d.K;
     a.pitch = d.pitch;
     a.iters = iters;
     a.omega = omega;
-    a.barrier_extra = inject_timeout ? 1u : 0u;  // one arrival that never comes
-    OO_CUDA_TRY(cudaMemsetAsync(ctl, 0, 16, s));
+    a.cap = (int)std::min<long long>(per_cta, kFusedSmem / (NCOEF * sizeof(float)));
+    a.wait_extra = inject_timeout ? 1u : 0u;  // a CTA that never comes
+    const size_t smem = (size_t)a.cap * NCOEF * sizeof(float);
+    OO_CUDA_TRY(cudaMemsetAsync(ctl, 0, fused_words_bytes(), s));
     void *args[] = {&a};
-    OO_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)jacobi_fused_kernel, dim3(grid), dim3(512), args, 0, s));
-}
-
-unsigned jacobi_fused_check(void *ctl, cudaStream_t s) {
-    unsigned e = 0;
-    OO_CUDA_TRY(cudaMemcpyAsync(&e, static_cast<char *>(ctl) + 8, 4, cudaMemcpyDeviceToHost, s));
-    OO_CUDA_TRY(cudaStreamSynchronize(s));
-    return e;
+    // cooperative: every CTA is resident (the launch fails otherwise), so the waits end
+    OO_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)jacobi_fused_kernel, dim3(grid), dim3(kFusedThreads + 64),
+                                            args, smem, s));
+    return iters & 1 ? wrk2 : p;
 }
 
 // ================================================================== stencil
@@ -476,10 +664,11 @@ struct StencilMaps {
 
 struct StencilArgs {
     int I, J, K, pitch;
-    int n_kt, n_jt, n_seg, n_units;
+    int n_kt;
+    int whole, n_col, seg, i_cut, tail;  // work split (Runs)
     float omega;
     float *wrk2;
-    double *partials;   // n_units
+    double *partials;   // consumer warps x CTAs
     unsigned *counter;  // CTAs finished (reset by the last one)
     unsigned *err;      // error bits
     double *res;        // FP64 residual of this sweep
@@ -487,9 +676,9 @@ struct StencilArgs {
 
 namespace {
 
-// residual partial slots per work unit in the scratch array: one per
-// consumer warp, so no variant may have more consumer warps than this
-constexpr int kMaxConsumerWarps = 16;
+// residual partial slots in the scratch array: one per consumer warp of
+// every CTA, so no variant may have more of either than this
+constexpr int kMaxConsumerWarps = 16, kMaxCtasPerSm = 2;
 
 template <int TK, int TJ>
 struct Tile {
@@ -501,17 +690,58 @@ struct Tile {
     static constexpr uint32_t CBYTES = NCOEF * CTILE * 4;
 };
 
-__device__ __forceinline__ void decode_unit(const StencilArgs &a, int u, int I, int TK, int TJ,
-                                            int &k0, int &j0, int &ib, int &ie) {
-    const int kt = u % a.n_kt;
-    const int jt = (u / a.n_kt) % a.n_jt;
-    const int sg = u / (a.n_kt * a.n_jt);
-    k0 = kt * TK;
-    j0 = 1 + jt * TJ;
-    const long long span = I - 2;
-    ib = 1 + (int)(span * sg / a.n_seg);
-    ie = 1 + (int)(span * (sg + 1) / a.n_seg);
-}
+// Work split.  The (k tile, j tile) columns of the interior, k tiles
+// fastest, go to the CTAs like this: `whole` rounds of one column per CTA,
+// then the n_col columns left, cut at plane i_cut: `seg` CTAs march an equal
+// segment of a column below the cut each, the `tail` CTAs that are left share
+// the planes above it (column after column, one contiguous range per CTA), and
+// the cut is where both take equally long (fill_stencil_plan).  So every CTA
+// is busy to the end, and most of them are at about the same plane as their
+// neighbours' CTAs, whose halo rows they then find in L2.  Measured at 257 x
+// 257 x 513 / 129 x 129 x 257 with the launches of an iteration: equal
+// segments only, dealt out in rounds, 327 / 56.5 us; one contiguous range of
+// all tile planes per CTA 336 / 48.9 us (its CTAs are at unrelated planes, p
+// is read 2.5 times from HBM); this split 303 / 47.6 us.
+// next(): the runs of planes of one column that CTA b marches through, in order.
+struct Runs {
+    int step, b;
+    long long pos, end;     // a tail CTA's range of tile planes above the cut
+    __device__ __forceinline__ explicit Runs(int b_) : step(0), b(b_), pos(0), end(0) {}
+    __device__ __forceinline__ bool next(const StencilArgs &a, int TK, int TJ, int &k0, int &j0, int &ib, int &ie) {
+        const int span = a.I - 2;
+        int col, i0, i1;
+        if (step < a.whole) {
+            col = step * (int)gridDim.x + b;
+            i0 = 0;
+            i1 = span;
+        } else if (b < a.seg * a.n_col) {
+            if (step > a.whole) return false;
+            const int s = b / a.n_col;
+            col = b % a.n_col;
+            i0 = (int)((long long)a.i_cut * s / a.seg);
+            i1 = (int)((long long)a.i_cut * (s + 1) / a.seg);
+        } else {
+            const int t = b - a.seg * a.n_col, h = span - a.i_cut;
+            if (step == a.whole) {
+                if (t >= a.tail) return false;
+                pos = (long long)a.n_col * h * t / a.tail;
+                end = (long long)a.n_col * h * (t + 1) / a.tail;
+            }
+            if (pos >= end) return false;
+            col = (int)(pos / h);
+            i0 = a.i_cut + (int)(pos % h);
+            i1 = (int)min((long long)span, i0 + end - pos);
+            pos += i1 - i0;
+        }
+        if (step >= a.whole) col += a.whole * (int)gridDim.x;
+        ++step;
+        k0 = col % a.n_kt * TK;
+        j0 = 1 + col / a.n_kt * TJ;
+        ib = 1 + i0;
+        ie = 1 + i1;
+        return true;
+    }
+};
 
 // INJ (tests of the bounded waits only): the producer never issues its first
 // p-tile copy, so the consumers' wait for it runs out; a separate
@@ -520,7 +750,8 @@ template <int TK, int TJ, int NCW, int DC, int DP, int PPT, int MINB, bool INJ>
 __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
     stencil_kernel(const __grid_constant__ StencilMaps maps, const StencilArgs a) {
     using T = Tile<TK, TJ>;
-    static_assert(NCW <= kMaxConsumerWarps, "more consumer warps than partial slots per unit");
+    static_assert(NCW <= kMaxConsumerWarps, "more consumer warps than partial slots per CTA");
+    static_assert(MINB <= kMaxCtasPerSm, "more CTAs per SM than partial slots");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // TMA destinations need 128-byte alignment; the launch adds 128 bytes of slack
     unsigned char *smem_base = reinterpret_cast<unsigned char *>(
@@ -535,6 +766,8 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
     int *last_flag = const_cast<int *>(reinterpret_cast<volatile int *>(abort_flag + 1));
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // a face pass launched behind this sweep (launch_bc_faces) may run beside it
+    asm volatile("griddepcontrol.launch_dependents;");
     if (threadIdx.x == 0) {
         for (int c = 0; c < DC; ++c) {
             mbar_init(smem_u32(&full_c[c]), 1);
@@ -550,7 +783,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
     }
     __syncthreads();
 
-    const int I = a.I, J = a.J, K = a.K;
+    const int J = a.J, K = a.K;
 
     if (warp == NCW) {
         // ------------------------------------------------------ producer
@@ -559,9 +792,31 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
             const uint64_t pol_p = policy_evict_last();
             uint32_t cfill = 0, pfill = 0;
             bool ok = true;
-            for (int u = blockIdx.x; ok && u < a.n_units; u += gridDim.x) {
-                int k0, j0, ib, ie;
-                decode_unit(a, u, I, TK, TJ, k0, j0, ib, ie);
+            // the twelve coefficient tiles of plane i into the next free slot
+            auto load_coef = [&](int k0, int j0, int i) {
+                const uint32_t slot = cfill % DC, use = cfill / DC;
+                if (use > 0 && !mbar_wait(smem_u32(&empty_c[slot]), (use - 1) & 1, abort_flag, a.err, 2u))
+                    return false;
+                const uint32_t bar = smem_u32(&full_c[slot]);
+                mbar_expect_tx(bar, T::CBYTES);
+                float *dst = coef_s + (size_t)slot * NCOEF * T::CTILE;
+#pragma unroll
+                for (int c = 0; c < NCOEF; ++c)
+                    tma_load_3d(smem_u32(dst + c * T::CTILE), &maps.coef[c], k0, j0, i, bar, pol_stream);
+                ++cfill;
+                return true;
+            };
+            // A sweep launched to overlap its predecessor's end (launch_stencil,
+            // `chained`) may fill its coefficient ring -- no launch writes those
+            // arrays then -- before it waits for the predecessor's p.
+            Runs runs(blockIdx.x);
+            int k0, j0, ib, ie;
+            bool more = runs.next(a, TK, TJ, k0, j0, ib, ie);
+            for (int i = ib; more && i < ie && i < ib + DC; ++i) load_coef(k0, j0, i);
+            uint32_t ahead = cfill;  // coefficient planes of this run already loaded
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("fence.proxy.async.global;" ::: "memory");
+            for (; ok && more; more = runs.next(a, TK, TJ, k0, j0, ib, ie), ahead = 0) {
                 for (int q = ib - 1; q <= ie; ++q) {
                     {
                         const uint32_t slot = pfill % DP, use = pfill / DP;
@@ -578,21 +833,11 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
                         }
                         ++pfill;
                     }
-                    if (q >= ib + 1) {
-                        const uint32_t slot = cfill % DC, use = cfill / DC;
-                        if (use > 0 &&
-                            !mbar_wait(smem_u32(&empty_c[slot]), (use - 1) & 1, abort_flag, a.err, 2u)) {
+                    if (q >= ib + 1 && q - 1 - ib >= (int)ahead) {
+                        if (!load_coef(k0, j0, q - 1)) {
                             ok = false;
                             break;
                         }
-                        const uint32_t bar = smem_u32(&full_c[slot]);
-                        mbar_expect_tx(bar, T::CBYTES);
-                        float *dst = coef_s + (size_t)slot * NCOEF * T::CTILE;
-#pragma unroll
-                        for (int c = 0; c < NCOEF; ++c)
-                            tma_load_3d(smem_u32(dst + c * T::CTILE), &maps.coef[c], k0, j0, q - 1, bar,
-                                        pol_stream);
-                        ++cfill;
                     }
                 }
             }
@@ -619,7 +864,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
     } else {
         // ------------------------------------------------------ consumers
         // Each thread owns PPT consecutive k points of one tile row and marches
-        // them through the unit's planes.  Carried in registers from plane to
+        // them through the run's planes.  Carried in registers from plane to
         // plane: the row-(j) window of planes i-1 and i, the j+-1 centres of
         // plane i, D = p(j+1) - p(j-1) on plane i (exact two-sum pairs, all
         // window positions) and its centres on plane i-1.  Per plane only the
@@ -658,12 +903,13 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
         };
         uint32_t cuse = 0, pseq = 0;
         bool ok = true;
-        for (int u = blockIdx.x; ok && u < a.n_units; u += gridDim.x) {
-            int k0, j0, ib, ie;
-            decode_unit(a, u, I, TK, TJ, k0, j0, ib, ie);
+        double racc = 0.0;           // this thread's ss^2 sum, run after run
+        Runs runs(blockIdx.x);
+        int k0, j0, ib, ie;
+        while (ok && runs.next(a, TK, TJ, k0, j0, ib, ie)) {
             const int j = j0 + r, kb = k0 + PPT * cg;
             const bool row_in = (j <= J - 2);
-            float RH = 0.0f, RL = 0.0f;  // this thread's ss^2 sum over the unit (float-float)
+            float RH = 0.0f, RL = 0.0f;  // this thread's ss^2 sum over the run (float-float)
             const uint32_t pbase = pseq;
             for (uint32_t s = pbase; s < pbase + 2; ++s)
                 if (!mbar_wait(smem_u32(&full_p[s % DP]), (s / DP) & 1, abort_flag, a.err, 4u)) {
@@ -816,7 +1062,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
                 }
             }
             if (!ok) break;
-            // release the unit's last two planes
+            // release the run's last two planes
             __syncwarp();
             if (lane == 0) {
                 const uint32_t s1 = pbase + (uint32_t)(ie - ib);
@@ -824,13 +1070,13 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
                 mbar_arrive(smem_u32(&empty_p[(s1 + 1) % DP]));
             }
             pseq = pbase + (uint32_t)(ie - ib + 2);
-            // unit partial residual of this warp in FP64 (no cross-warp
-            // barrier, so an aborting warp can never leave another waiting)
-            double racc = (double)RH + (double)RL;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) racc += __shfl_xor_sync(0xffffffffu, racc, o);
-            if (lane == 0) a.partials[(size_t)u * NCW + warp] = racc;
+            racc += (double)RH + (double)RL;
         }
+        // partial residual of this warp in FP64 (no cross-warp barrier, so an
+        // aborting warp can never leave another waiting)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) racc += __shfl_xor_sync(0xffffffffu, racc, o);
+        if (lane == 0) a.partials[(size_t)blockIdx.x * NCW + warp] = racc;
         if (lane == 0) __threadfence();  // partials visible before the CTA is counted
     }
     __syncthreads();
@@ -844,7 +1090,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
     __syncthreads();
     if (*last_flag) {
         __threadfence();
-        const int np = a.n_units * NCW;
+        const int np = (int)gridDim.x * NCW;
         double s = 0.0;
         for (int u = threadIdx.x; u < np; u += blockDim.x) s += __ldcg(&a.partials[u]);
         // fixed-shape tree: within warps, then warp sums in warp order
@@ -864,7 +1110,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
 // variants: (TK, TJ, NCW, DC, DP, PPT, MINB)
 struct VariantInfo {
     int TK, TJ, ctas_per_sm, ncw;
-    void (*launch)(int grid, const StencilMaps &m, const StencilArgs &a, cudaStream_t s, bool inject);
+    void (*launch)(int grid, const StencilMaps &m, const StencilArgs &a, cudaStream_t s, bool inject, bool chained);
 };
 
 template <int TK, int TJ, int NCW, int DC, int DP, int PPT, int MINB>
@@ -875,18 +1121,23 @@ struct Variant {
         return 128 + (size_t)DC * NCOEF * T::CTILE * 4 + (size_t)DP * T::PSLOT * 4 +
                2 * (DC + DP) * 8 + 32 * 8 + 16;
     }
-    static void launch(int grid, const StencilMaps &m, const StencilArgs &a, cudaStream_t s, bool inject) {
+    static void launch(int grid, const StencilMaps &m, const StencilArgs &a, cudaStream_t s, bool inject,
+                       bool chained) {
         static std::atomic<uint64_t> done{0}, done_inj{0};
-        if (inject) {
-            set_smem_limit_once((const void *)stencil_kernel<TK, TJ, NCW, DC, DP, PPT, MINB, true>, smem_bytes(),
-                                done_inj);
-            stencil_kernel<TK, TJ, NCW, DC, DP, PPT, MINB, true><<<grid, kThreads, smem_bytes(), s>>>(m, a);
-        } else {
-            set_smem_limit_once((const void *)stencil_kernel<TK, TJ, NCW, DC, DP, PPT, MINB, false>, smem_bytes(),
-                                done);
-            stencil_kernel<TK, TJ, NCW, DC, DP, PPT, MINB, false><<<grid, kThreads, smem_bytes(), s>>>(m, a);
-        }
-        OO_CUDA_TRY(cudaGetLastError());
+        auto kernel = inject ? stencil_kernel<TK, TJ, NCW, DC, DP, PPT, MINB, true>
+                             : stencil_kernel<TK, TJ, NCW, DC, DP, PPT, MINB, false>;
+        set_smem_limit_once((const void *)kernel, smem_bytes(), inject ? done_inj : done);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)grid);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = smem_bytes();
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = chained ? 1 : 0;
+        OO_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, m, a));
     }
     static VariantInfo info() { return VariantInfo{TK, TJ, MINB, NCW, &launch}; }
 };
@@ -894,8 +1145,8 @@ struct Variant {
 // 0: 128x8 tile, 8 consumer warps x 4 points, 1 CTA/SM
 // 1: 128x8 tile, 16 consumer warps x 2 points, 1 CTA/SM
 // 2: 128x4 tile, 8 consumer warps x 2 points, 2 CTAs/SM
-// 3: 64x8 tile, 4 consumer warps x 4 points (short rows, K <= 65)
-// 4: 64x8 tile, 8 consumer warps x 2 points, 2 CTAs/SM (short rows)
+// 3: 64x8 tile, 4 consumer warps x 4 points, 1 CTA/SM (short rows, K <= 65)
+// 4: 64x8 tile, 8 consumer warps x 2 points, 2 CTAs/SM (short rows, and rows that 128 pads badly)
 const VariantInfo &variant(int v) {
     static const VariantInfo table[] = {
         Variant<128, 8, 8, 3, 5, 4, 1>::info(),
@@ -943,6 +1194,8 @@ struct StencilPlan {
     int variant = -1;  // tile variant; -1 on creation: the default rule picks
     int TK = 128, TJ = 8;
     StencilMaps maps;
+    CUtensorMap p_flip;      // wrk2 as the array read (sweeps with p and wrk2 exchanged)
+    float *out_flip = nullptr;
     StencilArgs args{};
     int grid = 0;
     void *scratch = nullptr;
@@ -950,11 +1203,9 @@ struct StencilPlan {
 };
 
 namespace {
-// tensor maps, tile shape and the i-segment split of a plan (no scratch yet)
-// max_slots > 0 caps the partial-residual slots (units x consumer warps)
-// the i-segment split may use
+// tensor maps, tile shape and work split of a plan (no scratch yet)
 void fill_stencil_plan(StencilPlan *sp, const JacobiDims &d, const float *const coef[NCOEF], const float *p,
-                       float *wrk2, int num_sms, long long max_slots = 0) {
+                       float *wrk2, int num_sms) {
     sp->d = d;
     // default tile shape by row length (16 consumer warps x 2 points measured
     // ~0.6 % faster than 8 x 4 at 257 x 257 x 513) unless the caller chose
@@ -964,38 +1215,38 @@ void fill_stencil_plan(StencilPlan *sp, const JacobiDims &d, const float *const 
     sp->TJ = variant(sp->variant).TJ;
     for (int c = 0; c < NCOEF; ++c) make_map(&sp->maps.coef[c], coef[c], d, sp->TK, sp->TJ);
     make_map(&sp->maps.p, p, d, sp->TK + 8, sp->TJ + 2);
+    make_map(&sp->p_flip, wrk2, d, sp->TK + 8, sp->TJ + 2);
+    sp->out_flip = const_cast<float *>(p);
     StencilArgs &a = sp->args;
     a.I = d.I;
     a.J = d.J;
     a.K = d.K;
     a.pitch = d.pitch;
     a.n_kt = (d.K - 1 + sp->TK - 1) / sp->TK;
-    a.n_jt = (d.J - 2 + sp->TJ - 1) / sp->TJ;
-    const int cols = a.n_kt * a.n_jt;
-    const int span = d.I - 2;
-    // segments of the i range: balance units over one CTA per SM, with a
-    // charge for the two halo planes and the prologue every unit pays
+    const int cols = a.n_kt * ((d.J - 2 + sp->TJ - 1) / sp->TJ), span = d.I - 2;
     const int G = std::max(1, num_sms * variant(sp->variant).ctas_per_sm);
-    const int ncw = variant(sp->variant).ncw;
-    OO_REQUIRE(max_slots <= 0 || (long long)cols * ncw <= max_slots, OO_EINVAL,
-               "grid too large for the static scratch: ceil((K-1)/tile_k) * ceil((J-2)/tile_j) * consumer warps "
-               "must be <= " + std::to_string(max_slots));
-    double best = 1e300;
-    int best_seg = 1;
-    for (int ns = 1; ns <= span; ++ns) {
-        if (max_slots > 0 && (long long)cols * ns * ncw > max_slots) break;
-        const int smax = (span + ns - 1) / ns;
-        const long long units = (long long)cols * ns;
-        const long long rounds = (units + G - 1) / G;
-        const double cost = (double)rounds * (smax + 0.6);
-        if (cost < best - 1e-9) {
-            best = cost;
-            best_seg = ns;
+    a.whole = cols / G;
+    a.n_col = cols % G;
+    a.seg = a.n_col ? std::min(G / a.n_col, span) : 0;
+    a.tail = a.n_col && a.seg < span ? std::min((long long)G - (long long)a.seg * a.n_col, (long long)a.n_col * span) : 0;
+    a.i_cut = span;
+    if (a.tail > 0) {
+        // the cut that makes the longest CTA shortest; starting a run costs
+        // about kRunStart planes (two more p planes, a pipeline to refill)
+        constexpr double kRunStart = 0.5;
+        double best = 1e300;
+        for (int cut = 1; cut < span; ++cut) {
+            const double above = std::ceil((double)a.n_col * (span - cut) / a.tail);
+            const double t = std::max(std::ceil((double)cut / a.seg) + kRunStart,
+                                      above + kRunStart * (1.0 + std::ceil(above / (span - cut))));
+            if (t <= best) {
+                best = t;
+                a.i_cut = cut;
+            }
         }
+        if (std::ceil((double)span / a.seg) + kRunStart <= best) a.tail = 0, a.i_cut = span;
     }
-    a.n_seg = best_seg;
-    a.n_units = cols * best_seg;
-    sp->grid = std::min(a.n_units, G);
+    sp->grid = a.whole ? G : a.seg * a.n_col + a.tail;
     a.wrk2 = wrk2;
 }
 void attach_scratch(StencilPlan *sp, void *scratch) {
@@ -1003,20 +1254,17 @@ void attach_scratch(StencilPlan *sp, void *scratch) {
     sp->scratch = scratch;
     a.partials = reinterpret_cast<double *>(scratch);
     a.counter = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(scratch) +
-                                             (size_t)a.n_units * kMaxConsumerWarps * 8);
+                                             (size_t)sp->grid * kMaxConsumerWarps * 8);
     a.err = a.counter + 1;
 }
 size_t plan_scratch_bytes(const StencilPlan *sp) {
-    return (size_t)sp->args.n_units * kMaxConsumerWarps * 8 + 256;
+    return (size_t)sp->grid * kMaxConsumerWarps * 8 + 256;
 }
 }  // namespace
 
 size_t stencil_scratch_bytes(const JacobiDims &d, int num_sms) {
-    // upper bound over the tile variants (smallest tile 64 x 4) and every
-    // i-segment split (at most one unit per plane)
-    (void)num_sms;
-    const long long kt = (d.K - 1 + 63) / 64, jt = (d.J - 2 + 3) / 4;
-    return (size_t)(kt * jt * std::max(1, d.I - 2)) * kMaxConsumerWarps * 8 + 256;
+    (void)d;
+    return (size_t)num_sms * kMaxCtasPerSm * kMaxConsumerWarps * 8 + 256;  // of any tile variant
 }
 
 StencilPlan *stencil_plan_create_ext(const JacobiDims &d, const float *const coef[NCOEF], const float *p, float *wrk2,
@@ -1064,7 +1312,15 @@ StencilPlan *stencil_plan_create(const JacobiDims &d, const float *const coef[NC
 
 int stencil_plan_variant(const StencilPlan *sp) { return sp->variant; }
 int stencil_variant_count() { return kNumVariants; }
-int stencil_default_variant(const JacobiDims &d) { return d.K - 1 > 64 ? 1 : 4; }
+// Default tile: 128 wide (variant 1), or 64 wide (4) where that pads the row
+// so much less that its 10 % lower rate per padded point pays: at 150 x 131 x
+// 270 (320 against 384 columns for 269) 69.5 against 77.1 us a sweep, at 257 x
+// 257 x 400 (448 against 512 for 399) 287 against 295, at 257 x 257 x 513
+// (512 both) 334 against 303.
+int stencil_default_variant(const JacobiDims &d) {
+    const int w128 = (d.K - 1 + 127) / 128 * 128, w64 = (d.K - 1 + 63) / 64 * 64;
+    return 1.12 * w64 < w128 ? 4 : 1;
+}
 
 void stencil_plan_destroy(StencilPlan *sp) {
     if (!sp) return;
@@ -1072,10 +1328,19 @@ void stencil_plan_destroy(StencilPlan *sp) {
     delete sp;
 }
 
-void launch_stencil(StencilPlan *sp, float omega, double *res_dev, cudaStream_t s, bool inject_timeout) {
+void launch_stencil(StencilPlan *sp, float omega, double *res_dev, cudaStream_t s, bool inject_timeout, bool flip,
+                    bool chained) {
     sp->args.omega = omega;
     sp->args.res = res_dev;
-    variant(sp->variant).launch(sp->grid, sp->maps, sp->args, s, inject_timeout);
+    if (!flip) {
+        variant(sp->variant).launch(sp->grid, sp->maps, sp->args, s, inject_timeout, chained);
+        return;
+    }
+    StencilMaps maps = sp->maps;
+    StencilArgs args = sp->args;
+    maps.p = sp->p_flip;
+    args.wrk2 = sp->out_flip;
+    variant(sp->variant).launch(sp->grid, maps, args, s, inject_timeout, chained);
 }
 
 const unsigned *stencil_plan_err_ptr(const StencilPlan *sp) { return sp->args.err; }
@@ -1142,13 +1407,25 @@ extern "C" oo_status oo_stencil_noalloc_dev(oo_ctx *ctx, int I, int J, int K, in
         OO_REQUIRE(((uintptr_t)wrk2 & 15u) == 0, OO_EINVAL, "wrk2 must be 16-byte aligned");
         OO_REQUIRE(std::isfinite(omega), OO_EINVAL, "omega must be finite");
         OO_CUDA_TRY(cudaSetDevice(c.device));
-        // the plan lives on the host stack: tile variant and i-segment split
-        // as oo_stencil_dev chooses them (the context's option or tuned
-        // choice, else the default rule), the split capped at the static
-        // array's slots
+        // the plan lives on the host stack: tile variant and work split as
+        // oo_stencil_dev chooses them (the context's option or tuned choice,
+        // else the default rule).  Grids beyond the documented limit are
+        // refused, though a sweep needs few of the static array's slots.
+        {
+            static const int shape[kNumVariants][3] = {  // tile_k, tile_j, consumer warps the limit counts
+                {128, 8, 8}, {128, 8, 16}, {128, 4, 8}, {64, 8, 4}, {64, 8, 8}};
+            int v = c.stencil_variant_for(I, J, K);
+            if (v < 0 || v >= kNumVariants) v = K - 1 > 64 ? 1 : 4;
+            const long long cols = (long long)((K - 1 + shape[v][0] - 1) / shape[v][0]) *
+                                   ((J - 2 + shape[v][1] - 1) / shape[v][1]);
+            OO_REQUIRE(cols * shape[v][2] <= kStaticPartials, OO_EINVAL,
+                       "grid too large for the static scratch: ceil((K-1)/tile_k) * ceil((J-2)/tile_j) * consumer "
+                       "warps must be <= " + std::to_string(kStaticPartials));
+        }
         StencilPlan sp;
         sp.variant = c.stencil_variant_for(I, J, K);
-        fill_stencil_plan(&sp, JacobiDims{I, J, K, pitch}, coef, p, wrk2, c.num_sms, kStaticPartials);
+        fill_stencil_plan(&sp, JacobiDims{I, J, K, pitch}, coef, p, wrk2, c.num_sms);
+        OO_REQUIRE((long long)sp.grid * kMaxConsumerWarps <= kStaticPartials, OO_EINVAL, "more SMs than the static scratch serves");
         char *scratch = static_cast<char *>(static_scratch_ptr(c.device));
         StencilArgs &sa = sp.args;
         sa.partials = reinterpret_cast<double *>(scratch);
@@ -1161,7 +1438,7 @@ extern "C" oo_status oo_stencil_noalloc_dev(oo_ctx *ctx, int I, int J, int K, in
         OO_CUDA_TRY(cudaMemsetAsync(sa.counter, 0, 8, c.stream));
         const bool inject = c.inject_wait == OO_INJECT_STENCIL_LOAD;
         if (inject) c.inject_wait = OO_INJECT_NONE;
-        variant(sp.variant).launch(sp.grid, sp.maps, sa, c.stream, inject);
+        variant(sp.variant).launch(sp.grid, sp.maps, sa, c.stream, inject, false);
         OO_CUDA_TRY(cudaGetLastError());
         c.last_error.clear();
         return OO_OK;

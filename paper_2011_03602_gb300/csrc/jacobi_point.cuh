@@ -89,37 +89,27 @@ __device__ __forceinline__ float stencil_point_core(const float cf[NCOEF], const
     return out;
 }
 
-// Plane window around element c, read through L2 (p is rewritten by other
-// SMs between iterations, so never a stale L1 line); `full` false reads the
-// centre cross only (planes i +- 1).
+// Plane window around element c; `full` false reads the centre cross only
+// (planes i +- 1).  p is rewritten by other SMs between iterations: with L1
+// false it is read through L2; with L1 true through L1, for a caller that
+// has ordered its reads behind those writes with a fence of its own (which
+// drops stale L1 lines) before each iteration.
+template <bool L1 = false>
 __device__ __forceinline__ void load_pwin(const float *p, size_t c, size_t sj, bool full, PWin &P) {
-    P.w[1][1] = __ldcg(p + c);
-    P.w[2][1] = __ldcg(p + c + sj);
-    P.w[0][1] = __ldcg(p + c - sj);
-    P.w[1][2] = __ldcg(p + c + 1);
-    P.w[1][0] = __ldcg(p + c - 1);
+    auto ld = [](const float *x) { return L1 ? *x : __ldcg(x); };
+    P.w[1][1] = ld(p + c);
+    P.w[2][1] = ld(p + c + sj);
+    P.w[0][1] = ld(p + c - sj);
+    P.w[1][2] = ld(p + c + 1);
+    P.w[1][0] = ld(p + c - 1);
     if (full) {
-        P.w[2][2] = __ldcg(p + c + sj + 1);
-        P.w[0][2] = __ldcg(p + c - sj + 1);
-        P.w[2][0] = __ldcg(p + c + sj - 1);
-        P.w[0][0] = __ldcg(p + c - sj - 1);
+        P.w[2][2] = ld(p + c + sj + 1);
+        P.w[0][2] = ld(p + c - sj + 1);
+        P.w[2][0] = ld(p + c + sj - 1);
+        P.w[0][0] = ld(p + c - sj - 1);
     } else {
         P.w[2][2] = P.w[0][2] = P.w[2][0] = P.w[0][0] = 0.0f;
     }
-}
-
-// One interior point c (element offset; si, sj the i and j strides in
-// elements), without tiling: wrk2[c] from p; ss^2 added to (RH, RL).
-__device__ __forceinline__ void stencil_point_ff(const float *const *coef, const float *p, size_t c, size_t si,
-                                                 size_t sj, float omega, float *wrk2, float &RH, float &RL) {
-    float cf[NCOEF];
-#pragma unroll
-    for (int q = 0; q < NCOEF; ++q) cf[q] = coef[q][c];
-    PWin W, C, E;
-    load_pwin(p, c - si, sj, false, W);
-    load_pwin(p, c, sj, true, C);
-    load_pwin(p, c + si, sj, false, E);
-    wrk2[c] = stencil_point_core(cf, W, C, E, omega, RH, RL);
 }
 
 // face value of the Dirichlet boundary: (k / (K - 1))^2 as one correctly

@@ -83,7 +83,7 @@ struct JacobiWork {
     size_t dev_stride = 0;            // floats between arrays
     double *res_dev = nullptr;        // iters_cap doubles
     float *host = nullptr;            // NARR arrays, each n_host() floats (pinned)
-    double *res_host = nullptr;       // iters_cap doubles (pinned)
+    double *res_host = nullptr;       // iters_cap doubles (pinned), then one for an error word
     StencilPlan *splan = nullptr;
     void *fused_ctl = nullptr;        // fused-iteration barrier words + residual partials
     float *dptr(int v) const { return dev + (size_t)v * dev_stride; }
@@ -352,6 +352,8 @@ void launch_pinit(const JacobiDims &d, float *p, float *wrk2, cudaStream_t s);
 void launch_copyback(const JacobiDims &d, float *p, const float *wrk2, cudaStream_t s);
 // N3 + N4 + N5 in one pass (all three on the GPU, no copy between them)
 void launch_copyback_faces(const JacobiDims &d, float *p, const float *wrk2, cudaStream_t s);
+// N4 + N5 on the array the stencil sweep launched just before writes, beside it
+void launch_bc_faces(const JacobiDims &d, float *p, cudaStream_t s);
 void launch_bc_ij(const JacobiDims &d, float *p, cudaStream_t s);
 void launch_bc_k(const JacobiDims &d, float *p, cudaStream_t s);
 
@@ -374,16 +376,24 @@ void stencil_plan_destroy(StencilPlan *sp);
 // inject_timeout: fault injection for tests -- the producer never issues the
 // first p-tile fill, so the consumers' bounded wait runs out (~1 s) and the
 // sweep reports an error bit instead of a result
-void launch_stencil(StencilPlan *sp, float omega, double *res_dev, cudaStream_t s, bool inject_timeout = false);
+// flip: the sweep reads the plan's wrk2 and writes its p (whose memory must
+// be the caller's to write)
+// chained: the launch before it on s is a launch_bc_faces whose sweep, like
+// this one, finds its coefficients unchanged; the sweep may then set itself
+// up and load coefficients while its predecessor ends
+void launch_stencil(StencilPlan *sp, float omega, double *res_dev, cudaStream_t s, bool inject_timeout = false,
+                    bool flip = false, bool chained = false);
 // All iterations of the all-GPU iteration nests in one cooperative launch
-// (small grids): ctl is jacobi_fused_ctl_bytes() of device scratch.
+// (small grids): ctl is jacobi_fused_ctl_bytes() of device scratch, whose
+// first word is nonzero afterwards if a bounded wait ran out.  Both
+// arrays hold the faces' values on entry (the setup nest); returns the one
+// of p and wrk2 that holds the final pressure.
 size_t jacobi_fused_ctl_bytes();
-// option: -1 the size rule (at most 2^20 points), 0 never, 1 always
+// option: -1 the size rule, 0 never, 1 always
 bool jacobi_fused_eligible(const JacobiDims &d, int option);
-void launch_jacobi_fused(const JacobiDims &d, const float *const coef[NCOEF], float *p, float *wrk2, float omega,
-                         int iters, double *res_dev, void *ctl, cudaStream_t s,
-                         bool inject_timeout = false);
-unsigned jacobi_fused_check(void *ctl, cudaStream_t s);
+float *launch_jacobi_fused(const JacobiDims &d, const float *const coef[NCOEF], float *p, float *wrk2, float omega,
+                           int iters, double *res_dev, void *ctl, cudaStream_t s,
+                           bool inject_timeout = false);
 // Device address of the plan's error word (0 = fine).
 const unsigned *stencil_plan_err_ptr(const StencilPlan *sp);
 // Reads and clears the device-side error word of the plan (0 = fine).

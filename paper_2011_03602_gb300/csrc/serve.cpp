@@ -193,12 +193,16 @@ void start(Server &S, SReq &q) {
         // nothing crosses until the final p and res
         launch_coef(d, coefw, s);
         launch_pinit(d, a[VAR_P], a[VAR_WRK2], s);
+        // p and wrk2 exchange roles from one iteration to the next (pattern.cpp)
+        const float *p_dev = a[VAR_P];
         for (int it = 0; it < r.iters; ++it) {
-            launch_stencil(q.splan, r.omega, res + it, s);
-            launch_copyback_faces(d, a[VAR_P], a[VAR_WRK2], s);  // N3 + N4 + N5
+            float *out = a[it & 1 ? VAR_P : VAR_WRK2];
+            launch_stencil(q.splan, r.omega, res + it, s, false, it & 1, it > 0);
+            launch_bc_faces(d, out, s);  // N4 + N5
+            p_dev = out;
         }
         const size_t wb = (size_t)d.K * 4;
-        OO_CUDA_TRY(cudaMemcpy2DAsync(hst + q.h_out, wb, a[VAR_P], (size_t)d.pitch * 4, wb, (size_t)d.I * d.J,
+        OO_CUDA_TRY(cudaMemcpy2DAsync(hst + q.h_out, wb, p_dev, (size_t)d.pitch * 4, wb, (size_t)d.I * d.J,
                                       cudaMemcpyDeviceToHost, s));
         if (r.iters > 0)
             OO_CUDA_TRY(cudaMemcpyAsync(hst + q.h_res, res, (size_t)r.iters * 8, cudaMemcpyDeviceToHost, s));
