@@ -332,6 +332,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
 // 0 that their accumulator buffer is free.  The D_pq of a K-block are exact
 // whatever the instruction shape, and the epilogue adds the units in the
 // same order, so the result is the single-CTA kernel's bit for bit.
+// The producer and the MMA issuer run as whole warps (tc.cuh): with one lane
+// running each loop, the issuer's own instructions took 611 clocks a K step,
+// and 1050 while the epilogue ran, for 512 clocks of MMA; n = 4096 took 2.92
+// ms in this kernel, 2.29 ms so (3.13 -> 2.56 ms with the splits).
 constexpr int kStagesPair = 6;
 constexpr uint32_t kStageBytesPair = 2 * kTile;  // A_p and this CTA's B tile
 constexpr uint32_t kIdescPair2 = idesc_bf16(2 * kBM, 2 * kBN);
@@ -361,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tempty + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const bool leader = rank == 0;
     const int cid = (int)(blockIdx.x >> 1), ncl = (int)(gridDim.x >> 1);
@@ -388,77 +392,91 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
     __syncthreads();
     cluster_sync_all();  // both CTAs' barriers and TMEM exist before either uses the other's
     fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     int loaded = 0, units_mma = 0;
-    if (warp == 0 && lane == 0) {
-        // ---------------------------------------------------- TMA producer (both CTAs)
-        int it = 0;
+    if (warp == 0) {
+        // ---------------------------------------------------- TMA producer (both CTAs, whole warp)
+        const uint32_t el = elect_one();
+        const uint32_t sm0 = su32(sm), empty0 = su32(empty);
+        const uint32_t full_here = su32(full), full0 = map_to_rank(full_here, 0);
+        int s = 0;
+        uint32_t phase = 1;  // the ring's first use needs no wait
         bool ok = true;
         for (int t = cid; ok && t < tiles; t += ncl) {
             int m0, n0;
             eq_tile_pair(a, t, m0, n0);
-            for (int u = 0; ok && u < units; ++u) {
-                const int kbi = u / a.nunits, pr = u % a.nunits;  // K-block outer: its slices stay in L2
-                const bool pair = a.uq2[pr] != kNone;
-                const int rowA = a.up[pr] * a.m + m0 + (int)rank * kBM;
-                const int rowB = pair ? (rank ? a.uq2[pr] : a.uq1[pr]) * a.n + n0
-                                      : a.uq1[pr] * a.n + n0 + (int)rank * (kBN / 2);
-                const uint32_t tx = pair ? 2 * 2 * kTile : 2 * (kTile + kTile / 2);
-                const int ks1 = min(a.ksteps, (kbi + 1) * a.kb_steps);
-                for (int ks = kbi * a.kb_steps; ks < ks1; ++ks, ++it) {
-                    const int s = it % kStagesPair;
-                    const uint32_t use = it / kStagesPair;
-                    if (use > 0 && !bar_wait_cluster(su32(&empty[s]), (use - 1) & 1, abort_flag, a.err, 1u)) {
-                        ok = false;
-                        break;
+            for (int kbi = 0; ok && kbi < a.nkb; ++kbi)  // K-block outer: its slices stay in L2
+                for (int pr = 0; ok && pr < a.nunits; ++pr) {
+                    const bool pair = a.uq2[pr] != kNone;
+                    const int rowA = a.up[pr] * a.m + m0 + (int)rank * kBM;
+                    const int rowB = pair ? (rank ? a.uq2[pr] : a.uq1[pr]) * a.n + n0
+                                          : a.uq1[pr] * a.n + n0 + (int)rank * (kBN / 2);
+                    const uint32_t tx = pair ? 2 * 2 * kTile : 2 * (kTile + kTile / 2);
+                    const CUtensorMap *mb = pair ? &maps.b : &maps.bh;
+                    const int ks1 = min(a.ksteps, (kbi + 1) * a.kb_steps);
+                    for (int ks = kbi * a.kb_steps; ks < ks1; ++ks) {
+                        if (loaded >= kStagesPair && !warp_wait<true>(empty0 + s * 8, phase, abort_flag, a.err, 1u)) {
+                            ok = false;
+                            break;
+                        }
+                        const uint32_t st = sm0 + s * kStageBytesPair, fb = full0 + s * 8;
+                        if (leader) bar_expect_tx_if(el, full_here + s * 8, tx);
+                        tma_2d_pair_if(el, st, &maps.a, ks * kBK, rowA, fb);
+                        tma_2d_pair_if(el, st + kTile, mb, ks * kBK, rowB, fb);
+                        ++loaded;
+                        if (++s == kStagesPair) {
+                            s = 0;
+                            phase ^= 1;
+                        }
                     }
-                    unsigned char *st = sm + (size_t)s * kStageBytesPair;
-                    if (leader) bar_expect_tx(su32(&full[s]), tx);
-                    const uint32_t fb = map_to_rank(su32(&full[s]), 0);
-                    tma_2d_pair(su32(st), &maps.a, ks * kBK, rowA, fb);
-                    tma_2d_pair(su32(st + kTile), pair ? &maps.b : &maps.bh, ks * kBK, rowB, fb);
-                    ++loaded;
                 }
-            }
         }
-    } else if (warp == 1 && lane == 0 && leader) {
-        // ---------------------------------------------------- MMA issuer (rank 0)
-        int it = 0, gu = 0;
+    } else if (warp == 1 && leader) {
+        // ---------------------------------------------------- MMA issuer (rank 0, whole warp)
+        const uint32_t el = elect_one();
+        const uint64_t da0 = sdesc_sw128(su32(sm)), db0 = sdesc_sw128(su32(sm) + kTile);
+        const uint32_t full0 = su32(full), empty0 = su32(empty), tfull0 = su32(tfull), tempty0 = su32(tempty);
+        int s = 0, gu = 0;
+        uint32_t phase = 0;
         bool ok = true;
         for (int t = cid; ok && t < tiles; t += ncl) {
-            for (int u = 0; ok && u < units; ++u, ++gu) {
-                const int b = gu & 1;
-                const uint32_t buse = gu >> 1;
-                if (buse > 0 && !bar_wait_cluster(su32(&tempty[b]), (buse - 1) & 1, abort_flag, a.err, 2u)) {
-                    ok = false;
-                    break;
-                }
-                fence_after();
-                const uint32_t d = tmem + (uint32_t)(b * 2 * kBN);
-                const int kbi = u / a.nunits, pr = u % a.nunits;
-                const uint32_t idesc = a.uq2[pr] != kNone ? kIdescPair2 : kIdescOne2;
-                const int ks0 = kbi * a.kb_steps, ks1 = min(a.ksteps, (kbi + 1) * a.kb_steps);
-                for (int ks = ks0; ks < ks1; ++ks, ++it) {
-                    const int s = it % kStagesPair;
-                    if (!bar_wait_cluster(su32(&full[s]), (it / kStagesPair) & 1, abort_flag, a.err, 2u)) {
+            for (int kbi = 0; ok && kbi < a.nkb; ++kbi)
+                for (int pr = 0; ok && pr < a.nunits; ++pr, ++gu) {
+                    const int b = gu & 1;
+                    if (gu > 1 &&
+                        !warp_wait<true>(tempty0 + b * 8, ((gu >> 1) - 1) & 1, abort_flag, a.err, 2u)) {
                         ok = false;
                         break;
                     }
                     fence_after();
-                    const uint32_t sa = su32(sm + (size_t)s * kStageBytesPair), sb = sa + kTile;
+                    const uint32_t d = tmem + (uint32_t)(b * 2 * kBN);
+                    const uint32_t idesc = a.uq2[pr] != kNone ? kIdescPair2 : kIdescOne2;
+                    const int steps = min(a.ksteps, (kbi + 1) * a.kb_steps) - kbi * a.kb_steps;
+                    uint32_t acc = 0;
+                    for (int ks = 0; ks < steps; ++ks) {
+                        if (!warp_wait<true>(full0 + s * 8, phase, abort_flag, a.err, 2u)) {
+                            ok = false;
+                            break;
+                        }
+                        fence_after();
+                        const uint64_t da = da0 + (uint64_t)(s * (int)(kStageBytesPair >> 4)),
+                                       db = db0 + (uint64_t)(s * (int)(kStageBytesPair >> 4));
 #pragma unroll
-                    for (int kk = 0; kk < kBK / 16; ++kk) {
-                        const uint32_t off = kk * 32;
-                        const uint32_t acc = (ks == ks0 && kk == 0) ? 0u : 1u;
-                        mma_bf16_pair(d, sdesc_sw128(sa + off), sdesc_sw128(sb + off), idesc, acc);
+                        for (int kk = 0; kk < kBK / 16; ++kk) {  // 32 bytes of each row per MMA
+                            mma_bf16_pair_if(el, d, da + kk * 2, db + kk * 2, idesc, acc);
+                            acc = 1;
+                        }
+                        mma_commit_pair_if(el, empty0 + s * 8, 3);  // stage s free in both CTAs
+                        if (++s == kStagesPair) {
+                            s = 0;
+                            phase ^= 1;
+                        }
                     }
-                    mma_commit_pair(su32(&empty[s]), 3);  // stage s free in both CTAs
+                    if (!ok) break;
+                    mma_commit_pair_if(el, tfull0 + b * 8, 3);  // this unit's accumulators complete in both CTAs
+                    ++units_mma;
                 }
-                if (!ok) break;
-                mma_commit_pair(su32(&tfull[b]), 3);  // this unit's accumulators complete in both CTAs
-                ++units_mma;
-            }
         }
     } else if (warp >= 2) {
         // ---------------------------------------------------- epilogue (both CTAs)

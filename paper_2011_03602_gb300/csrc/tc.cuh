@@ -210,6 +210,96 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t cols)
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
 
+// ---- roles run by a whole warp.  A loop that one lane runs alone computes
+// every operand of a TMA copy or an MMA in per-thread registers and moves it
+// to the uniform registers these instructions read from: about 100 clocks an
+// instruction, twice that while the epilogue warps of the same scheduler are
+// busy (FP64-equivalent pair kernel at n = 4096: 611 and 1050 clocks per K
+// step of four MMAs, 512 clocks of tensor work).  Run by the whole warp, with
+// warp-uniform control flow and one elected lane issuing, the operands are
+// computed in uniform registers to begin with.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t el;
+    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(el));
+    return el;
+}
+// the warp's index as a value the compiler knows to be warp-uniform
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+// bounded wait of a whole warp; CLUSTER: ordered after the other CTA's arrivals
+template <bool CLUSTER>
+__device__ __forceinline__ bool warp_wait(uint32_t b, uint32_t par, volatile int *abort_flag, unsigned *err,
+                                          unsigned code) {
+    auto done = [&] { return __all_sync(0xffffffffu, CLUSTER ? bar_try_cluster(b, par) : bar_try(b, par)); };
+    if (done()) return true;
+    const long long t0 = clock64();
+    while (true) {
+        if (done()) return true;
+        const bool out = clock64() - t0 > kWaitLimit;
+        if (__any_sync(0xffffffffu, out)) {
+            *abort_flag = 1;
+            if ((threadIdx.x & 31) == 0) atomicOr(err, code);
+            return false;
+        }
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+    }
+}
+__device__ __forceinline__ void bar_expect_tx_if(uint32_t el, uint32_t b, uint32_t bytes) {
+    asm volatile(
+        "{\n\t.reg .b64 st;\n\t.reg .pred Q;\n\tsetp.ne.b32 Q, %2, 0;\n\t"
+        "@Q mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(b),
+        "r"(bytes), "r"(el)
+        : "memory");
+}
+__device__ __forceinline__ void tma_2d_if(uint32_t el, uint32_t dst, const CUtensorMap *map, int c0, int c1,
+                                          uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred Q;\n\tsetp.ne.b32 Q, %5, 0;\n\t"
+        "@Q cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+        "[%4];\n\t}" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar), "r"(el)
+        : "memory");
+}
+__device__ __forceinline__ void tma_2d_pair_if(uint32_t el, uint32_t dst, const CUtensorMap *map, int c0, int c1,
+                                               uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred Q;\n\tsetp.ne.b32 Q, %5, 0;\n\t"
+        "@Q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+        "%3}], [%4];\n\t}" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar), "r"(el)
+        : "memory");
+}
+__device__ __forceinline__ void mma_bf16_if(uint32_t el, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                            uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, Q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 Q, %5, 0;\n\t"
+        "@Q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(el)
+        : "memory");
+}
+__device__ __forceinline__ void mma_bf16_pair_if(uint32_t el, uint32_t d_tmem, uint64_t a, uint64_t b,
+                                                 uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, Q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 Q, %5, 0;\n\t"
+        "@Q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(el)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit_if(uint32_t el, uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred Q;\n\tsetp.ne.b32 Q, %1, 0;\n\t"
+        "@Q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
+        "r"(el)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit_pair_if(uint32_t el, uint32_t bar, uint16_t mask) {
+    asm volatile(
+        "{\n\t.reg .pred Q;\n\tsetp.ne.b32 Q, %2, 0;\n\t"
+        "@Q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], "
+        "%1;\n\t}" ::"r"(bar),
+        "h"(mask), "r"(el)
+        : "memory");
+}
+
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
