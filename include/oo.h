@@ -454,7 +454,8 @@ enum { OO_EQ_PAIRS = 0, OO_EQ_LEVELS = 1 };
 oo_status oo_gemm_scheme(int k, int *scheme, int *per_accumulator);
 
 /* Tile widths of the FP64-equivalent product in batches and in the single
- * products of a level scheme: output tiles are 128 rows by 32, 64 or 128
+ * products of a level scheme (whose tiles are at most 64 wide in batches and
+ * single calls): output tiles are 128 rows by 32, 64 or 128
  * columns.  The width of a problem's full tiles is looked up by its n and k
  * in a table of OO_TILE_NBUCKETS x OO_TILE_KBUCKETS entries, entry
  * [nb * OO_TILE_KBUCKETS + kb] with nb for n <= 32, 64, 128, 256, 512 or

@@ -26,7 +26,10 @@
 // eight epilogue warps (two per lane quarter) add each finished unit, scaled
 // by its power of two, into a float-float sum in registers and write FP64 C
 // after the tile's last unit; warps whose rows or columns lie wholly outside
-// the problem skip the reads.  Every mbarrier wait is bounded.
+// the problem skip the reads.  Every mbarrier wait is bounded.  Tiles of
+// level schemes run in a kernel of their own in batches and single calls
+// ("level schemes" below, at most 64 columns wide); the device-resident loop
+// runs them in these roles, with the same additions in the same order.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -60,7 +63,7 @@ constexpr unsigned char kNone = 0xff;
 constexpr int kClasses = 6;
 // scheme tables: 0 pairs with 8-bit digits (padded k <= 256), 1 pairs with
 // 7-bit digits, 2 levels with 7-bit digits, 3 levels with 6-bit digits
-constexpr int kTables = 4;
+constexpr int kTables = 4, kTabLevel7 = 2, kTabLevel6 = 3;
 
 struct SchemeTab {
     int nunits, nterms;
@@ -269,6 +272,36 @@ __device__ __forceinline__ bool mma_tile(const GArgs &a, const Pipe &pp, const G
     return true;
 }
 
+// (Sh, Sl) += d f, f a power of two: the levels of a level scheme, nine at
+// most, so the low parts are summed without renormalising (7 operations for
+// 12; each level's own rounding stays below 2^-47 of the sum).
+__device__ __forceinline__ void level_add(float &Sh, float &Sl, float d, float f) {
+    const float s = __fmaf_rn(d, f, Sh);
+    const float bb = __fsub_rn(s, Sh);
+    const float e = __fadd_rn(__fsub_rn(Sh, __fsub_rn(s, bb)), __fmaf_rn(d, f, -bb));
+    Sh = s;
+    Sl = __fadd_rn(Sl, e);
+}
+
+// (h + l) 2^S as a double, rounded once, for a level sum: the high part's
+// bits and the low part as an integer in units of the double's last place
+// (ff::to_double's case analysis took twice the instructions).  Zero, results
+// near the ends of the range and the flag scales of non-finite rows and
+// columns take the general conversion.
+__device__ __forceinline__ double level_value(float h, float l, int S) {
+    float s, e;
+    ff::two_sum(h, l, s, e);
+    const unsigned b = __float_as_uint(s), m = b & 0x7fffffu;
+    const int es = (int)((b >> 23) & 0xffu), ed = es - 127 + 1023 + S;
+    if ((unsigned)(es - 64) > 126u || (unsigned)(ed - 2) > 2043u) return nan_or_scaled(ff::to_double(h, l), S);
+    int t = __float2int_rn(__fmul_rn(e, __uint_as_float((unsigned)(306 - es) << 23)));  // |t| <= 2^28
+    if (b >> 31) t = -t;
+    if (m == 0 && t < 0) t += t;  // the last place is half as large below a power of two
+    const unsigned long long v = ((unsigned long long)(unsigned)ed << 52) + ((unsigned long long)m << 29) +
+                                 (unsigned long long)(long long)t;
+    return __longlong_as_double((long long)(v | ((unsigned long long)(b >> 31) << 63)));
+}
+
 // One epilogue warp (of eight: lane quarter q = warp & 3, column half h):
 // add every finished unit of one tile, scaled by its power of two, into a
 // float-float running sum (Sh, Sl) of this row's columns, then write FP64
@@ -285,6 +318,7 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
     const int ncols = min(cpw, P.n - td.z - cw0);
     const bool active = row0 < P.m && ncols > 0;  // warp-uniform
     const int units = P.nkb * S.nunits;
+    const bool levels = P.scheme >= kTabLevel7;
     for (int uu = 0; uu < units; ++uu, ++gu) {
         const int b = gu & 1;
         if (!bar_wait(su32(&pp.tfull[b]), (gu >> 1) & 1, pp.abort_flag, a.err, 4u)) return false;
@@ -305,6 +339,8 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
                         if (uu == 0) {
                             Sh[c + j] = w;
                             Sl[c + j] = 0.0f;
+                        } else if (levels) {
+                            level_add(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), fL);
                         } else {
                             ff::add(Sh[c + j], Sl[c + j], w, 0.0f, Sh[c + j], Sl[c + j]);
                         }
@@ -315,7 +351,10 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             const float w = __fmul_rn(__uint_as_float(v[j]), fR);
-                            ff::add(Sh[c + j], Sl[c + j], w, 0.0f, Sh[c + j], Sl[c + j]);
+                            if (levels)
+                                level_add(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), fR);
+                            else
+                                ff::add(Sh[c + j], Sl[c + j], w, 0.0f, Sh[c + j], Sl[c + j]);
                         }
                     }
                 }
@@ -339,7 +378,9 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
         for (int j = 0; j < 64; ++j) {
             if (j < ncols) {
                 const int sb = __shfl_sync(0xffffffffu, j < 32 ? e0 : e1, j & 31);
-                if (row_ok) crow[j] = nan_or_scaled(ff::to_double(Sh[j], Sl[j]), sa + sb);
+                if (row_ok)
+                    crow[j] = levels ? level_value(Sh[j], Sl[j], sa + sb)
+                                     : nan_or_scaled(ff::to_double(Sh[j], Sl[j]), sa + sb);
             }
         }
     }
@@ -411,11 +452,343 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_eq_group_kernel(const __grid
     eq_tiles_body(maps, a, src);
 }
 
-__global__ void __launch_bounds__(kThreads, 1) gemm_eq_single_kernel(const __grid_constant__ GMaps maps,
-                                                                    const __grid_constant__ GArgs a,
-                                                                    const __grid_constant__ GProb P) {
+// ---------------------------------------------------------- level schemes
+// Tiles of the level schemes (k <= 512, one K-block: every D_pq of a level
+// s = p + q in one accumulator) in a kernel of their own, which stages each
+// digit slice of a tile once per K step.  The unit-based roles above stage A_p
+// and B_q for every product, 14 to 20 times 48 KB per K step; they ran the
+// 4096 products of the batched workload (m, n, k log-uniform in [16, 512]) in
+// 4.0 ms, waiting on operands (tensor pipe 17 % busy); this kernel takes
+// 1.40 ms (0.65 ms of MMA at full rate, 0.63 ms of operand intake).  One 256 x
+// 256 x 256 product: 119 -> 16 us.
+//
+// With the B slices' tiles of w <= 64 rows stacked in shared memory and the
+// levels' accumulators side by side in tensor memory (S w <= 512 columns),
+// all products of one A slice are one MMA: A_p x [B_1 .. B_{L-p}] adds to
+// the levels p + 1 .. L.  p runs downwards, so stage j of a K step needs one
+// more slice of each operand: (A_S, B_1), (A_{S-1}, B_2), ..., (A_1, B_S); A
+// slices go through a five-slot ring, B slices stay for their K step (two
+// buffers).  A K step of 64 moves S (rows of A + w) x 128 bytes for S (S + 1)
+// w / 512 x 128 clocks of MMA: 192 KB for 4608 clocks at S = 8, w = 64 and full
+// rows, 42 bytes a clock (an SM takes in up to 65).  A's rows beyond
+// the problem are not loaded (their accumulator rows are not read).
+//
+// The tensor memory holds one tile.  Level s is first touched at stage
+// j = L + 1 - s, so the next tile's first stages, whose MMAs are short, need
+// only the highest levels: the epilogue drains those first and frees level by
+// level, and the next tile's MMAs run behind it.
+constexpr int kLvSlots = 5, kLvWidth = 64, kLvMax = 8;
+constexpr int kLvThreads = 352;  // A producer, MMA issuer, 8 epilogue warps, B producer
+constexpr uint32_t kLvB = kLvMax * kLvWidth * kBK * 2;  // B slices of a K step: 64 KB
+constexpr uint32_t kLvOut = 32 * 8 * 8;                 // an epilogue warp's 32 rows x 8 columns
+constexpr size_t kLvSmem = 1024 + (size_t)kLvSlots * kTileA + 2 * (size_t)kLvB + kEpiWarps * kLvOut + 256;
+static_assert(kLvSmem <= 232448, "level kernel exceeds the shared memory of a CTA");
+
+struct LvMaps {
+    CUtensorMap a[3][kClasses], b[2][kClasses];  // boxes of 32, 64, 128 rows
+};
+struct LvPipe {
+    unsigned char *sa, *sb, *so;
+    uint64_t *afull, *aempty;  // per A slot; afull counts both producers' tiles of the stage
+    uint64_t *bempty;          // per B buffer
+    uint64_t *lfull, *lempty;  // tile accumulated; per level: drained
+    uint64_t *drain;           // after an abort
+    volatile int *abort_flag;
+    uint32_t tmem;
+};
+
+__device__ __forceinline__ int lv_slices(const GProb &P) { return P.scheme == kTabLevel7 ? 7 : 8; }
+__device__ __forceinline__ int lv_beta(const GProb &P) { return P.scheme == kTabLevel7 ? 7 : 6; }
+
+// TMA producers (a whole warp each) of one tile: the A slices, or the B
+// slices.  A copy costs its issuer about 64 clocks and 1 clock per 75 bytes
+// (measured: boxes of 4 / 16 / 32 KB 34 / 58 / 65 bytes a clock from one warp,
+// 16 KB boxes from two warps 65), so boxes are as tall as the rows allow and
+// the operands have a warp each.
+template <bool A>
+__device__ __forceinline__ bool lv_produce(const LvMaps &maps, unsigned *err, const LvPipe &pp, const GProb &P,
+                                           const int4 &td, uint32_t el, int &st, int &kc) {
+    const int S = lv_slices(P), rows = A ? min(kBM, P.m - td.y) : td.w;
+    const int box = rows <= 32 ? 0 : (rows <= 64 ? 1 : 2);
+    const CUtensorMap *map = A ? &maps.a[box][P.cls] : &maps.b[box & 1][P.cls];
+    const uint32_t bytes = kBox << box;
+    const uint32_t full0 = su32(pp.afull), empty0 = su32(pp.aempty);
+    int slot = st % kLvSlots;
+    uint32_t use = st / kLvSlots;
+    for (int ks = 0; ks < P.ksteps; ++ks, ++kc) {
+        const int buf = kc & 1;
+        if (!A && kc >= 2 &&
+            !warp_wait<false>(su32(pp.bempty) + buf * 8, ((kc >> 1) - 1) & 1, pp.abort_flag, err, 1u))
+            return false;
+        // A_S, A_{S-1}, ... into the ring; B_1, B_2, ... stacked in the K step's buffer
+        int row = A ? P.ra + (S - 1) * P.m + td.y : P.rb + td.z;
+        uint32_t dst = A ? 0u : su32(pp.sb) + (uint32_t)buf * kLvB;
+        for (int j = 0; j < S; ++j) {
+            if (use > 0 && !warp_wait<false>(empty0 + slot * 8, (use - 1) & 1, pp.abort_flag, err, 1u)) return false;
+            const uint32_t fb = full0 + slot * 8;
+            bar_expect_tx_if(el, fb, bytes);
+            tma_2d_if(el, A ? su32(pp.sa) + slot * kTileA : dst, map, ks * kBK, row, fb);
+            row += A ? -P.m : P.n;
+            if (!A) dst += bytes;
+            ++st;
+            if (++slot == kLvSlots) {
+                slot = 0;
+                ++use;
+            }
+        }
+    }
+    return true;
+}
+
+// MMA issuer (a whole warp) of one tile; last_w: the width of the CTA's tile
+// before this one (0: none)
+__device__ __forceinline__ bool lv_mma(unsigned *err, const LvPipe &pp, const GProb &P, const int4 &td, uint32_t el,
+                                       int tile, int &st, int &kc, int &last_w) {
+    const int S = lv_slices(P), w = td.w, most = 256 / w;  // B slices of one MMA
+    if (last_w != w && tile > 0)  // the level blocks lie elsewhere: wait for every one of the last tile's
+        for (int l = 0; l < kLvMax; ++l)
+            if (!warp_wait<false>(su32(pp.lempty) + l * 8, (tile - 1) & 1, pp.abort_flag, err, 2u)) return false;
+    last_w = w;
+    const uint64_t da0 = sdesc_sw128(su32(pp.sa)), db0 = sdesc_sw128(su32(pp.sb));
+    const uint32_t full0 = su32(pp.afull), empty0 = su32(pp.aempty), lempty0 = su32(pp.lempty);
+    const uint32_t id1 = idesc_n(w);
+    int slot = st % kLvSlots;
+    uint32_t use = st / kLvSlots;
+    for (int ks = 0; ks < P.ksteps; ++ks, ++kc) {
+        const uint64_t db = db0 + (uint64_t)((kc & 1) * (int)(kLvB >> 4));
+        for (int j = 1; j <= S; ++j) {
+            const int l0 = S - j;  // level block of q = 1 (block x: level x + 2)
+            if (!warp_wait<false>(full0 + slot * 8, use & 1, pp.abort_flag, err, 2u)) return false;
+            if (ks == 0 && tile > 0 && !warp_wait<false>(lempty0 + l0 * 8, (tile - 1) & 1, pp.abort_flag, err, 2u))
+                return false;
+            fence_after();
+            const uint64_t da = da0 + (uint64_t)(slot * (int)(kTileA >> 4));
+            // B_1 .. B_j in one or two MMAs (c1, c2 slices); 32 bytes of each row per MMA
+            const int c1 = min(j, most), c2 = j - c1;
+            const uint32_t d1 = pp.tmem + (uint32_t)(l0 * w), d2 = d1 + (uint32_t)(c1 * w);
+            const uint64_t db2 = db + (uint64_t)(c1 * w * 8);
+            const uint32_t i1 = idesc_n(c1 * w), i2 = idesc_n(c2 * w);
+            if (ks == 0) {
+                // the tile's first MMA at this stage starts the sum of the block
+                // it touches first, and of no other
+                mma_bf16_if(el, d1, da, db, id1, 0u);
+                if (c1 > 1) mma_bf16_if(el, d1 + (uint32_t)w, da, db + (uint64_t)(w * 8), idesc_n((c1 - 1) * w), 1u);
+            } else {
+                mma_bf16_if(el, d1, da, db, i1, 1u);
+            }
+            if (c2 > 0) mma_bf16_if(el, d2, da, db2, i2, 1u);
+#pragma unroll
+            for (int kk = 1; kk < kBK / 16; ++kk) {
+                mma_bf16_if(el, d1, da + kk * 2, db + kk * 2, i1, 1u);
+                if (c2 > 0) mma_bf16_if(el, d2, da + kk * 2, db2 + kk * 2, i2, 1u);
+            }
+            mma_commit_if(el, empty0 + slot * 8);
+            ++st;
+            if (++slot == kLvSlots) {
+                slot = 0;
+                ++use;
+            }
+        }
+        mma_commit_if(el, su32(pp.bempty) + (kc & 1) * 8);
+    }
+    mma_commit_if(el, su32(pp.lfull));
+    return true;
+}
+
+// One epilogue warp of one tile: every level into a float-float sum per
+// column of the lane's row, then C through a small shared-memory transpose.
+// The loops over levels and rows stay rolled and 8-byte stores go out as
+// 64-byte row segments: unrolled over 32 columns, with a row per lane, the
+// conversion and the stores took 27,000 clocks a tile, most of them
+// instruction fetches and store replays.
+__device__ __forceinline__ bool lv_epilogue(unsigned *err, const LvPipe &pp, const GProb &P, const int4 &td,
+                                            int tile) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q = warp & 3, h = (warp - 2) >> 2;
+    const int S = lv_slices(P), L = S + 1, beta = lv_beta(P);
+    const int cpw = td.w >> 1, cw0 = h * cpw;  // 32 or 16 columns per warp
+    const int row0 = td.y + q * 32, c0 = td.z + cw0;
+    const int ncols = min(cpw, P.n - c0), nrows = min(32, P.m - row0);
+    const bool active = nrows > 0 && ncols > 0;
+    const uint32_t acc = pp.tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)cw0;
+    // scales: lane l holds row l's and column l's
+    const int eb = active && lane < ncols ? P.eb[c0 + lane] : 0;
+    const int ea = active && lane < nrows ? P.ea[row0 + lane] : 0;
+    if (!bar_wait(su32(pp.lfull), tile & 1, pp.abort_flag, err, 4u)) return false;
+    fence_after();
+    if (lane == 0)  // blocks this tile does not have
+        for (int l = S; l < kLvMax; ++l) bar_arrive(su32(&pp.lempty[l]));
+    float Sh[32], Sl[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) Sh[j] = Sl[j] = 0.0f;
+    // smallest contributions first, two levels at a time (s, s + 1): the order
+    // of the unit-based roles
+    for (int x = 0; x < S; ++x) {
+        const int s = (L & 1) == 0 ? (x == 0 ? L : L - 2 * ((x + 1) >> 1) + ((x + 1) & 1)) : L - 1 - 2 * (x >> 1) + (x & 1);
+        const int blk = s - 2;
+        uint32_t v[32];
+        if (active) {
+            OO_TMEM_LD16(acc + (uint32_t)(blk * td.w), v);
+            if (cpw > 16) {
+                uint32_t *v2 = v + 16;
+                OO_TMEM_LD16(acc + (uint32_t)(blk * td.w) + 16, v2);
+            }
+            tmem_wait_ld();
+        }
+        fence_before();
+        __syncwarp();
+        if (lane == 0) bar_arrive(su32(&pp.lempty[blk]));
+        if (active) {
+            const float f = __uint_as_float((uint32_t)(127 - beta * s) << 23);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) level_add(Sh[j], Sl[j], __uint_as_float(v[j]), f);
+            if (cpw > 16) {
+#pragma unroll
+                for (int j = 16; j < 32; ++j) level_add(Sh[j], Sl[j], __uint_as_float(v[j]), f);
+            }
+        }
+    }
+    if (active) {
+        float2 *out = reinterpret_cast<float2 *>(pp.so + (warp - 2) * kLvOut);
+        const int col = lane & 7;
+#pragma unroll
+        for (int c = 0; c < 32; c += 8) {
+            if (c >= ncols) continue;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) out[lane * 8 + (j ^ (lane & 7))] = make_float2(Sh[c + j], Sl[c + j]);
+            __syncwarp();
+            const int sb = __shfl_sync(0xffffffffu, eb, c + col);
+            const bool col_ok = c + col < ncols;
+            double *dst = P.C + (long long)(row0 + (lane >> 3)) * P.ldc + c0 + c + col;
+#pragma unroll 1
+            for (int r = lane >> 3; r < 32; r += 4, dst += 4 * P.ldc) {
+                const float2 v = out[r * 8 + (col ^ (r & 7))];
+                const int sa = __shfl_sync(0xffffffffu, ea, r);
+                if (col_ok && r < nrows) *dst = level_value(v.x, v.y, sa + sb);
+            }
+            __syncwarp();
+        }
+    }
+    return true;
+}
+
+// The CTA's tiles in turn, each with its problem's descriptor in registers (a
+// reference into global memory is read again, from L2, after every barrier),
+// the next one's read while the current one is in work.  UNIFORM: the fields
+// the issuing warps use, as values the compiler knows to be warp-uniform.
+template <bool UNIFORM, class Src, class F>
+__device__ __forceinline__ void lv_for_tiles(const Src &src, F &&work) {
+    const int tiles = src.count();
+    int t = blockIdx.x;
+    if (t >= tiles) return;
+    int4 td = src.tile(t);
+    GProb P = src.prob(td.x);
+    for (;;) {
+        t += gridDim.x;
+        const bool more = t < tiles;
+        int4 tn = td;
+        GProb Pn = P;
+        if (more) {
+            tn = src.tile(t);
+            Pn = src.prob(tn.x);
+        }
+        if (UNIFORM) {
+            auto u = [](int &x) { x = __shfl_sync(0xffffffffu, x, 0); };
+            u(td.y), u(td.z), u(td.w), u(P.m), u(P.n), u(P.ksteps), u(P.ra), u(P.rb), u(P.cls), u(P.scheme);
+        }
+        if (!work(P, td) || !more) return;
+        td = tn;
+        P = Pn;
+    }
+}
+
+template <class Src>
+__device__ __forceinline__ void eq_levels_body(const LvMaps &maps, unsigned *err, const Src &src) {
+    extern __shared__ __align__(1024) unsigned char gsm_raw[];
+    LvPipe pp;
+    pp.sa = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(gsm_raw) + 1023) &
+                                              ~static_cast<uintptr_t>(1023));
+    pp.sb = pp.sa + kLvSlots * kTileA;
+    pp.so = pp.sb + 2 * kLvB;
+    pp.afull = reinterpret_cast<uint64_t *>(pp.so + kEpiWarps * kLvOut);
+    pp.aempty = pp.afull + kLvSlots;
+    pp.bempty = pp.aempty + kLvSlots;
+    pp.lfull = pp.bempty + 2;
+    pp.lempty = pp.lfull + 1;
+    pp.drain = pp.lempty + kLvMax;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(pp.drain + 1);
+    pp.abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kLvSlots; ++s) {
+            bar_init(su32(&pp.afull[s]), 2);
+            bar_init(su32(&pp.aempty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) bar_init(su32(&pp.bempty[b]), 1);
+        bar_init(su32(pp.lfull), 1);
+        for (int l = 0; l < kLvMax; ++l) bar_init(su32(&pp.lempty[l]), kEpiWarps);
+        bar_init(su32(pp.drain), 1);
+        *pp.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        tmem_alloc(su32(tmem_slot), 512);
+        fence_before();
+    }
+    __syncthreads();
+    fence_after();
+    pp.tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    int st = 0, kc = 0, tile = 0, last_w = 0;
+    if (warp == 0) {
+        const uint32_t el = elect_one();
+        lv_for_tiles<true>(src, [&](const GProb &P, const int4 &td) {
+            return lv_produce<true>(maps, err, pp, P, td, el, st, kc);
+        });
+    } else if (warp == 2 + kEpiWarps) {
+        const uint32_t el = elect_one();
+        lv_for_tiles<true>(src, [&](const GProb &P, const int4 &td) {
+            return lv_produce<false>(maps, err, pp, P, td, el, st, kc);
+        });
+    } else if (warp == 1) {
+        const uint32_t el = elect_one();
+        lv_for_tiles<true>(src, [&](const GProb &P, const int4 &td) {
+            return lv_mma(err, pp, P, td, el, tile++, st, kc, last_w);
+        });
+    } else {
+        lv_for_tiles<false>(src, [&](const GProb &P, const int4 &td) { return lv_epilogue(err, pp, P, td, tile++); });
+    }
+    // after an abort: wait (bounded) for issued MMAs and copies before tensor
+    // memory is released and the CTA exits
+    if (*pp.abort_flag) {
+        if (warp == 1 && lane == 0) {
+            mma_commit(su32(pp.drain));
+            bar_drain(su32(pp.drain), 0);
+        }
+        if ((warp == 0 || warp == 2 + kEpiWarps) && lane == 0)
+            for (int x = (st > kLvSlots ? st - kLvSlots : 0); x < st; ++x)
+                bar_drain(su32(&pp.afull[x % kLvSlots]), (x / kLvSlots) & 1);
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        fence_after();
+        tmem_dealloc(pp.tmem, 512);
+    }
+}
+
+__global__ void __launch_bounds__(kLvThreads, 1) eq_levels_group_kernel(const __grid_constant__ LvMaps maps,
+                                                                     unsigned *err, const GProb *probs,
+                                                                     const int4 *tiles, int ntiles) {
+    const GroupTiles src{probs, tiles, ntiles};
+    eq_levels_body(maps, err, src);
+}
+
+__global__ void __launch_bounds__(kLvThreads, 1) eq_levels_single_kernel(const __grid_constant__ LvMaps maps,
+                                                                      unsigned *err,
+                                                                      const __grid_constant__ GProb P) {
     const SingleTiles src{&P};
-    eq_tiles_body(maps, a, src);
+    eq_levels_body(maps, err, src);
 }
 
 // ------------------------------------------------ the device-resident loop
@@ -707,6 +1080,7 @@ int bucket_k(int k) {
 
 // relative cost of a tile, for ordering the work list (largest first)
 double tile_cost(const eq::Shape &e, int ksteps, int width) {
+    if (e.scheme != eq::kSchemePairs) return (double)width * (ksteps * (double)e.nprod * 2.0 + 110.0);
     return (double)width * ((double)ksteps * e.nprod + 8.0 * e.nkb * (e.scheme == eq::kSchemePairs
                                                                         ? (e.nprod + e.slices) / 2.0
                                                                         : (e.levels + 1) / 2.0));
@@ -742,16 +1116,27 @@ int eq_tile_width(const int *widths, int n, int k) {
     return (w == 32 || w == 64 || w == 128) ? w : eq_default_width(bucket_n(n), bucket_k(k));
 }
 
+// tile width of a level scheme's product from a table's width: two tiles'
+// worth of a 128-wide one
+int level_width(int w) { return std::min(w, kLvWidth); }
+
+void level_maps(LvMaps *m, int c, const void *a, long long rows_a, const void *b, long long rows_b, long long pitch) {
+    for (int x = 0; x < 3; ++x) map_slices(&m->a[x][c], a, rows_a, pitch, kBRows << x);
+    for (int x = 0; x < 2; ++x) map_slices(&m->b[x][c], b, rows_b, pitch, kBRows << x);
+}
+
 struct EqGroup {
     void *arena = nullptr;
-    GMaps maps{};
+    GMaps maps{};    // pair scheme
+    LvMaps lmaps{};  // level schemes
     GArgs args{};
     GProb *d_probs = nullptr;
     int4 *d_tiles = nullptr;
     eq::GSplit *d_split = nullptr;
     int4 *d_jobs = nullptr;
     unsigned *d_err = nullptr;
-    int ntiles = 0, njobs = 0, nrow_jobs = 0, grid = 1;
+    int ntiles = 0, nlevel = 0, njobs = 0, nrow_jobs = 0;  // nlevel: the list's first tiles, of level schemes
+    int num_sms = 1;
     double flops = 0;
 };
 
@@ -799,15 +1184,18 @@ EqGroup *eq_group_create(const std::vector<GemmDesc> &v, int num_sms, const int 
     std::vector<int4> tiles, jobs, col_jobs;  // row jobs first, then column jobs
     std::vector<double> cost;
     double flops = 0;
+    int nlevel = 0;
     for (size_t i = 0; i < np; ++i) {
         const GemmDesc &d = v[i];
         flops += 2.0 * d.m * d.n * d.k;
-        const int W = eq_tile_width(widths, d.n, d.k);
+        const bool level = sh[i].scheme != eq::kSchemePairs;
+        const int Wt = eq_tile_width(widths, d.n, d.k), W = level ? level_width(Wt) : Wt;
         for (int m0 = 0; m0 < d.m; m0 += kBM)
             for (int n0 = 0; n0 < d.n; n0 += W) {
                 const int w = d.n - n0 >= W ? W : narrowest_width(d.n - n0);
                 tiles.push_back(make_int4((int)i, m0, n0, w));
                 cost.push_back(tile_cost(sh[i], kp[i] / kBK, w));
+                nlevel += level;
             }
         for (int r0 = 0; r0 < d.m; r0 += 8) jobs.push_back(make_int4(0, (int)i, r0, 0));
         for (int c0 = 0; c0 < d.n; c0 += 64) col_jobs.push_back(make_int4(1, (int)i, c0, 0));
@@ -817,7 +1205,11 @@ EqGroup *eq_group_create(const std::vector<GemmDesc> &v, int num_sms, const int 
     OO_REQUIRE(tiles.size() < (1u << 31) && jobs.size() < (1u << 31), OO_EINVAL, "too many tiles");
     std::vector<size_t> order(tiles.size());
     for (size_t t = 0; t < order.size(); ++t) order[t] = t;
-    std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) { return cost[x] > cost[y]; });
+    auto level_tile = [&](size_t t) { return sh[tiles[t].x].scheme != eq::kSchemePairs; };
+    std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) {
+        const bool lx = level_tile(x), ly = level_tile(y);
+        return lx != ly ? lx : cost[x] > cost[y];
+    });
     std::vector<int4> sorted(tiles.size());
     for (size_t t = 0; t < order.size(); ++t) sorted[t] = tiles[order[t]];
     const size_t off_probs = at;
@@ -842,6 +1234,7 @@ EqGroup *eq_group_create(const std::vector<GemmDesc> &v, int num_sms, const int 
             if (rows_a[c] == 0) continue;
             map_slices(&g->maps.a[c], base + off_a[c], rows_a[c], KP[c], kBM);
             map_slices(&g->maps.b[c], base + off_b[c], rows_b[c], KP[c], kBRows);
+            level_maps(&g->lmaps, c, base + off_a[c], rows_a[c], base + off_b[c], rows_b[c], KP[c]);
         }
         std::vector<GProb> probs(np);
         std::vector<eq::GSplit> splits(np);
@@ -883,7 +1276,8 @@ EqGroup *eq_group_create(const std::vector<GemmDesc> &v, int num_sms, const int 
         g->ntiles = (int)sorted.size();
         g->njobs = (int)jobs.size();
         g->nrow_jobs = nrow_jobs;
-        g->grid = std::max(1, std::min(g->ntiles, num_sms));
+        g->nlevel = nlevel;
+        g->num_sms = std::max(1, num_sms);
         g->flops = flops;
     } catch (...) {
         if (g->arena) cudaFree(g->arena);
@@ -895,11 +1289,20 @@ EqGroup *eq_group_create(const std::vector<GemmDesc> &v, int num_sms, const int 
 
 void eq_group_launch(EqGroup *g, cudaStream_t s) {
     launch_eq_group_split(g->d_split, g->d_jobs, g->nrow_jobs, g->njobs - g->nrow_jobs, s);
-    static std::atomic<uint64_t> attr{0};
-    set_smem_limit_once((const void *)gemm_eq_group_kernel, smem_bytes(), attr);
-    gemm_eq_group_kernel<<<g->grid, kThreads, smem_bytes(), s>>>(g->maps, g->args, g->d_probs, g->d_tiles,
-                                                                 g->ntiles);
-    OO_CUDA_TRY(cudaGetLastError());
+    static std::atomic<uint64_t> attr{0}, lattr{0};
+    if (g->nlevel > 0) {
+        set_smem_limit_once((const void *)eq_levels_group_kernel, kLvSmem, lattr);
+        eq_levels_group_kernel<<<std::min(g->nlevel, g->num_sms), kLvThreads, kLvSmem, s>>>(
+            g->lmaps, g->d_err, g->d_probs, g->d_tiles, g->nlevel);
+        OO_CUDA_TRY(cudaGetLastError());
+    }
+    const int pairs = g->ntiles - g->nlevel;
+    if (pairs > 0) {
+        set_smem_limit_once((const void *)gemm_eq_group_kernel, smem_bytes(), attr);
+        gemm_eq_group_kernel<<<std::min(pairs, g->num_sms), kThreads, smem_bytes(), s>>>(
+            g->maps, g->args, g->d_probs, g->d_tiles + g->nlevel, pairs);
+        OO_CUDA_TRY(cudaGetLastError());
+    }
 }
 
 unsigned eq_group_check(EqGroup *g, cudaStream_t s) {
@@ -926,9 +1329,9 @@ void launch_gemm_eq_tiles(int m, int n, int k, const void *As, const void *Bs, c
                           double *C, long long ldc, int width, unsigned *err, int num_sms, cudaStream_t s) {
     const eq::Shape e = eq::shape(eq_scheme_for(k), k);
     const int kp = (k + kBK - 1) / kBK * kBK;
-    GMaps maps{};
-    map_slices(&maps.a[0], As, (long long)e.slices * m, kp, kBM);
-    map_slices(&maps.b[0], Bs, (long long)e.slices * n, kp, kBRows);
+    OO_REQUIRE(e.scheme != eq::kSchemePairs && e.nkb == 1 && e.slices <= kLvMax, OO_EINVAL, "not a level scheme");
+    LvMaps maps{};
+    level_maps(&maps, 0, As, (long long)e.slices * m, Bs, (long long)e.slices * n, kp);
     GProb P{};
     P.C = C;
     P.ea = ea;
@@ -943,16 +1346,17 @@ void launch_gemm_eq_tiles(int m, int n, int k, const void *As, const void *Bs, c
     P.rb = 0;
     P.cls = 0;
     P.scheme = table_of(e.scheme, k);
-    P.bn = (width == 32 || width == 64 || width == 128) ? width : 128;
     P.m_tiles = (m + kBM - 1) / kBM;
+    // narrow tiles where wide ones would leave half the SMs without one
+    P.bn = level_width(width == 32 || width == 64 || width == 128 ? width : 128);
+    if ((long long)P.m_tiles * ((n + P.bn - 1) / P.bn) * 2 <= num_sms) P.bn = 32;
     P.n_tiles = (n + P.bn - 1) / P.bn;
     const long long tiles = (long long)P.m_tiles * P.n_tiles;
     OO_REQUIRE(tiles < (1ll << 31), OO_EINVAL, "too many tiles");
-    const GArgs a = make_args(err);
     static std::atomic<uint64_t> attr{0};
-    set_smem_limit_once((const void *)gemm_eq_single_kernel, smem_bytes(), attr);
+    set_smem_limit_once((const void *)eq_levels_single_kernel, kLvSmem, attr);
     const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, num_sms));
-    gemm_eq_single_kernel<<<grid, kThreads, smem_bytes(), s>>>(maps, a, P);
+    eq_levels_single_kernel<<<grid, kLvThreads, kLvSmem, s>>>(maps, err, P);
     OO_CUDA_TRY(cudaGetLastError());
 }
 
