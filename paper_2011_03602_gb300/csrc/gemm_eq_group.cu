@@ -1135,7 +1135,8 @@ struct EqGroup {
     eq::GSplit *d_split = nullptr;
     int4 *d_jobs = nullptr;
     unsigned *d_err = nullptr;
-    int ntiles = 0, nlevel = 0, njobs = 0, nrow_jobs = 0;  // nlevel: the list's first tiles, of level schemes
+    int ntiles = 0, nlevel = 0;  // nlevel: the list's first tiles, of level schemes
+    int split_count[6] = {0, 0, 0, 0, 0, 0};
     int num_sms = 1;
     double flops = 0;
 };
@@ -1181,7 +1182,7 @@ EqGroup *eq_group_create(const std::vector<GemmDesc> &v, int num_sms, const int 
         at += up((size_t)v[i].n * 4, 16);
     }
     at = up(at, 256);
-    std::vector<int4> tiles, jobs, col_jobs;  // row jobs first, then column jobs
+    std::vector<int4> tiles, jobs, split_jobs[6];
     std::vector<double> cost;
     double flops = 0;
     int nlevel = 0;
@@ -1197,11 +1198,9 @@ EqGroup *eq_group_create(const std::vector<GemmDesc> &v, int num_sms, const int 
                 cost.push_back(tile_cost(sh[i], kp[i] / kBK, w));
                 nlevel += level;
             }
-        for (int r0 = 0; r0 < d.m; r0 += 8) jobs.push_back(make_int4(0, (int)i, r0, 0));
-        for (int c0 = 0; c0 < d.n; c0 += 64) col_jobs.push_back(make_int4(1, (int)i, c0, 0));
+        eq_group_split_jobs(sh[i].scheme, (int)i, d.m, d.n, split_jobs);
     }
-    const int nrow_jobs = (int)jobs.size();
-    jobs.insert(jobs.end(), col_jobs.begin(), col_jobs.end());
+    for (const auto &list : split_jobs) jobs.insert(jobs.end(), list.begin(), list.end());
     OO_REQUIRE(tiles.size() < (1u << 31) && jobs.size() < (1u << 31), OO_EINVAL, "too many tiles");
     std::vector<size_t> order(tiles.size());
     for (size_t t = 0; t < order.size(); ++t) order[t] = t;
@@ -1274,8 +1273,7 @@ EqGroup *eq_group_create(const std::vector<GemmDesc> &v, int num_sms, const int 
         g->d_err = reinterpret_cast<unsigned *>(base + off_err);
         g->args = make_args(g->d_err);
         g->ntiles = (int)sorted.size();
-        g->njobs = (int)jobs.size();
-        g->nrow_jobs = nrow_jobs;
+        for (int x = 0; x < 6; ++x) g->split_count[x] = (int)split_jobs[x].size();
         g->nlevel = nlevel;
         g->num_sms = std::max(1, num_sms);
         g->flops = flops;
@@ -1288,7 +1286,7 @@ EqGroup *eq_group_create(const std::vector<GemmDesc> &v, int num_sms, const int 
 }
 
 void eq_group_launch(EqGroup *g, cudaStream_t s) {
-    launch_eq_group_split(g->d_split, g->d_jobs, g->nrow_jobs, g->njobs - g->nrow_jobs, s);
+    launch_eq_group_split(g->d_split, g->d_jobs, g->split_count, s);
     static std::atomic<uint64_t> attr{0}, lattr{0};
     if (g->nlevel > 0) {
         set_smem_limit_once((const void *)eq_levels_group_kernel, kLvSmem, lattr);

@@ -734,14 +734,180 @@ EqLayout eq_layout(int m, int n, int k) {
 
 }  // namespace
 
-// The grouped products' digit split (their tensor-core kernel is in
-// gemm_eq_group.cu, which reads only through L2 for the device-resident
-// loop's sake; the split's second pass over a row wants L1): jobs (0,
-// problem, first row), eight rows of A each, in one kernel that uses no
-// shared memory -- so more of its blocks fit on an SM and L1 keeps the rows
-// for their second pass -- then jobs (1, problem, first column), 64 columns
-// of B each, through shared-memory tiles (eq_digits.cuh).
+// ------------------------------------------- level schemes' digit split
+// The split of products with k <= 512, in batches and single calls (eight
+// BF16 digits of 16 bytes leave a thread at once; digit width and count are
+// constants, so a digit is a shift, a mask, a subtraction and half a
+// permute).  Bound by HBM in batches (8 bytes read and 2 S written an entry)
+// and by latency for one product.  4096 products, m, n, k log-uniform in [16,
+// 512]: rows 625 us and columns 1030 us with a warp per row or 64 columns per
+// block, 4-byte stores and every entry of B read twice; 520 and 795 us so.  One
+// 256 x 256 x 256 product: 34 us in four launches and two clears, 11 us in one.
 namespace {
+
+template <int BETA, int S>
+struct LevelSplit {
+    // digits of eight consecutive entries relative to 2^(mx - 1022) -> dst, one
+    // 16-byte store per slice
+    static __device__ __forceinline__ void eight(const double (&v)[8], int mx, __nv_bfloat16 *dst, size_t plane) {
+        unsigned long long X[8];
+        unsigned sign[4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            unsigned n = 0;
+            X[i] = mx != 0 ? fixed_frac(v[i], mx, n) : 0ull;
+            if (mx == 0) n = 0;
+            if (i & 1)
+                sign[i >> 1] |= n << 31;
+            else
+                sign[i >> 1] = n << 15;
+        }
+#pragma unroll
+        for (int p = 0; p < S; ++p) {
+            unsigned w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                // d < 2^8 is exact as 2^23 + d - 2^23, its BF16 bits the float's top half
+                auto digit = [&](unsigned long long x) {
+                    const unsigned d = (unsigned)(x >> (64 - BETA * (p + 1))) & ((1u << BETA) - 1u);
+                    return __float_as_uint(__fsub_rn(__uint_as_float(0x4b000000u | d), 8388608.0f));
+                };
+                w[i] = __byte_perm(digit(X[2 * i]), digit(X[2 * i + 1]), 0x7632) | sign[i];
+            }
+            *reinterpret_cast<uint4 *>(dst + p * plane) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+
+    // rows [r0, r0 + 32) of A: eight lanes a row, eight entries a lane
+    static __device__ __forceinline__ void rows(const eq::GSplit &G, int r0) {
+        const int lane = threadIdx.x & 31, sub = lane & 7;
+        const int row = r0 + (threadIdx.x >> 5) * 4 + (lane >> 3);
+        const bool in = row < G.m;
+        const double *src = G.A + (long long)(in ? row : 0) * G.lda;
+        const int k = in ? G.k : 0;
+        const bool vec = (((uintptr_t)G.A | (uintptr_t)(G.lda * 8)) & 15u) == 0;
+        auto load = [&](int l, double (&v)[8]) {
+            if (vec && l + 8 <= k) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const double2 x = reinterpret_cast<const double2 *>(src + l)[i];
+                    v[2 * i] = x.x;
+                    v[2 * i + 1] = x.y;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = l + i < k ? src[l + i] : 0.0;
+            }
+        };
+        int mx = 0;
+        double v[8];
+        for (int l = 8 * sub; l < G.kp; l += 64) {
+            load(l, v);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) mx = max(mx, eff_exp(v[i]));
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (!in) return;
+        if (sub == 0) G.ea[row] = mx == 0 ? 0 : mx - 1022;
+        __nv_bfloat16 *dst = G.As + (size_t)row * G.pitch;
+        for (int l = 8 * sub; l < G.kp; l += 64) {
+            if (G.kp > 64) load(l, v);  // from L1; one chunk is still in registers
+            eight(v, mx, dst + l, (size_t)G.m * G.pitch);
+        }
+    }
+
+    // columns [c0, c0 + C) of B through shared memory, read once: t holds C
+    // columns of kp + 1 doubles (an odd pitch, so a row's stores fall in
+    // different banks), red 256 ints.  Every thread of the block calls it.
+    template <int C>
+    static __device__ __forceinline__ void cols(const eq::GSplit &G, int c0, double *t, int *red) {
+        constexpr int R = 256 / C;  // rows read at a time
+        const int tx = threadIdx.x % C, ty = threadIdx.x / C, col = c0 + tx, pitch = G.kp + 1;
+        int mx = 0;
+#pragma unroll 8
+        for (int l = ty; l < G.kp; l += R) {
+            const double x = l < G.k && col < G.n ? G.B[(long long)l * G.ldb + col] : 0.0;
+            mx = max(mx, eff_exp(x));
+            t[tx * pitch + l] = x;
+        }
+        red[threadIdx.x] = mx;
+        __syncthreads();
+        if (ty == 0) {
+#pragma unroll 8
+            for (int y = 1; y < R; ++y) mx = max(mx, red[y * C + tx]);
+            red[tx] = mx;
+            if (col < G.n) G.eb[col] = mx == 0 ? 0 : mx - 1022;
+        }
+        __syncthreads();
+        const int sub = threadIdx.x & 7, chunks = G.kp / 64;
+        for (int u = threadIdx.x >> 3; u < C * chunks; u += 32) {
+            const int c = u % C, l = (u / C) * 64 + 8 * sub;
+            if (c0 + c >= G.n) continue;
+            double v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = t[c * pitch + l + i];
+            eight(v, red[c], G.Bs + (size_t)(c0 + c) * G.pitch + l, (size_t)G.n * G.pitch);
+        }
+    }
+};
+
+// columns per job and its shared memory: small enough for a full SM of blocks
+template <int BETA>
+struct LevelCols;
+template <>
+struct LevelCols<7> {  // k <= 128
+    static constexpr int C = 16, kMax = 128;
+};
+template <>
+struct LevelCols<6> {  // k <= 512
+    static constexpr int C = 8, kMax = 512;
+};
+template <int BETA>
+constexpr size_t level_cols_smem(int kp) {
+    return (size_t)LevelCols<BETA>::C * (kp + 1) * 8;
+}
+
+// jobs (first row), then jobs (first column) of one kind per launch
+template <int BETA, int S>
+__global__ void __launch_bounds__(256) eq_level_rows_kernel(const eq::GSplit *gs, const int4 *jobs) {
+    const int4 jb = jobs[blockIdx.x];
+    const eq::GSplit G = gs[jb.y];
+    LevelSplit<BETA, S>::rows(G, jb.z);
+}
+template <int BETA, int S>
+__global__ void __launch_bounds__(256) eq_level_cols_kernel(const eq::GSplit *gs, const int4 *jobs) {
+    extern __shared__ __align__(16) double lv_t[];
+    __shared__ int red[256];
+    const int4 jb = jobs[blockIdx.x];
+    const eq::GSplit G = gs[jb.y];
+    LevelSplit<BETA, S>::template cols<LevelCols<BETA>::C>(G, jb.z, lv_t, red);
+}
+// one product: the first row_blocks blocks take rows, the others columns
+template <int BETA, int S>
+__global__ void __launch_bounds__(256) eq_level_split_kernel(const __grid_constant__ eq::GSplit G, int row_blocks,
+                                                            unsigned *err) {
+    extern __shared__ __align__(16) double lv_t[];
+    __shared__ int red[256];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *err = 0;  // of the product kernel that follows
+    if ((int)blockIdx.x < row_blocks)
+        LevelSplit<BETA, S>::rows(G, blockIdx.x * 32);
+    else
+        LevelSplit<BETA, S>::template cols<LevelCols<BETA>::C>(G, (blockIdx.x - row_blocks) * LevelCols<BETA>::C,
+                                                               lv_t, red);
+}
+
+template <int BETA, int S>
+void launch_level_split(const eq::GSplit &G, unsigned *err, cudaStream_t s) {
+    constexpr int C = LevelCols<BETA>::C;
+    const int row_blocks = (G.m + 31) / 32, col_blocks = (G.n + C - 1) / C;
+    eq_level_split_kernel<BETA, S><<<row_blocks + col_blocks, 256, level_cols_smem<BETA>(G.kp), s>>>(G, row_blocks,
+                                                                                                   err);
+    OO_CUDA_TRY(cudaGetLastError());
+}
+
+// The grouped split of pair-scheme products (k > 512): eight rows of A a
+// block, then 64 columns of B a block (eq_digits.cuh).
 __global__ void __launch_bounds__(256) eq_group_split_rows_kernel(const eq::GSplit *gs, const int4 *jobs) {
     const int4 jb = jobs[blockIdx.x];
     eq::split_rows_job(gs[jb.y], jb.z);
@@ -754,13 +920,30 @@ __global__ void __launch_bounds__(256) eq_group_split_cols_kernel(const eq::GSpl
 }
 }  // namespace
 
-void launch_eq_group_split(const eq::GSplit *gs, const int4 *jobs, int nrow_jobs, int ncol_jobs, cudaStream_t s) {
-    if (nrow_jobs > 0) {
-        eq_group_split_rows_kernel<<<nrow_jobs, 256, 0, s>>>(gs, jobs);
-        OO_CUDA_TRY(cudaGetLastError());
-    }
-    if (ncol_jobs > 0) {
-        eq_group_split_cols_kernel<<<ncol_jobs, 256, 0, s>>>(gs, jobs + nrow_jobs);
+void eq_group_split_jobs(int scheme, int problem, int m, int n, std::vector<int4> (&jobs)[6]) {
+    const bool pairs = scheme == eq::kSchemePairs;
+    const int base = pairs ? 0 : (scheme == eq::kSchemeLevel7 ? 2 : 4);
+    const int rows = pairs ? 8 : 32;
+    const int cols = pairs ? 64 : (scheme == eq::kSchemeLevel7 ? LevelCols<7>::C : LevelCols<6>::C);
+    for (int r = 0; r < m; r += rows) jobs[base].push_back(make_int4(0, problem, r, 0));
+    for (int c = 0; c < n; c += cols) jobs[base + 1].push_back(make_int4(1, problem, c, 0));
+}
+
+void launch_eq_group_split(const eq::GSplit *gs, const int4 *jobs, const int (&count)[6], cudaStream_t s) {
+    for (int x = 0; x < 6; jobs += count[x++]) {
+        if (count[x] == 0) continue;
+        switch (x) {
+            case 0: eq_group_split_rows_kernel<<<count[x], 256, 0, s>>>(gs, jobs); break;
+            case 1: eq_group_split_cols_kernel<<<count[x], 256, 0, s>>>(gs, jobs); break;
+            case 2: eq_level_rows_kernel<7, 7><<<count[x], 256, 0, s>>>(gs, jobs); break;
+            case 3:
+                eq_level_cols_kernel<7, 7><<<count[x], 256, level_cols_smem<7>(LevelCols<7>::kMax), s>>>(gs, jobs);
+                break;
+            case 4: eq_level_rows_kernel<6, 8><<<count[x], 256, 0, s>>>(gs, jobs); break;
+            case 5:
+                eq_level_cols_kernel<6, 8><<<count[x], 256, level_cols_smem<6>(LevelCols<6>::kMax), s>>>(gs, jobs);
+                break;
+        }
         OO_CUDA_TRY(cudaGetLastError());
     }
 }
@@ -791,6 +974,19 @@ void launch_gemm_fp64eq(int m, int n, int k, const double *A, long long lda, con
     int *mxo = reinterpret_cast<int *>(p + L.mxo);
     auto *As = reinterpret_cast<__nv_bfloat16 *>(p + L.as);
     auto *Bs = reinterpret_cast<__nv_bfloat16 *>(p + L.bs);
+    int dev = 0, sms = 148;
+    OO_CUDA_TRY(cudaGetDevice(&dev));
+    OO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (e.scheme != eq::kSchemePairs) {
+        // level schemes: split and tiled kernel as in batches
+        const eq::GSplit G{A, B, lda, ldb, kp, m, n, k, kp, e.beta, e.slices, As, Bs, ea, eb};
+        if (e.scheme == eq::kSchemeLevel7)
+            launch_level_split<7, 7>(G, err, s);
+        else
+            launch_level_split<6, 8>(G, err, s);
+        launch_gemm_eq_tiles(m, n, k, As, Bs, ea, eb, C, ldc, width, err, sms, s);
+        return;
+    }
     OO_CUDA_TRY(cudaMemsetAsync(err, 0, 4, s));
     OO_CUDA_TRY(cudaMemsetAsync(mxo, 0, (size_t)n * 4, s));
     {
@@ -812,14 +1008,6 @@ void launch_gemm_fp64eq(int m, int n, int k, const double *A, long long lda, con
         OO_REQUIRE(grid.y <= 65535, OO_EINVAL, "k too large");
         eq_split_cols_t_kernel<<<grid, 256, 0, s>>>(B, ldb, k, n, kp, e.beta, e.slices, mxo, Bs);
         OO_CUDA_TRY(cudaGetLastError());
-    }
-    int dev = 0, sms = 148;
-    OO_CUDA_TRY(cudaGetDevice(&dev));
-    OO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (e.scheme != eq::kSchemePairs) {
-        // level schemes: the tiled kernel (gemm_eq_group.cu), as in batches
-        launch_gemm_eq_tiles(m, n, k, As, Bs, ea, eb, C, ldc, width, err, sms, s);
-        return;
     }
     EqMaps maps;
     map_bf16(&maps.a, As, (long long)e.slices * m, kp, kBM);

@@ -182,9 +182,11 @@ void eq_group_launch(EqGroup *g, cudaStream_t s);
 namespace eq {
 struct GSplit;
 }
-// the grouped products' digit split (gemm_fp64eq.cu): njobs jobs of eight A
-// rows or 64 B columns
-void launch_eq_group_split(const eq::GSplit *gs, const int4 *jobs, int nrow_jobs, int ncol_jobs, cudaStream_t s);
+// the grouped products' digit split (gemm_fp64eq.cu): the jobs of one problem
+// (rows and columns of the pair scheme, of 7-bit levels, of 6-bit levels: six
+// lists), and a launch per list that has any; jobs stored list after list
+void eq_group_split_jobs(int scheme, int problem, int m, int n, std::vector<int4> (&jobs)[6]);
+void launch_eq_group_split(const eq::GSplit *gs, const int4 *jobs, const int (&count)[6], cudaStream_t s);
 unsigned eq_group_check(EqGroup *g, cudaStream_t s);
 double eq_group_flops(const EqGroup *g);
 int eq_group_tiles(const EqGroup *g);
