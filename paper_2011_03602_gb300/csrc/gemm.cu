@@ -226,7 +226,7 @@ __device__ __forceinline__ void gemm_body(const Src &src, unsigned *err) {
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStages + 4);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int tiles = src.count();
 
     if (threadIdx.x == 0) {
@@ -251,13 +251,16 @@ __device__ __forceinline__ void gemm_body(const Src &src, unsigned *err) {
     }
     __syncthreads();
     fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     int loaded = 0;          // producer: stages issued
     int tiles_mma = 0;       // MMA issuer: tiles whose accumulation was issued
-    if (warp == 0 && lane == 0) {
-        // ---------------------------------------------------- TMA producer
-        int it = 0;
+    if (warp == 0) {
+        // ---------------------------------------------------- TMA producer (whole warp)
+        const uint32_t el = elect_one();
+        const uint32_t sm0 = su32(gsm), full0 = su32(full), empty0 = su32(empty);
+        int s = 0;
+        uint32_t phase = 1;  // the ring's first use needs no wait
         bool ok = true;
         // the next tile's descriptor is fetched one tile ahead so that its
         // (dependent) global loads stay off the critical path
@@ -265,64 +268,74 @@ __device__ __forceinline__ void gemm_body(const Src &src, unsigned *err) {
         for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
             const TileJob jb = nx;
             if (t + (int)gridDim.x < tiles) nx = src.job(t + gridDim.x);
-            for (int ks = 0; ks < jb.ksteps; ++ks, ++it) {
-                const int s = it % kStages;
-                const uint32_t use = it / kStages;
-                if (use > 0 && !bar_wait(su32(&empty[s]), (use - 1) & 1, abort_flag, err, 1u)) {
+            const int ksteps = uniform(jb.ksteps), ra = uniform(jb.ra + jb.m0), rb = uniform(jb.rb + jb.n0);
+            for (int ks = 0; ks < ksteps; ++ks) {
+                if (loaded >= kStages && !warp_wait<false>(empty0 + s * 8, phase, abort_flag, err, 1u)) {
                     ok = false;
                     break;
                 }
-                unsigned char *st = gsm + (size_t)s * kStageBytes;
-                const uint32_t fb = su32(&full[s]);
-                bar_expect_tx(fb, kStageBytes);
+                const uint32_t st = sm0 + s * kStageBytes, fb = full0 + s * 8;
+                bar_expect_tx_if(el, fb, kStageBytes);
                 const int k0 = ks * (TF32 ? kBKTF32 : kBK);
-                tma_2d(su32(st), jb.a1, k0, jb.ra + jb.m0, fb);
-                tma_2d(su32(st + kTileA), jb.a2, k0, jb.ra + jb.m0, fb);
-                tma_2d(su32(st + 2 * kTileA), jb.b1, k0, jb.rb + jb.n0, fb);
-                tma_2d(su32(st + 2 * kTileA + kTileB), jb.b2, k0, jb.rb + jb.n0, fb);
+                tma_2d_if(el, st, jb.a1, k0, ra, fb);
+                tma_2d_if(el, st + kTileA, jb.a2, k0, ra, fb);
+                tma_2d_if(el, st + 2 * kTileA, jb.b1, k0, rb, fb);
+                tma_2d_if(el, st + 2 * kTileA + kTileB, jb.b2, k0, rb, fb);
                 ++loaded;
+                if (++s == kStages) {
+                    s = 0;
+                    phase ^= 1;
+                }
             }
         }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------------------------------------------- MMA issuer
-        int it = 0, lt = 0;
+    } else if (warp == 1) {
+        // ---------------------------------------------------- MMA issuer (whole warp)
+        const uint32_t el = elect_one();
+        const uint64_t d0 = sdesc_sw128(su32(gsm));
+        const uint32_t full0 = su32(full), empty0 = su32(empty), tfull0 = su32(tfull), tempty0 = su32(tempty);
+        int s = 0, lt = 0;
+        uint32_t phase = 0;
         bool ok = true;
         int ks_next = blockIdx.x < (unsigned)tiles ? src.ksteps(blockIdx.x) : 0;
         for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x, ++lt) {
-            const int ksteps = ks_next;
+            const int ksteps = uniform(ks_next);
             if (t + (int)gridDim.x < tiles) ks_next = src.ksteps(t + gridDim.x);
             const int b = lt & 1;
-            const uint32_t buse = lt >> 1;
-            if (buse > 0 && !bar_wait(su32(&tempty[b]), (buse - 1) & 1, abort_flag, err, 2u)) break;
+            if (lt > 1 && !warp_wait<false>(tempty0 + b * 8, ((lt >> 1) - 1) & 1, abort_flag, err, 2u)) break;
             fence_after();
             const uint32_t d_hh = tmem + (uint32_t)(b * 256), d_x = d_hh + 128;
-            for (int ks = 0; ks < ksteps; ++ks, ++it) {
-                const int s = it % kStages;
-                const uint32_t use = it / kStages;
-                if (!bar_wait(su32(&full[s]), use & 1, abort_flag, err, 2u)) {
+            uint32_t acc = 0;
+            for (int ks = 0; ks < ksteps; ++ks) {
+                if (!warp_wait<false>(full0 + s * 8, phase, abort_flag, err, 2u)) {
                     ok = false;
                     break;
                 }
                 fence_after();
-                const uint32_t base = su32(gsm + (size_t)s * kStageBytes);
-                const uint32_t a1 = base, a2 = base + kTileA, b1 = base + 2 * kTileA, b2 = b1 + kTileB;
+                // descriptors: 32 bytes (16 BF16, 8 TF32) of each row per MMA are 2 units
+                const uint64_t a1 = d0 + (uint64_t)(s * (int)(kStageBytes >> 4)), a2 = a1 + (kTileA >> 4),
+                               b1 = a1 + (2 * kTileA >> 4), b2 = b1 + (kTileB >> 4);
 #pragma unroll
                 for (int kk = 0; kk < kBK / 16; ++kk) {
-                    const uint32_t off = kk * 32;  // 16 BF16 (8 TF32) along K inside the 128-byte row
-                    const uint32_t acc = (ks == 0 && kk == 0) ? 0u : 1u;
+                    const uint64_t o = kk * 2;
                     if constexpr (TF32) {
-                        mma_tf32<kIdescTF32>(d_hh, sdesc_sw128(a1 + off), sdesc_sw128(b1 + off), acc);
-                        mma_tf32<kIdescTF32>(d_x, sdesc_sw128(a1 + off), sdesc_sw128(b2 + off), acc);
-                        mma_tf32<kIdescTF32>(d_x, sdesc_sw128(a2 + off), sdesc_sw128(b1 + off), 1u);
+                        mma_tf32_if(el, d_hh, a1 + o, b1 + o, kIdescTF32, acc);
+                        mma_tf32_if(el, d_x, a1 + o, b2 + o, kIdescTF32, acc);
+                        mma_tf32_if(el, d_x, a2 + o, b1 + o, kIdescTF32, 1u);
                     } else {  // one accumulator: A1 B1, A1 B2, A2 B1 in this order
-                        mma_bf16<kIdesc>(d_hh, sdesc_sw128(a1 + off), sdesc_sw128(b1 + off), acc);
-                        mma_bf16<kIdesc>(d_hh, sdesc_sw128(a1 + off), sdesc_sw128(b2 + off), 1u);
-                        mma_bf16<kIdesc>(d_hh, sdesc_sw128(a2 + off), sdesc_sw128(b1 + off), 1u);
+                        mma_bf16_if(el, d_hh, a1 + o, b1 + o, kIdesc, acc);
+                        mma_bf16_if(el, d_hh, a1 + o, b2 + o, kIdesc, 1u);
+                        mma_bf16_if(el, d_hh, a2 + o, b1 + o, kIdesc, 1u);
                     }
+                    acc = 1;
                 }
-                mma_commit(su32(&empty[s]));
+                mma_commit_if(el, empty0 + s * 8);
+                if (++s == kStages) {
+                    s = 0;
+                    phase ^= 1;
+                }
             }
-            mma_commit(su32(&tfull[b]));  // accumulators of this tile complete
+            if (!ok) break;
+            mma_commit_if(el, tfull0 + b * 8);  // accumulators of this tile complete
             ++tiles_mma;
         }
     } else if (warp >= 4) {

@@ -223,8 +223,9 @@ __device__ __forceinline__ uint32_t elect_one() {
     asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(el));
     return el;
 }
-// the warp's index as a value the compiler knows to be warp-uniform
-__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+// a value that is the same in every lane, as one the compiler knows to be
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+__device__ __forceinline__ int uniform_warp() { return uniform((int)(threadIdx.x >> 5)); }
 // bounded wait of a whole warp; CLUSTER: ordered after the other CTA's arrivals
 template <bool CLUSTER>
 __device__ __forceinline__ bool warp_wait(uint32_t b, uint32_t par, volatile int *abort_flag, unsigned *err,
@@ -273,6 +274,14 @@ __device__ __forceinline__ void mma_bf16_if(uint32_t el, uint32_t d_tmem, uint64
     asm volatile(
         "{\n\t.reg .pred p, Q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 Q, %5, 0;\n\t"
         "@Q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(el)
+        : "memory");
+}
+__device__ __forceinline__ void mma_tf32_if(uint32_t el, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                            uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, Q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 Q, %5, 0;\n\t"
+        "@Q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(el)
         : "memory");
 }
