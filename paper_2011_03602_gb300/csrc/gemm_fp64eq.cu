@@ -570,9 +570,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
 
 // ------------------------------------------------------------ splitting
 // A (m x k, lda) -> ea and slices As[p] (m x kp each, p < s); one warp per row
-__global__ void eq_split_rows_kernel(const double *A, long long lda, int m, int k, int kp, int beta, int s,
-                                     int *ea, __nv_bfloat16 *As) {
-    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+__device__ __forceinline__ void split_rows(const double *A, long long lda, int m, int k, int kp, int beta, int s,
+                                           int *ea, __nv_bfloat16 *As, int block) {
+    const int row = block * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= m) return;
     const int lane = threadIdx.x & 31;
     const double *src = A + (long long)row * lda;
@@ -597,9 +597,8 @@ __global__ void eq_split_rows_kernel(const double *A, long long lda, int m, int 
 // Same split, one 256-thread CTA per row and 16-byte loads (lda even, A
 // 16-byte aligned): the row's second read hits L1, and each thread keeps
 // eight loads in flight in the exponent pass.
-__global__ void __launch_bounds__(256) eq_split_rows_v2_kernel(const double *A, long long lda, int m, int k, int kp,
-                                                             int beta, int s, int *ea, __nv_bfloat16 *As) {
-    const int row = blockIdx.x;
+__device__ __forceinline__ void split_row_v2(const double *A, long long lda, int m, int k, int kp, int beta, int s,
+                                             int *ea, __nv_bfloat16 *As, int row) {
     const double2 *src = reinterpret_cast<const double2 *>(A + (long long)row * lda);
     const int k2 = k >> 1;
     int mx = 0;
@@ -637,25 +636,48 @@ __global__ void __launch_bounds__(256) eq_split_rows_v2_kernel(const double *A, 
     }
 }
 
-// largest effective exponent of each column of B (k x n); grid.x column
-// blocks of 32, grid.y row chunks
-__global__ void eq_col_maxexp_kernel(const double *B, long long ldb, int k, int n, int rows_per, int *mxo) {
-    const int col = blockIdx.x * 32 + threadIdx.x;
-    const int r0 = blockIdx.y * rows_per, r1 = min(k, r0 + rows_per);
-    if (col >= n) return;
+// The split of A and, before it in the grid, the largest effective exponents
+// of B's columns (mxo, zero on entry; blocks of 32 columns x rows_per rows),
+// which the split of B waits for: one launch, so that the column blocks'
+// latency hides behind the rows' traffic.
+template <bool V2>
+__global__ void __launch_bounds__(256) eq_split_rows_kernel(const double *A, long long lda, int m, int k, int kp,
+                                                          int beta, int s, int *ea, __nv_bfloat16 *As,
+                                                          const double *B, long long ldb, int n, int rows_per,
+                                                          int col_blocks, int max_blocks, int *mxo) {
+    if ((int)blockIdx.x >= max_blocks) {
+        if (V2)
+            split_row_v2(A, lda, m, k, kp, beta, s, ea, As, blockIdx.x - max_blocks);
+        else
+            split_rows(A, lda, m, k, kp, beta, s, ea, As, blockIdx.x - max_blocks);
+        return;
+    }
+    const int col = (int)(blockIdx.x % col_blocks) * 32 + (threadIdx.x & 31);
+    const int r0 = (int)(blockIdx.x / col_blocks) * rows_per, r1 = min(k, r0 + rows_per);
     int mx = 0;
+    if (col < n) {
 #pragma unroll 8
-    for (int l = r0 + threadIdx.y; l < r1; l += blockDim.y) mx = max(mx, eff_exp(B[(long long)l * ldb + col]));
-    if (mx > 0) atomicMax(mxo + col, mx);
+        for (int l = r0 + (threadIdx.x >> 5); l < r1; l += 8) mx = max(mx, eff_exp(B[(long long)l * ldb + col]));
+    }
+    __shared__ int red[256];
+    red[threadIdx.x] = mx;
+    __syncthreads();
+    if (threadIdx.x < 32 && col < n) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) mx = max(mx, red[w * 32 + threadIdx.x]);
+        if (mx > 0) atomicMax(mxo + col, mx);
+    }
 }
 
-// B tile of 64 (k) x 64 (columns) -> transposed slices Bs[q] (n x kp each);
-// mxo holds the column maxima (exponent fields); 256 threads
+// B tile of 64 (k) x 64 (columns) -> transposed slices Bs[q] (n x kp each) and
+// the columns' scale exponents eb; mxo holds the column maxima (exponent
+// fields); 256 threads
 __global__ void eq_split_cols_t_kernel(const double *B, long long ldb, int k, int n, int kp, int beta, int s,
-                                       const int *mxo, __nv_bfloat16 *Bs) {
+                                       const int *mxo, int *eb, __nv_bfloat16 *Bs) {
     __shared__ double t[64][65];
     const int c0 = blockIdx.x * 64, l0 = blockIdx.y * 64;
     const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    if (l0 == 0 && ty == 0 && c0 + tx < n) eb[c0 + tx] = mxo[c0 + tx] == 0 ? 0 : mxo[c0 + tx] - 1022;
 #pragma unroll
     for (int yy = ty; yy < 64; yy += 4) {
         const int l = l0 + yy, c = c0 + tx;
@@ -675,11 +697,6 @@ __global__ void eq_split_cols_t_kernel(const double *B, long long ldb, int k, in
         for (int p = 0; p < s; ++p)
             reinterpret_cast<unsigned *>(dst)[p * (plane / 2)] = eq::digit_pair(X0, n0, X1, n1, beta, p);
     }
-}
-
-__global__ void eq_col_scale_kernel(const int *mxo, int *eb, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) eb[i] = mxo[i] == 0 ? 0 : mxo[i] - 1022;
 }
 
 size_t smem_eq() { return 1024 + (size_t)kStages * kStageBytes + 256; }
@@ -723,10 +740,10 @@ EqLayout eq_layout(int m, int n, int k) {
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     EqLayout L{};
     L.err = 0;
-    L.ea = 256;
+    L.mxo = 256;
+    L.ea = L.mxo + up((size_t)n * 4);
     L.eb = L.ea + up((size_t)m * 4);
-    L.mxo = L.eb + up((size_t)n * 4);
-    L.as = L.mxo + up((size_t)n * 4);
+    L.as = L.eb + up((size_t)n * 4);
     L.bs = L.as + up((size_t)e.slices * m * kp * 2);
     L.total = L.bs + up((size_t)e.slices * n * kp * 2);
     return L;
@@ -987,26 +1004,21 @@ void launch_gemm_fp64eq(int m, int n, int k, const double *A, long long lda, con
         launch_gemm_eq_tiles(m, n, k, As, Bs, ea, eb, C, ldc, width, err, sms, s);
         return;
     }
-    OO_CUDA_TRY(cudaMemsetAsync(err, 0, 4, s));
-    OO_CUDA_TRY(cudaMemsetAsync(mxo, 0, (size_t)n * 4, s));
+    OO_CUDA_TRY(cudaMemsetAsync(err, 0, L.ea - L.err, s));  // the error word and the column maxima
     {
-        const int rows_per = 256;
-        dim3 grid((n + 31) / 32, (k + rows_per - 1) / rows_per), block(32, 8);
-        OO_REQUIRE(grid.y <= 65535, OO_EINVAL, "k too large");
-        eq_col_maxexp_kernel<<<grid, block, 0, s>>>(B, ldb, k, n, rows_per, mxo);
-        OO_CUDA_TRY(cudaGetLastError());
-        eq_col_scale_kernel<<<(n + 255) / 256, 256, 0, s>>>(mxo, eb, n);
+        constexpr int kRowsPer = 128;  // 16 loads a thread, in two batches
+        const int col_blocks = (n + 31) / 32, max_blocks = col_blocks * ((k + kRowsPer - 1) / kRowsPer);
+        const bool v2 = lda % 2 == 0 && ((uintptr_t)A & 15u) == 0;
+        const long long blocks = (long long)max_blocks + (v2 ? m : (m + 7) / 8);
+        OO_REQUIRE(blocks < (1ll << 31), OO_EINVAL, "matrix too large");
+        (v2 ? eq_split_rows_kernel<true> : eq_split_rows_kernel<false>)<<<(unsigned)blocks, 256, 0, s>>>(
+            A, lda, m, k, kp, e.beta, e.slices, ea, As, B, ldb, n, kRowsPer, col_blocks, max_blocks, mxo);
         OO_CUDA_TRY(cudaGetLastError());
     }
-    if (lda % 2 == 0 && ((uintptr_t)A & 15u) == 0)
-        eq_split_rows_v2_kernel<<<m, 256, 0, s>>>(A, lda, m, k, kp, e.beta, e.slices, ea, As);
-    else
-        eq_split_rows_kernel<<<(m + 7) / 8, 256, 0, s>>>(A, lda, m, k, kp, e.beta, e.slices, ea, As);
-    OO_CUDA_TRY(cudaGetLastError());
     {
         dim3 grid((n + 63) / 64, kp / 64);
         OO_REQUIRE(grid.y <= 65535, OO_EINVAL, "k too large");
-        eq_split_cols_t_kernel<<<grid, 256, 0, s>>>(B, ldb, k, n, kp, e.beta, e.slices, mxo, Bs);
+        eq_split_cols_t_kernel<<<grid, 256, 0, s>>>(B, ldb, k, n, kp, e.beta, e.slices, mxo, eb, Bs);
         OO_CUDA_TRY(cudaGetLastError());
     }
     EqMaps maps;
