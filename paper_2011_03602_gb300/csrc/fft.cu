@@ -58,11 +58,11 @@ struct FftArgs {
 // stored in Stockham order: butterfly j's output p at column position
 // j R + p.  COLFAST: value r of the thread is t0 + r L/8 of one column, so
 // butterfly g takes r = g + m 8/R; otherwise value r = g R + m is
-// tid + m 512 of column g (L = 512 R).
+// tid + m T of column g (L = T R, T threads).
 template <int R, bool COLFAST, class Pos>
 __device__ __forceinline__ void first_stage_regs(float4 *sd, const float4 *v, const Pos &dst, int log2L, bool inv,
                                                  int ps) {
-    static_assert(kFftElems / kFftThreads == 8, "eight values per thread");
+    static_assert(kFftPer == 8, "eight values per thread");
     constexpr int G = 8 / R;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
@@ -86,26 +86,33 @@ __device__ __forceinline__ void first_stage_regs(float4 *sd, const float4 *v, co
 // and stores overlap the other's butterflies: 2^22 in 0.229 ms instead of
 // 0.262 ms with one.  PAD: the padded shared-memory layout (every pass
 // length but 2048, fft_padded), a template parameter so that the layout
-// shift is a constant.
-template <int MODE, bool PAD>
-__global__ void __launch_bounds__(kFftThreads, 2) fft_pass_kernel(FftArgs a) {
+// shift is a constant.  T threads hold 8 T values (fft_threads).
+template <int MODE, bool PAD, int T>
+__global__ void __launch_bounds__(T, 2 * (kFftThreads / T)) fft_pass_kernel(FftArgs a) {
     extern __shared__ __align__(16) float4 fsmem[];
     float4 *sd = fsmem;
     const int log2L = MODE == 0 ? a.log2n : (MODE == 1 ? a.log2n1 : a.log2n2);
     const int L = 1 << log2L;
-    const int C = kFftElems >> log2L;  // columns (transforms / rows) in this CTA
+    constexpr int E = T * kFftPer, kSlots = PAD ? E + E / 8 : E;
+    const int C = E >> log2L;  // columns (transforms / rows) in this CTA
     const bool inv = a.inverse != 0;
-    const float4 *stw = a.tw;  // the 4096-point table is read in place
+    // The stage table goes after the data (the 4096-point one is read in
+    // place): copied when the data's loads are in flight, one latency instead of
+    // two, but here in the full CTAs of the four-step passes, which have no
+    // registers for both (2^22 in 212 us with the spills that costs).
+    constexpr bool kTableFirst = MODE != 0 && T == kFftThreads;
+    const float4 *stw = a.tw;
     if (twiddles_staged(log2L)) {
-        float4 *t_s = fsmem + (PAD ? kFftElemsPad : kFftElems);
-        for (int t = threadIdx.x; t < stage_table_count(log2L); t += kFftThreads) t_s[t] = a.tw[t];
+        float4 *t_s = fsmem + kSlots;
+        if (kTableFirst)
+            for (int t = threadIdx.x; t < stage_table_count(log2L); t += T) t_s[t] = a.tw[t];
         stw = t_s;
     }
     // the columns' largest exponents (modes 0, 1), after the staged table
-    int *smax = reinterpret_cast<int *>(fsmem + (PAD ? kFftElemsPad : kFftElems) + (twiddles_staged(log2L) ? L : 0));
+    int *smax = reinterpret_cast<int *>(fsmem + kSlots + (twiddles_staged(log2L) ? L : 0));
     constexpr int ps = PAD ? 3 : 30;  // data layout: fft_pad_shift(log2L)
     if (MODE != 2)
-        for (int t = threadIdx.x; t < C; t += kFftThreads) smax[t] = 0;
+        for (int t = threadIdx.x; t < C; t += T) smax[t] = 0;
 
     const long long n = a.n;
     const int N1 = 1 << a.log2n1, N2 = 1 << a.log2n2;
@@ -121,25 +128,27 @@ __global__ void __launch_bounds__(kFftThreads, 2) fft_pass_kernel(FftArgs a) {
     // ---- load: all of this thread's 16-byte loads are issued before any is
     // used (eight in flight), then split and stored to shared memory -- after
     // the first stage, done in registers where this thread holds whole
-    // butterflies of it: column-fastest loads (MODE 1) give it x[t0 + r L/8],
-    // r < 8, of one column; row-fastest loads (MODE 0 / 2) give it, for
-    // L = 1024, 2048, 4096, x[tid + m 512], m < L / 512 = the first radix, of
-    // each of its columns
-    constexpr int kPer = kFftElems / kFftThreads;
+    // butterflies of it: column-fastest loads (MODE 1), and row-fastest ones
+    // of a small CTA that holds one column, give it x[t0 + r L/8], r < 8, of
+    // one column; row-fastest loads of a full CTA give it x[tid + m T], m <
+    // L / T, of each of its columns, the butterflies where L / T is the first
+    // radix (L = 1024, 2048, 4096)
+    constexpr int kPer = kFftPer;
+    constexpr bool kColFast = MODE == 1 || T < kFftThreads;
     const int b0 = first_radix_log2(log2L);
-    const bool first_here = MODE == 1 ? log2L >= 3 : (log2L >= 10 && log2L <= 12);
+    const bool first_here = MODE == 1 ? log2L >= 3 : (kColFast ? L == E : (log2L >= 10 && log2L <= 12));
     {
         // shared-memory position of value r of this thread: column c, element
         // t at (c << log2L) + t, which row-fastest is q itself
         auto dst = [&](int r) {
-            const int q = threadIdx.x + r * kFftThreads;
+            const int q = threadIdx.x + r * T;
             if (MODE == 1) return ((q & (C - 1)) << log2L) + (q >> (31 - __clz(C)));
             return q;
         };
         double2 raw[kPer];
 #pragma unroll
         for (int r = 0; r < kPer; ++r) {
-            const int q = threadIdx.x + r * kFftThreads;
+            const int q = threadIdx.x + r * T;
             int c, t;
             if (MODE == 1) {  // column-fastest for coalescing
                 c = q & (C - 1);
@@ -159,6 +168,8 @@ __global__ void __launch_bounds__(kFftThreads, 2) fft_pass_kernel(FftArgs a) {
                                       __hiloint2double(__float_as_int(f.w), __float_as_int(f.z)));
             }
         }
+        if (!kTableFirst && twiddles_staged(log2L))
+            for (int t = threadIdx.x; t < stage_table_count(log2L); t += T) fsmem[kSlots + t] = a.tw[t];
         float4 v[kPer];
         if (MODE == 2) {
             // float-float intermediates: the 16 bytes as they were, brought
@@ -199,11 +210,11 @@ __global__ void __launch_bounds__(kFftThreads, 2) fft_pass_kernel(FftArgs a) {
         }
         if (first_here) {
             if (b0 == 1)
-                first_stage_regs<2, MODE == 1>(sd, v, dst, log2L, inv, ps);
+                first_stage_regs<2, kColFast>(sd, v, dst, log2L, inv, ps);
             else if (b0 == 2)
-                first_stage_regs<4, MODE == 1>(sd, v, dst, log2L, inv, ps);
+                first_stage_regs<4, kColFast>(sd, v, dst, log2L, inv, ps);
             else
-                first_stage_regs<8, MODE == 1>(sd, v, dst, log2L, inv, ps);
+                first_stage_regs<8, kColFast>(sd, v, dst, log2L, inv, ps);
         } else {
 #pragma unroll
             for (int r = 0; r < kPer; ++r) sd[sp(dst(r), ps)] = v[r];
@@ -212,12 +223,12 @@ __global__ void __launch_bounds__(kFftThreads, 2) fft_pass_kernel(FftArgs a) {
     __syncthreads();
 
     if (first_here)
-        fft_in_smem_after_first(sd, stw, log2L, inv, ps);
+        fft_in_smem_after_first<T>(sd, stw, log2L, inv, ps);
     else
-        fft_in_smem(sd, stw, log2L, inv, ps);
+        fft_in_smem<T>(sd, stw, log2L, inv, ps);
 
     // ---- store
-    for (int q = threadIdx.x; q < kFftElems; q += kFftThreads) {
+    for (int q = threadIdx.x; q < E; q += T) {
         int c, t;
         if (MODE == 0) {
             c = q >> log2L;
@@ -290,6 +301,56 @@ __global__ void __launch_bounds__(kFftThreads, 2)
         const FftItem item = items[it];
         fft_group_item(item, reqs, tlist, expo, fsmem, false);
     }
+}
+
+}  // namespace
+
+namespace {
+
+int num_sms() {
+    int dev = 0, n = 148;
+    OO_CUDA_TRY(cudaGetDevice(&dev));
+    OO_CUDA_TRY(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return n;
+}
+
+// Threads of a pass's CTAs (eight values each).  A CTA of 512 serves 4096
+// values at the best rate, but all of them in step: with few columns, most of
+// it is padding (one 1024-point transform in a CTA of four) and most SMs are
+// idle.  Where CTAs of 512 would not give every SM two, a CTA has 128
+// threads, more if that is less than one transform or, in a four-step pass,
+// two columns (a single column's loads use half of each sector).  Passes of
+// 1024 points and more keep full CTAs as long as every SM has one: 2^20 takes
+// 61 us in CTAs of 512, 66 and 69 with two columns and one.  us with CTAs of
+// 512 / so: 2^10 14.4 / 12.3, 2^13 33.5 / 21.7, 2^16 35.7 / 22.3, 64 x 2^14 55.4
+// / 48.9, 64 x 2^10 18.5 / 12.3; 256 x 2^14, which fills the SMs either way,
+// 172.4 in CTAs of 512.
+int fft_threads(int mode, int log2L, long long columns, int sms) {
+    const long long full = (columns * (1ll << log2L) + kFftElems - 1) / kFftElems;
+    if (full >= 2ll * sms || (mode != 0 && log2L >= 10 && full >= sms)) return kFftThreads;
+    return std::max(128, std::min(kFftThreads, (1 << log2L) * (mode == 0 ? 1 : 2) / kFftPer));
+}
+
+struct FftPass {
+    const void *fn;
+    std::atomic<uint64_t> *limit_set;
+};
+template <int MODE, bool PAD, int T>
+FftPass fft_pass_entry() {
+    static std::atomic<uint64_t> limit_set{0};
+    return {(const void *)fft_pass_kernel<MODE, PAD, T>, &limit_set};
+}
+template <int MODE>
+FftPass fft_pass_of(bool pad, int T) {
+    // unpadded passes have 2048 points: 256 threads or 512
+    if (!pad) return T == 256 ? fft_pass_entry<MODE, false, 256>() : fft_pass_entry<MODE, false, 512>();
+    return T == 128   ? fft_pass_entry<MODE, true, 128>()
+           : T == 256 ? fft_pass_entry<MODE, true, 256>()
+                      : fft_pass_entry<MODE, true, 512>();
+}
+// the pass kernel of a mode, in the layout of a pass length, for T threads
+FftPass fft_pass(int mode, bool pad, int T) {
+    return mode == 0 ? fft_pass_of<0>(pad, T) : (mode == 1 ? fft_pass_of<1>(pad, T) : fft_pass_of<2>(pad, T));
 }
 
 }  // namespace
@@ -415,48 +476,30 @@ void launch_fft(const FftPlan *p, int batch, int dir, const double *in, double *
     a.n = n;
     a.batch = batch;
     a.inverse = dir > 0 ? 1 : 0;
-    static std::atomic<uint64_t> attr_done[6];
-    auto smem_for = [&](int log2L) { return fft_smem_bytes(log2L); };
-    // the pass kernel of a mode in the layout of a pass length, its shared-
-    // memory limit raised once per device
-    auto pick = [&](int mode, int log2L) {
-        const bool pad = fft_padded(log2L);
-        const void *fn = mode == 0 ? (pad ? (const void *)fft_pass_kernel<0, true> : (const void *)fft_pass_kernel<0, false>)
-                       : mode == 1 ? (pad ? (const void *)fft_pass_kernel<1, true> : (const void *)fft_pass_kernel<1, false>)
-                                   : (pad ? (const void *)fft_pass_kernel<2, true> : (const void *)fft_pass_kernel<2, false>);
-        set_smem_limit_once(fn, kFftSmemMax, attr_done[2 * mode + (pad ? 1 : 0)]);
-        return fn;
-    };
-    auto launch = [&](const void *fn, long long grid, size_t smem) {
+    auto pass = [&](int mode, int log2L, long long columns) {
+        const int T = fft_threads(mode, log2L, columns, num_sms());
+        const FftPass p = fft_pass(mode, fft_padded(log2L), T);
+        set_smem_limit_once(p.fn, kFftSmemMax, *p.limit_set);
+        const long long C = (long long)(T * kFftPer) >> log2L;
         void *args[] = {&a};
-        OO_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kFftThreads), args, smem, s));
+        OO_CUDA_TRY(cudaLaunchKernel(p.fn, dim3((unsigned)((columns + C - 1) / C)), dim3(T), args,
+                                     fft_smem_bytes(log2L, T * kFftPer), s));
     };
     if (!four_step) {
-        const int C = kFftElems >> p->log2n;
-        const int grid = (int)((batch + C - 1) / C);
         a.in_d = in;
         a.out_d = out;
         a.tw = p->tw_single;
-        launch(pick(0, p->log2n), grid, smem_for(p->log2n));
+        pass(0, p->log2n, batch);
         return;
     }
-    const int N1 = 1 << p->log2n1, N2 = 1 << p->log2n2;
     a.tw_hi = p->tw_hi;
     a.tw_lo = p->tw_lo;
-    {
-        a.in_d = in;
-        a.tw = p->tw_n1;
-        const int C = kFftElems / N1;
-        const long long grid = (long long)batch * (N2 / C);
-        launch(pick(1, p->log2n1), grid, smem_for(p->log2n1));
-    }
-    {
-        a.out_d = out;
-        a.tw = p->tw_n2;
-        const int R = kFftElems / N2;
-        const long long grid = (long long)batch * (N1 / R);
-        launch(pick(2, p->log2n2), grid, smem_for(p->log2n2));
-    }
+    a.in_d = in;
+    a.tw = p->tw_n1;
+    pass(1, p->log2n1, (long long)batch << p->log2n2);
+    a.out_d = out;
+    a.tw = p->tw_n2;
+    pass(2, p->log2n2, (long long)batch << p->log2n1);
 }
 
 // ------------------------------------------------------------ group plans

@@ -76,9 +76,9 @@ __device__ __forceinline__ cplx norm(const cplx &a) {
 
 namespace {
 
-constexpr int kFftThreads = 512;
-constexpr int kFftBpt = 2;                               // (8 values per thread: 8 / R radix-R butterflies)
-constexpr int kFftElems = 4 * kFftThreads * kFftBpt;     // 4096 values per CTA
+constexpr int kFftThreads = 512;                  // of a full CTA; launches of few CTAs use smaller ones (fft.cu)
+constexpr int kFftPer = 8;                        // values per thread: 8 / R radix-R butterflies
+constexpr int kFftElems = kFftThreads * kFftPer;  // 4096 values per full CTA
 // The values sit in shared memory with one float4 of padding after every
 // eight (value i at sp(i, 3)), so the strided stores of the Stockham stages
 // (R or R Ls float4 apart) and the loads across short columns fall in eight
@@ -90,7 +90,9 @@ constexpr int kFftElems = 4 * kFftThreads * kFftBpt;     // 4096 values per CTA
 constexpr int kFftElemsPad = kFftElems + kFftElems / 8;
 __host__ __device__ __forceinline__ bool fft_padded(int log2L) { return log2L != 11; }
 __host__ __device__ __forceinline__ int fft_pad_shift(int log2L) { return fft_padded(log2L) ? 3 : 30; }
-__host__ __device__ __forceinline__ int fft_data_slots(int log2L) { return fft_padded(log2L) ? kFftElemsPad : kFftElems; }
+__host__ __device__ __forceinline__ int fft_data_slots(int log2L, int elems = kFftElems) {
+    return fft_padded(log2L) ? elems + elems / 8 : elems;
+}
 __host__ __device__ __forceinline__ int sp(int i, int ps) { return ps >= 30 ? i : i + (i >> ps); }
 constexpr int kTwSplit = 11;                             // four-step twiddle split: 2^11
 
@@ -174,12 +176,12 @@ __host__ __device__ __forceinline__ bool twiddles_staged(int log2L) { return log
 // Shared memory of a CTA running a pass of length 2^log2L: the data, the
 // staged table (if any), then one int per column of the CTA (its largest
 // input exponent), 16-byte aligned.
-__host__ __device__ __forceinline__ size_t fft_colmax_bytes(int log2L) {
-    return ((size_t)(kFftElems >> log2L) * 4 + 15) / 16 * 16;
+__host__ __device__ __forceinline__ size_t fft_colmax_bytes(int log2L, int elems = kFftElems) {
+    return ((size_t)(elems >> log2L) * 4 + 15) / 16 * 16;
 }
-__host__ __device__ __forceinline__ size_t fft_smem_bytes(int log2L) {
-    return (size_t)(fft_data_slots(log2L) + (twiddles_staged(log2L) ? (1 << log2L) : 0)) * 16 +
-           fft_colmax_bytes(log2L);
+__host__ __device__ __forceinline__ size_t fft_smem_bytes(int log2L, int elems = kFftElems) {
+    return (size_t)(fft_data_slots(log2L, elems) + (twiddles_staged(log2L) ? (1 << log2L) : 0)) * 16 +
+           fft_colmax_bytes(log2L, elems);
 }
 // the largest of those (L = 2048, unpadded: 96 KB + 16 bytes)
 constexpr size_t kFftSmemMax = (size_t)(kFftElems + 2048) * 16 + 16;
@@ -266,17 +268,18 @@ __device__ __forceinline__ void dft_small(cplx *x, bool inv) {
 
 __host__ __device__ constexpr int ilog2c(int v) { return v <= 1 ? 0 : 1 + ilog2c(v >> 1); }
 
-// One Stockham stage of radix R over the CTA's kFftElems values (C columns of
-// length L): 8 / R butterflies per thread; value i at sd[sp(i, ps)].
-template <int R>
+// One Stockham stage of radix R over the values of a CTA of T threads (8 T
+// values, columns of length L): 8 / R butterflies per thread; value i at
+// sd[sp(i, ps)].
+template <int R, int T>
 __device__ __forceinline__ void stage_radix(float4 *sd, const float4 *stw, int log2L, int Ls, bool inv, int ps) {
-    constexpr int B = kFftElems / (R * kFftThreads);
+    constexpr int B = kFftPer / R;
     const int log2lr = log2L - ilog2c(R), lr = 1 << log2lr;
     cplx Y[B][R];
     int base_c[B], jj[B];
 #pragma unroll
     for (int b = 0; b < B; ++b) {
-        const int bidx = threadIdx.x + b * kFftThreads;
+        const int bidx = threadIdx.x + b * T;
         const int c = bidx >> log2lr, j = bidx & (lr - 1);
         base_c[b] = c << log2L;
         jj[b] = j;
@@ -302,24 +305,26 @@ __device__ __forceinline__ void stage_radix(float4 *sd, const float4 *stw, int l
 
 // the radix-8 stages after the first stage (which the caller has done);
 // inlined, so a caller's constant layout shift ps stays a constant
+template <int T>
 __device__ __forceinline__ void fft_in_smem_after_first(float4 *sd, const float4 *stw, int log2L, bool inv, int ps) {
     for (int Ls = 1 << first_radix_log2(log2L); Ls < (1 << log2L); Ls *= 8) {
-        stage_radix<8>(sd, stw, log2L, Ls, inv, ps);
+        stage_radix<8, T>(sd, stw, log2L, Ls, inv, ps);
         stw += 7 * Ls;
     }
 }
 
 // the whole transform of every column in shared memory
+template <int T>
 __device__ __forceinline__ void fft_in_smem(float4 *sd, const float4 *stw, int log2L, bool inv, int ps) {
     if (log2L == 0) return;
     const int b0 = first_radix_log2(log2L);
     if (b0 == 1)
-        stage_radix<2>(sd, stw, log2L, 1, inv, ps);
+        stage_radix<2, T>(sd, stw, log2L, 1, inv, ps);
     else if (b0 == 2)
-        stage_radix<4>(sd, stw, log2L, 1, inv, ps);
+        stage_radix<4, T>(sd, stw, log2L, 1, inv, ps);
     else
-        stage_radix<8>(sd, stw, log2L, 1, inv, ps);
-    fft_in_smem_after_first(sd, stw, log2L, inv, ps);
+        stage_radix<8, T>(sd, stw, log2L, 1, inv, ps);
+    fft_in_smem_after_first<T>(sd, stw, log2L, inv, ps);
 }
 
 // largest biased exponent among the 64-bit words [x0, x1) of p (stride
@@ -436,7 +441,7 @@ __device__ __forceinline__ void fft_group_item(const FftItem &item, const FftGro
     for (int t = threadIdx.x; t < C; t += kFftThreads) smax[t] = 0;
     const float4 *tws = staged ? stw : tw;
     const int N1 = 1 << R0.log2n1, N2 = 1 << R0.log2n2;
-    constexpr int kPer = kFftElems / kFftThreads;
+    constexpr int kPer = kFftPer;
     // value r of this thread: column c, position t
     auto coords = [&](int r, int &c, int &t) {
         const int q = threadIdx.x + r * kFftThreads;
@@ -503,7 +508,7 @@ __device__ __forceinline__ void fft_group_item(const FftItem &item, const FftGro
         }
     }
     __syncthreads();
-    fft_in_smem(sd, tws, log2L, inv, ps);
+    fft_in_smem<kFftThreads>(sd, tws, log2L, inv, ps);
     // ---- store
     for (int q = threadIdx.x; q < kFftElems; q += kFftThreads) {
         int c, t;
