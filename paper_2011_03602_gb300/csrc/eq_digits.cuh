@@ -18,8 +18,9 @@
 // Three ways to accumulate the products (a "scheme", a fixed function of k
 // so that a problem gives the same bits alone and inside a batch):
 //   kSchemePairs  one accumulator per product D_pq, products sharing A_p
-//                 paired into one N = 2 BN MMA (kb <= 1024: beta 8 when
-//                 kb <= 256, else 7); the epilogue reads every product.
+//                 paired into one N = 2 BN MMA (kb <= 1024, the K-blocks of a
+//                 product about equally long: beta 8 when kb <= 256, else 7);
+//                 the epilogue reads every product.
 //   kSchemeLevel7 one accumulator per level s = p + q: every D_pq of the
 //                 level summed in the same FP32 accumulator, which stays
 //                 exact with beta = 7 and kb = 128 ((L - 1) kb 127^2 < 2^24);
@@ -34,6 +35,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "ff.cuh"
 #include "tc.cuh"
 
 namespace oo {
@@ -64,7 +66,10 @@ inline Shape shape(int scheme, int k) {
         e.kb = std::min(kp, 512);
         e.beta = 6;
     } else {
-        e.kb = std::min(kp, 1024);
+        // the fewest K-blocks of at most 1024 terms, all about as long: a short
+        // last one costs as much as a full one, the epilogue's time
+        const int steps = kp / kBK, blocks = (kp + 1023) / 1024;
+        e.kb = (steps + blocks - 1) / blocks * kBK;
         e.beta = e.kb <= 256 ? 8 : 7;
     }
     e.levels = level_bound(e.beta);
@@ -124,6 +129,73 @@ __device__ __forceinline__ unsigned digit_bits(unsigned long long X, unsigned ne
 __device__ __forceinline__ unsigned digit_pair(unsigned long long X0, unsigned n0, unsigned long long X1, unsigned n1,
                                                int beta, int p) {
     return digit_bits(X0, n0, beta, p) | (digit_bits(X1, n1, beta, p) << 16);
+}
+
+// (Sh, Sl) += d f, f a power of two, without renormalising (7 operations; a
+// scaling and ff::add take 12): as it is for the levels of a level scheme, nine
+// at most; followed by renormalise(), which makes |Sl| <= ulp(Sh) / 2 again, for
+// the many products of the pair scheme (once per two products would save
+// three operations and cost 2 to 4 % in error from k = 4096 on).
+__device__ __forceinline__ void add_scaled(float &Sh, float &Sl, float d, float f) {
+    const float s = __fmaf_rn(d, f, Sh);
+    const float bb = __fsub_rn(s, Sh);
+    const float e = __fadd_rn(__fsub_rn(Sh, __fsub_rn(s, bb)), __fmaf_rn(d, f, -bb));
+    Sh = s;
+    Sl = __fadd_rn(Sl, e);
+}
+__device__ __forceinline__ void renormalise(float &Sh, float &Sl) { ff::fast_two_sum(Sh, Sl, Sh, Sl); }
+
+// (h + l) 2^S as a double, rounded once: the high part's bits and the low
+// part as an integer in units of the double's last place (ff::to_double's case
+// analysis took twice the instructions).  Zero, results near the ends of the
+// range and the flag scales of non-finite rows and columns take the general
+// conversion.
+__device__ __forceinline__ double scaled_value(float h, float l, int S) {
+    float s, e;
+    ff::two_sum(h, l, s, e);
+    const unsigned b = __float_as_uint(s), m = b & 0x7fffffu;
+    const int es = (int)((b >> 23) & 0xffu), ed = es - 127 + 1023 + S;
+    if ((unsigned)(es - 64) > 126u || (unsigned)(ed - 2) > 2043u) return tc::nan_or_scaled(ff::to_double(h, l), S);
+    // the last place is half as large below a power of two
+    const int below = m == 0 && (int)(__float_as_uint(e) ^ b) < 0;
+    int t = __float2int_rn(__fmul_rn(e, __uint_as_float((unsigned)(306 + below - es) << 23)));  // |t| <= 2^28
+    if (b >> 31) t = -t;
+    const unsigned long long v = ((unsigned long long)(unsigned)ed << 52) + ((unsigned long long)m << 29) +
+                                 (unsigned long long)(long long)t;
+    return __longlong_as_double((long long)(v | ((unsigned long long)(b >> 31) << 63)));
+}
+
+// An epilogue warp's sums -- lane l holds row row0 + l, columns c0 + j -- to C
+// through `out`, 32 rows x 8 columns of float pairs of the warp's own shared
+// memory (kOutBytes), so that 8-byte stores go out as 64-byte row segments and
+// the conversion is a loop, not unrolled over the columns.  With a row per
+// lane and the unrolled conversion a 256 x 128 tile of the pair scheme took
+// 122,000 clocks here, most of them instruction fetches and store replays.
+// ea: row l's scale; eb: columns l and 32 + l's; nrows, ncols: those that exist.
+constexpr uint32_t kOutBytes = 32 * 8 * 8;
+template <int NC>
+__device__ __forceinline__ void store_columns(const float (&Sh)[NC], const float (&Sl)[NC], unsigned char *stage,
+                                              double *C, long long ldc, int row0, int c0, int nrows, int ncols,
+                                              int ea, const int (&eb)[(NC + 31) / 32]) {
+    float2 *out = reinterpret_cast<float2 *>(stage);
+    const int lane = threadIdx.x & 31, col = lane & 7;
+#pragma unroll
+    for (int c = 0; c < NC; c += 8) {
+        if (c >= ncols) continue;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) out[lane * 8 + (j ^ (lane & 7))] = make_float2(Sh[c + j], Sl[c + j]);
+        __syncwarp();
+        const int sb = __shfl_sync(0xffffffffu, eb[c / 32], (c & 31) + col);
+        const bool col_ok = c + col < ncols;
+        double *dst = C + (long long)(row0 + (lane >> 3)) * ldc + c0 + c + col;
+#pragma unroll 1
+        for (int r = lane >> 3; r < 32; r += 4, dst += 4 * ldc) {
+            const float2 v = out[r * 8 + (col ^ (r & 7))];
+            const int sa = __shfl_sync(0xffffffffu, ea, r);
+            if (col_ok && r < nrows) *dst = scaled_value(v.x, v.y, sa + sb);
+        }
+        __syncwarp();
+    }
 }
 
 // One product's split job arguments (grouped products and the serving loop)

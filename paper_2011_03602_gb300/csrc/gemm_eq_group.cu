@@ -133,19 +133,10 @@ __device__ __forceinline__ void mma_rt(uint32_t d_tmem, uint64_t a, uint64_t b, 
         : "memory");
 }
 
-#define OO_TMEM_LD16(taddr, r)                                                                              \
-    asm volatile(                                                                                           \
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "  \
-        "[%16];"                                                                                            \
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),   \
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),          \
-          "=r"(r[15])                                                                                       \
-        : "r"(taddr))
-
 // Shared-memory pipeline of one tile CTA: a 4-stage operand ring, two
 // accumulator buffers in tensor memory, an abort flag.
 struct Pipe {
-    unsigned char *sm;
+    unsigned char *sm, *out;  // operand ring; the epilogue warps' store staging
     uint64_t *full, *empty, *tfull, *tempty;
     volatile int *abort_flag;
     uint32_t tmem;
@@ -158,7 +149,8 @@ __device__ __forceinline__ Pipe pipe_setup(uint64_t **extra_bars) {
     Pipe pp;
     pp.sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(gsm_raw) + 1023) &
                                               ~static_cast<uintptr_t>(1023));
-    uint64_t *bars = reinterpret_cast<uint64_t *>(pp.sm + kStages * kStageBytes);
+    pp.out = pp.sm + kStages * kStageBytes;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(pp.out + kEpiWarps * eq::kOutBytes);
     pp.full = bars;
     pp.empty = bars + kStages;
     pp.tfull = bars + 2 * kStages;
@@ -272,36 +264,6 @@ __device__ __forceinline__ bool mma_tile(const GArgs &a, const Pipe &pp, const G
     return true;
 }
 
-// (Sh, Sl) += d f, f a power of two: the levels of a level scheme, nine at
-// most, so the low parts are summed without renormalising (7 operations for
-// 12; each level's own rounding stays below 2^-47 of the sum).
-__device__ __forceinline__ void level_add(float &Sh, float &Sl, float d, float f) {
-    const float s = __fmaf_rn(d, f, Sh);
-    const float bb = __fsub_rn(s, Sh);
-    const float e = __fadd_rn(__fsub_rn(Sh, __fsub_rn(s, bb)), __fmaf_rn(d, f, -bb));
-    Sh = s;
-    Sl = __fadd_rn(Sl, e);
-}
-
-// (h + l) 2^S as a double, rounded once, for a level sum: the high part's
-// bits and the low part as an integer in units of the double's last place
-// (ff::to_double's case analysis took twice the instructions).  Zero, results
-// near the ends of the range and the flag scales of non-finite rows and
-// columns take the general conversion.
-__device__ __forceinline__ double level_value(float h, float l, int S) {
-    float s, e;
-    ff::two_sum(h, l, s, e);
-    const unsigned b = __float_as_uint(s), m = b & 0x7fffffu;
-    const int es = (int)((b >> 23) & 0xffu), ed = es - 127 + 1023 + S;
-    if ((unsigned)(es - 64) > 126u || (unsigned)(ed - 2) > 2043u) return nan_or_scaled(ff::to_double(h, l), S);
-    int t = __float2int_rn(__fmul_rn(e, __uint_as_float((unsigned)(306 - es) << 23)));  // |t| <= 2^28
-    if (b >> 31) t = -t;
-    if (m == 0 && t < 0) t += t;  // the last place is half as large below a power of two
-    const unsigned long long v = ((unsigned long long)(unsigned)ed << 52) + ((unsigned long long)m << 29) +
-                                 (unsigned long long)(long long)t;
-    return __longlong_as_double((long long)(v | ((unsigned long long)(b >> 31) << 63)));
-}
-
 // One epilogue warp (of eight: lane quarter q = warp & 3, column half h):
 // add every finished unit of one tile, scaled by its power of two, into a
 // float-float running sum (Sh, Sl) of this row's columns, then write FP64
@@ -319,6 +281,8 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
     const bool active = row0 < P.m && ncols > 0;  // warp-uniform
     const int units = P.nkb * S.nunits;
     const bool levels = P.scheme >= kTabLevel7;
+#pragma unroll
+    for (int j = 0; j < 64; ++j) Sh[j] = Sl[j] = 0.0f;
     for (int uu = 0; uu < units; ++uu, ++gu) {
         const int b = gu & 1;
         if (!bar_wait(su32(&pp.tfull[b]), (gu >> 1) & 1, pp.abort_flag, a.err, 4u)) return false;
@@ -334,27 +298,17 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
                     OO_TMEM_LD16(acc + c, v);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float w = __fmul_rn(__uint_as_float(v[j]), fL);  // exact: power of two
-                        if (uu == 0) {
-                            Sh[c + j] = w;
-                            Sl[c + j] = 0.0f;
-                        } else if (levels) {
-                            level_add(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), fL);
-                        } else {
-                            ff::add(Sh[c + j], Sl[c + j], w, 0.0f, Sh[c + j], Sl[c + j]);
-                        }
+                    for (int j = 0; j < 16; ++j) {  // fL, fR: powers of two, exact scales
+                        eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), fL);
+                        if (!levels) eq::renormalise(Sh[c + j], Sl[c + j]);
                     }
                     if (fR != 0.0f) {
                         OO_TMEM_LD16(acc + (uint32_t)td.w + c, v);
                         tmem_wait_ld();
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
-                            const float w = __fmul_rn(__uint_as_float(v[j]), fR);
-                            if (levels)
-                                level_add(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), fR);
-                            else
-                                ff::add(Sh[c + j], Sl[c + j], w, 0.0f, Sh[c + j], Sl[c + j]);
+                            eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), fR);
+                            if (!levels) eq::renormalise(Sh[c + j], Sl[c + j]);
                         }
                     }
                 }
@@ -365,24 +319,11 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
         if (lane == 0) bar_arrive(su32(&pp.tempty[b]));
     }
     if (active) {
-        // column scales: lane l holds columns l and l + 32 of this warp's
-        // range and hands them out by shuffle
-        const int row = row0 + lane;
         const int c0 = td.z + cw0;
-        const int e0 = lane < ncols ? P.eb[c0 + lane] : 0;
-        const int e1 = 32 + lane < ncols ? P.eb[c0 + 32 + lane] : 0;
-        const bool row_ok = row < P.m;
-        const int sa = row_ok ? P.ea[row] : 0;
-        double *crow = P.C + (long long)row * P.ldc + c0;
-#pragma unroll
-        for (int j = 0; j < 64; ++j) {
-            if (j < ncols) {
-                const int sb = __shfl_sync(0xffffffffu, j < 32 ? e0 : e1, j & 31);
-                if (row_ok)
-                    crow[j] = levels ? level_value(Sh[j], Sl[j], sa + sb)
-                                     : nan_or_scaled(ff::to_double(Sh[j], Sl[j]), sa + sb);
-            }
-        }
+        const int eb[2] = {lane < ncols ? P.eb[c0 + lane] : 0, 32 + lane < ncols ? P.eb[c0 + 32 + lane] : 0};
+        const int ea = row0 + lane < P.m ? P.ea[row0 + lane] : 0;
+        eq::store_columns(Sh, Sl, pp.out + (warp - 2) * eq::kOutBytes, P.C, P.ldc, row0, c0, min(32, P.m - row0),
+                          ncols, ea, eb);
     }
     return true;
 }
@@ -480,8 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_eq_group_kernel(const __grid
 constexpr int kLvSlots = 5, kLvWidth = 64, kLvMax = 8;
 constexpr int kLvThreads = 352;  // A producer, MMA issuer, 8 epilogue warps, B producer
 constexpr uint32_t kLvB = kLvMax * kLvWidth * kBK * 2;  // B slices of a K step: 64 KB
-constexpr uint32_t kLvOut = 32 * 8 * 8;                 // an epilogue warp's 32 rows x 8 columns
-constexpr size_t kLvSmem = 1024 + (size_t)kLvSlots * kTileA + 2 * (size_t)kLvB + kEpiWarps * kLvOut + 256;
+constexpr size_t kLvSmem = 1024 + (size_t)kLvSlots * kTileA + 2 * (size_t)kLvB + kEpiWarps * eq::kOutBytes + 256;
 static_assert(kLvSmem <= 232448, "level kernel exceeds the shared memory of a CTA");
 
 struct LvMaps {
@@ -596,11 +536,8 @@ __device__ __forceinline__ bool lv_mma(unsigned *err, const LvPipe &pp, const GP
 }
 
 // One epilogue warp of one tile: every level into a float-float sum per
-// column of the lane's row, then C through a small shared-memory transpose.
-// The loops over levels and rows stay rolled and 8-byte stores go out as
-// 64-byte row segments: unrolled over 32 columns, with a row per lane, the
-// conversion and the stores took 27,000 clocks a tile, most of them
-// instruction fetches and store replays.
+// column of the lane's row, then C (eq::store_columns; with the conversion
+// unrolled over the columns and a row per lane this took 27,000 clocks a tile).
 __device__ __forceinline__ bool lv_epilogue(unsigned *err, const LvPipe &pp, const GProb &P, const int4 &td,
                                             int tile) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -641,33 +578,16 @@ __device__ __forceinline__ bool lv_epilogue(unsigned *err, const LvPipe &pp, con
         if (active) {
             const float f = __uint_as_float((uint32_t)(127 - beta * s) << 23);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) level_add(Sh[j], Sl[j], __uint_as_float(v[j]), f);
+            for (int j = 0; j < 16; ++j) eq::add_scaled(Sh[j], Sl[j], __uint_as_float(v[j]), f);
             if (cpw > 16) {
 #pragma unroll
-                for (int j = 16; j < 32; ++j) level_add(Sh[j], Sl[j], __uint_as_float(v[j]), f);
+                for (int j = 16; j < 32; ++j) eq::add_scaled(Sh[j], Sl[j], __uint_as_float(v[j]), f);
             }
         }
     }
     if (active) {
-        float2 *out = reinterpret_cast<float2 *>(pp.so + (warp - 2) * kLvOut);
-        const int col = lane & 7;
-#pragma unroll
-        for (int c = 0; c < 32; c += 8) {
-            if (c >= ncols) continue;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) out[lane * 8 + (j ^ (lane & 7))] = make_float2(Sh[c + j], Sl[c + j]);
-            __syncwarp();
-            const int sb = __shfl_sync(0xffffffffu, eb, c + col);
-            const bool col_ok = c + col < ncols;
-            double *dst = P.C + (long long)(row0 + (lane >> 3)) * P.ldc + c0 + c + col;
-#pragma unroll 1
-            for (int r = lane >> 3; r < 32; r += 4, dst += 4 * P.ldc) {
-                const float2 v = out[r * 8 + (col ^ (r & 7))];
-                const int sa = __shfl_sync(0xffffffffu, ea, r);
-                if (col_ok && r < nrows) *dst = level_value(v.x, v.y, sa + sb);
-            }
-            __syncwarp();
-        }
+        const int ebs[1] = {eb};
+        eq::store_columns(Sh, Sl, pp.so + (warp - 2) * eq::kOutBytes, P.C, P.ldc, row0, c0, nrows, ncols, ea, ebs);
     }
     return true;
 }
@@ -710,7 +630,7 @@ __device__ __forceinline__ void eq_levels_body(const LvMaps &maps, unsigned *err
                                               ~static_cast<uintptr_t>(1023));
     pp.sb = pp.sa + kLvSlots * kTileA;
     pp.so = pp.sb + 2 * kLvB;
-    pp.afull = reinterpret_cast<uint64_t *>(pp.so + kEpiWarps * kLvOut);
+    pp.afull = reinterpret_cast<uint64_t *>(pp.so + kEpiWarps * eq::kOutBytes);
     pp.aempty = pp.afull + kLvSlots;
     pp.bempty = pp.aempty + kLvSlots;
     pp.lfull = pp.bempty + 2;
@@ -969,7 +889,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_tiles_kernel(const __gri
     if (threadIdx.x == 0 && *pp.abort_flag) r.ctl->fault = 1u;  // a wait ran out: the host stops serving
 }
 
-size_t smem_bytes() { return 1024 + (size_t)kStages * kStageBytes + 256; }
+size_t smem_bytes() { return 1024 + (size_t)kStages * kStageBytes + kEpiWarps * eq::kOutBytes + 256; }
 
 // ------------------------------------------------------------ scheme tables
 // Pair scheme: products (p, q), p + q <= L, paired by p over consecutive q,

@@ -24,7 +24,8 @@
 // most ~2.3e-13 of sum_l |a_il| |b_lj| when the entries of a row (column)
 // are of comparable size.
 //
-//   K-block kb = min(roundup64(k), 1024);  beta = 8 (kb <= 256) or 7;
+//   K-block kb: the fewest blocks of at most 1024 terms, multiples of 64,
+//   all about as long;  beta = 8 (kb <= 256) or 7;
 //   beta 8: L = 7 (21 products); beta 7: L = 8 (28 products).
 //
 // Kernel: persistent, one CTA per SM over 128 x 128 output tiles.  The
@@ -39,8 +40,7 @@
 // (two per tensor-memory lane quarter, one per 64-column half) add each
 // finished accumulator, scaled by 2^(-beta (p + q)), into a float-float
 // running sum held in registers; after the tile's last unit they write
-// FP64 C.  Sharing A_p raises the MMA work per staged byte by a third,
-// which is what bounds this kernel (operand latency, not tensor rate).
+// FP64 C.  Sharing A_p raises the MMA work per staged byte by a third.
 // Every mbarrier wait is bounded.
 // A row of A or column of B holding a NaN or an infinity gives NaN in every
 // entry of C it meets (tc.cuh, kNonFiniteExp); other entries are unaffected.
@@ -117,15 +117,6 @@ __device__ __forceinline__ void eq_tile(const EqArgs &a, int t, int &m0, int &n0
     m0 = (g * kGroupM + r % rows) * kBM;
     n0 = (r / rows) * kBN;
 }
-
-#define OO_TMEM_LD16(taddr, r)                                                                              \
-    asm volatile(                                                                                           \
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "  \
-        "[%16];"                                                                                            \
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),   \
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),          \
-          "=r"(r[15])                                                                                       \
-        : "r"(taddr))
 
 __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_constant__ EqMaps maps,
                                                                  const __grid_constant__ EqArgs a) {
@@ -247,6 +238,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
         for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
             int m0, n0;
             eq_tile(a, t, m0, n0);
+#pragma unroll
+            for (int j = 0; j < 64; ++j) Sh[j] = Sl[j] = 0.0f;
             for (int u = 0; u < units; ++u, ++gu) {
                 const int b = gu & 1;
                 if (!bar_wait(su32(&tfull[b]), (gu >> 1) & 1, abort_flag, a.err, 4u)) {
@@ -255,7 +248,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
                 }
                 fence_after();
                 const int pr = u % a.nunits;
-                const bool pair = a.uq2[pr] != kNone, first = u == 0;
+                const bool pair = a.uq2[pr] != kNone;
                 const float f1 = a.us1[pr], f2 = a.us2[pr];
                 const uint32_t acc = tmem + (uint32_t)(b * 2 * kBN) + lane_off + (uint32_t)(h * 64);
 #pragma unroll
@@ -266,16 +259,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
                         if (half == 1 && !pair) break;
                         OO_TMEM_LD16(acc + half * kBN + c, v);
                         tmem_wait_ld();
-                        const float f = half ? f2 : f1;
+                        const float f = half ? f2 : f1;  // a power of two: exact scale
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
-                            const float w = __fmul_rn(__uint_as_float(v[j]), f);  // exact: power-of-two scale
-                            if (first && half == 0) {
-                                Sh[c + j] = w;
-                                Sl[c + j] = 0.0f;
-                            } else {
-                                ff::add(Sh[c + j], Sl[c + j], w, 0.0f, Sh[c + j], Sl[c + j]);
-                            }
+                            eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), f);
+                            eq::renormalise(Sh[c + j], Sl[c + j]);
                         }
                     }
                 }
@@ -296,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
                     for (int j = 0; j < 64; ++j) {
                         const int sb = __shfl_sync(0xffffffffu, j < 32 ? e0 : e1, j & 31);
                         if (row_ok && c0 + j < a.n)
-                            crow[j] = nan_or_scaled(ff::to_double(Sh[j], Sl[j]), sa + sb);
+                            crow[j] = eq::scaled_value(Sh[j], Sl[j], sa + sb);
                     }
                 }
             }
@@ -336,6 +324,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
 // running each loop, the issuer's own instructions took 611 clocks a K step,
 // and 1050 while the epilogue ran, for 512 clocks of MMA; n = 4096 took 2.92
 // ms in this kernel, 2.29 ms so (3.13 -> 2.56 ms with the splits).
+// The epilogue: C is stored through shared memory (eq::store_columns) and a
+// running sum costs 10 operations a product, the power-of-two scale folded
+// into them.  With a row of C per lane and the conversion unrolled over the
+// columns the store took 122,000 clocks a tile, in which the tensor cores did
+// two units of the next tile and then waited: n = 4096 2.50 -> 2.18 ms, n =
+// 2048 444 -> 356 us, 1024 118 -> 105 us with the splits.  A unit's epilogue takes
+// about as long as a K-block of 1024 terms' MMAs, so K-blocks are balanced
+// (eq::shape): 1000 x 777 x 1300 in blocks of 1024 + 320 159 us, 704 + 640
+// 144 us with both.  What binds now at n = 4096 is the tensor rate, 0.93 of
+// 1.9 PFLOP/s over the products' 3.85 PFLOP, under the power limit.
 constexpr int kStagesPair = 6;
 constexpr uint32_t kStageBytesPair = 2 * kTile;  // A_p and this CTA's B tile
 constexpr uint32_t kIdescPair2 = idesc_bf16(2 * kBM, 2 * kBN);
@@ -359,7 +357,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
     extern __shared__ __align__(1024) unsigned char esm_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(esm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + kStagesPair * kStageBytesPair);
+    unsigned char *out = sm + kStagesPair * kStageBytesPair;  // the epilogue warps' store staging
+    uint64_t *bars = reinterpret_cast<uint64_t *>(out + kEpiWarps * eq::kOutBytes);
     uint64_t *full = bars, *empty = bars + kStagesPair;
     uint64_t *tfull = bars + 2 * kStagesPair, *tempty = tfull + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tempty + 2);
@@ -490,6 +489,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
             int m0, n0;
             eq_tile_pair(a, t, m0, n0);
             m0 += (int)rank * kBM;
+#pragma unroll
+            for (int j = 0; j < 64; ++j) Sh[j] = Sl[j] = 0.0f;
             for (int u = 0; u < units; ++u, ++gu) {
                 const int b = gu & 1;
                 if (!bar_wait_cluster(su32(&tfull[b]), (gu >> 1) & 1, abort_flag, a.err, 4u)) {
@@ -498,27 +499,22 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
                 }
                 fence_after();
                 const int pr = u % a.nunits;
-                const bool pair = a.uq2[pr] != kNone, first = u == 0;
+                const bool pair = a.uq2[pr] != kNone;
                 const float f1 = a.us1[pr], f2 = a.us2[pr];
                 const uint32_t acc = tmem + (uint32_t)(b * 2 * kBN) + lane_off + (uint32_t)(h * 64);
 #pragma unroll
-                for (int c = 0; c < 64; c += 16) {
-                    uint32_t v[16];
+                for (int c = 0; c < 64; c += 8) {
+                    uint32_t v[8], w[8];
+                    OO_TMEM_LD8(acc + c, v);
+                    if (pair) OO_TMEM_LD8(acc + kBN + c, w);
+                    tmem_wait_ld();
 #pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        if (half == 1 && !pair) break;
-                        OO_TMEM_LD16(acc + half * kBN + c, v);
-                        tmem_wait_ld();
-                        const float f = half ? f2 : f1;
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const float w = __fmul_rn(__uint_as_float(v[j]), f);  // exact: power-of-two scale
-                            if (first && half == 0) {
-                                Sh[c + j] = w;
-                                Sl[c + j] = 0.0f;
-                            } else {
-                                ff::add(Sh[c + j], Sl[c + j], w, 0.0f, Sh[c + j], Sl[c + j]);
-                            }
+                    for (int j = 0; j < 8; ++j) {  // f1, f2: powers of two, exact scales
+                        eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), f1);
+                        eq::renormalise(Sh[c + j], Sl[c + j]);
+                        if (pair) {
+                            eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(w[j]), f2);
+                            eq::renormalise(Sh[c + j], Sl[c + j]);
                         }
                     }
                 }
@@ -530,21 +526,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
                     else
                         bar_arrive_remote(map_to_rank(su32(&tempty[b]), 0));
                 }
-                if (u == units - 1) {
-                    const int row = m0 + q * 32 + lane;
-                    const int c0 = n0 + h * 64;
-                    const int e0 = c0 + lane < a.n ? a.eb[c0 + lane] : 0;
-                    const int e1 = c0 + 32 + lane < a.n ? a.eb[c0 + 32 + lane] : 0;
-                    const bool row_ok = row < a.m;
-                    const int sa = row_ok ? a.ea[row] : 0;
-                    double *crow = a.C + (long long)row * a.ldc + c0;
-#pragma unroll
-                    for (int j = 0; j < 64; ++j) {
-                        const int sb = __shfl_sync(0xffffffffu, j < 32 ? e0 : e1, j & 31);
-                        if (row_ok && c0 + j < a.n)
-                            crow[j] = nan_or_scaled(ff::to_double(Sh[j], Sl[j]), sa + sb);
-                    }
-                }
+            }
+            const int row0 = m0 + q * 32, c0 = n0 + h * 64, ncols = min(64, a.n - c0);
+            if (ok && row0 < a.m && ncols > 0) {
+                // scales: lane l holds row row0 + l's and columns c0 + l's and c0 + 32 + l's
+                const int ea = row0 + lane < a.m ? a.ea[row0 + lane] : 0;
+                const int eb[2] = {lane < ncols ? a.eb[c0 + lane] : 0, 32 + lane < ncols ? a.eb[c0 + 32 + lane] : 0};
+                eq::store_columns(Sh, Sl, out + (warp - 2) * eq::kOutBytes, a.C, a.ldc, row0, c0,
+                                  min(32, a.m - row0), ncols, ea, eb);
             }
         }
     }
@@ -700,7 +689,7 @@ __global__ void eq_split_cols_t_kernel(const double *B, long long ldb, int k, in
 }
 
 size_t smem_eq() { return 1024 + (size_t)kStages * kStageBytes + 256; }
-constexpr size_t kSmemEqPair = 1024 + (size_t)kStagesPair * kStageBytesPair + 256;
+constexpr size_t kSmemEqPair = 1024 + (size_t)kStagesPair * kStageBytesPair + kEpiWarps * eq::kOutBytes + 256;
 static_assert(kSmemEqPair <= 232448, "pair kernel exceeds the shared memory of a CTA");
 
 // 2-CTA clusters of the pair kernel that fit on the device at once (cached)
