@@ -34,6 +34,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <vector>
 
 #include "ff.cuh"
 #include "tc.cuh"
@@ -129,6 +130,30 @@ __device__ __forceinline__ unsigned digit_bits(unsigned long long X, unsigned ne
 __device__ __forceinline__ unsigned digit_pair(unsigned long long X0, unsigned n0, unsigned long long X1, unsigned n1,
                                                int beta, int p) {
     return digit_bits(X0, n0, beta, p) | (digit_bits(X1, n1, beta, p) << 16);
+}
+
+// A unit of the pair scheme: slice p of A against slices q .. q + nq - 1 of B
+// (0-based), accumulated side by side
+struct PairUnit {
+    int p, q, nq;
+};
+// Products (p, q), 1-based, p + q <= L, in groups of up to four consecutive q
+// of one p, from the smallest contributions up; most = 2 cuts each group into
+// its upper and its lower half.  A unit's products are added from the highest
+// q down, so that both cuts add all products in one order and a tile has the
+// same bits whichever kernel forms it.
+inline std::vector<PairUnit> pair_units(const Shape &e, int most) {
+    std::vector<PairUnit> four, u;
+    for (int p = 0; p < e.slices; ++p)
+        for (int q = 0; q < e.levels - 1 - p; q += 4) four.push_back({p, q, std::min(4, e.levels - 1 - p - q)});
+    std::stable_sort(four.begin(), four.end(),
+                     [](const PairUnit &a, const PairUnit &b) { return a.p + a.q > b.p + b.q; });
+    if (most == 4) return four;
+    for (const PairUnit &x : four) {
+        if (x.nq > 2) u.push_back({x.p, x.q + 2, x.nq - 2});
+        u.push_back({x.p, x.q, std::min(2, x.nq)});
+    }
+    return u;
 }
 
 // (Sh, Sl) += d f, f a power of two, without renormalising (7 operations; a

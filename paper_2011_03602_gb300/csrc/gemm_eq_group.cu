@@ -288,26 +288,29 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
         if (!bar_wait(su32(&pp.tfull[b]), (gu >> 1) & 1, pp.abort_flag, a.err, 4u)) return false;
         fence_after();
         const int u = uu % S.nunits;
-        const float fL = S.usL[u], fR = S.usR[u];
+        // powers of two, exact scales; the pair scheme adds the right half first (eq::pair_units)
+        const bool swap = !levels && S.usR[u] != 0.0f;
+        const float f1 = swap ? S.usR[u] : S.usL[u], f2 = swap ? S.usL[u] : S.usR[u];
         if (active) {
             const uint32_t acc = pp.tmem + (uint32_t)(b * 256) + lane_off + (uint32_t)cw0;
+            const uint32_t acc1 = acc + (swap ? td.w : 0), acc2 = acc + (swap ? 0 : td.w);
 #pragma unroll
             for (int c = 0; c < 64; c += 16) {
                 if (c < ncols) {
                     uint32_t v[16];
-                    OO_TMEM_LD16(acc + c, v);
+                    OO_TMEM_LD16(acc1 + c, v);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {  // fL, fR: powers of two, exact scales
-                        eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), fL);
+                    for (int j = 0; j < 16; ++j) {
+                        eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), f1);
                         if (!levels) eq::renormalise(Sh[c + j], Sl[c + j]);
                     }
-                    if (fR != 0.0f) {
-                        OO_TMEM_LD16(acc + (uint32_t)td.w + c, v);
+                    if (f2 != 0.0f) {
+                        OO_TMEM_LD16(acc2 + c, v);
                         tmem_wait_ld();
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
-                            eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), fR);
+                            eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), f2);
                             if (!levels) eq::renormalise(Sh[c + j], Sl[c + j]);
                         }
                     }
@@ -893,7 +896,7 @@ size_t smem_bytes() { return 1024 + (size_t)kStages * kStageBytes + kEpiWarps * 
 
 // ------------------------------------------------------------ scheme tables
 // Pair scheme: products (p, q), p + q <= L, paired by p over consecutive q,
-// smallest contributions first (the single-problem kernel's order).  Level
+// in the single-problem kernels' order (eq::pair_units).  Level
 // schemes: unit = levels (s, s + 1), s = 2, 4, ..., terms A_p x [B_{s-p} |
 // B_{s+1-p}] for p = 1 .. s (halves past level L or with q < 1 not fed),
 // smallest levels first.  Slices 0-based in the table.
@@ -903,16 +906,10 @@ SchemeTab make_tab(int scheme, int k) {
     std::vector<std::vector<std::array<int, 3>>> units;
     std::vector<std::array<int, 2>> lv;  // 1-based levels of each unit's halves (0: none)
     if (scheme == eq::kSchemePairs) {
-        struct U {
-            int p, q1, q2;
-        };
-        std::vector<U> u;
-        for (int p = 1; p <= e.slices; ++p)
-            for (int q = 1; q <= e.levels - p; q += 2) u.push_back({p, q, q + 1 <= e.levels - p ? q + 1 : 0});
-        std::stable_sort(u.begin(), u.end(), [](const U &x, const U &y) { return x.p + x.q1 > y.p + y.q1; });
-        for (const U &x : u) {
-            units.push_back({{x.p - 1, x.q1 - 1, x.q2 ? x.q2 - 1 : (int)kNone}});
-            lv.push_back({x.p + x.q1, x.q2 ? x.p + x.q2 : 0});
+        for (const eq::PairUnit &x : eq::pair_units(e, 2)) {
+            const bool two = x.nq == 2;
+            units.push_back({{x.p, x.q, two ? x.q + 1 : (int)kNone}});
+            lv.push_back({x.p + x.q + 2, two ? x.p + x.q + 3 : 0});
         }
     } else {
         std::vector<std::vector<std::array<int, 3>>> us;

@@ -72,28 +72,10 @@ constexpr int kGroupM = 8;
 constexpr int kMaxUnits = 24;
 constexpr uint32_t kIdescPair = idesc_bf16(kBM, 2 * kBN);
 constexpr uint32_t kIdescOne = idesc_bf16(kBM, kBN);
-constexpr unsigned char kNone = 0xff;
 
 using EqShape = eq::Shape;
-// the pair scheme this file's kernel runs
-EqShape eq_shape(int k) { return eq::shape(eq::kSchemePairs, k); }
 // the scheme the library uses for inner dimension k
 EqShape eq_used_shape(int k) { return eq::shape(eq_scheme_for(k), k); }
-
-// A unit: slice p of A against slices q1 and q2 (q2 = kNone: alone) of B
-struct EqUnit {
-    int p, q1, q2;
-};
-// Products (p, q), 1-based, p + q <= L, grouped by p in pairs of
-// consecutive q; ordered from the smallest contributions up.
-std::vector<EqUnit> eq_units(const EqShape &e) {
-    std::vector<EqUnit> u;
-    for (int p = 1; p <= e.slices; ++p)
-        for (int q = 1; q <= e.levels - p; q += 2)
-            u.push_back({p - 1, q - 1, q + 1 <= e.levels - p ? q : (int)kNone});
-    std::stable_sort(u.begin(), u.end(), [](const EqUnit &a, const EqUnit &b) { return a.p + a.q1 > b.p + b.q1; });
-    return u;
-}
 
 struct EqMaps {
     CUtensorMap a, b;  // all slices stacked: slice p at rows [p m, (p + 1) m)
@@ -106,8 +88,9 @@ struct EqArgs {
     long long ldc;
     const int *ea, *eb;
     unsigned *err;
-    unsigned char up[kMaxUnits], uq1[kMaxUnits], uq2[kMaxUnits];  // 0-based slices; uq2 kNone: alone
-    float us1[kMaxUnits], us2[kMaxUnits];                           // 2^(-beta (p + q)), 1-based p, q
+    unsigned char up[kMaxUnits], uq[kMaxUnits], unq[kMaxUnits];  // 0-based slices p, q .. q + nq - 1
+    float us[kMaxUnits];                                         // 2^(-beta (p + q)), 1-based p and first q
+    float uq_step;                                               // 2^-beta
 };
 
 __device__ __forceinline__ void eq_tile(const EqArgs &a, int t, int &m0, int &n0) {
@@ -165,9 +148,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
             eq_tile(a, t, m0, n0);
             for (int u = 0; ok && u < units; ++u) {
                 const int kbi = u / a.nunits, pr = u % a.nunits;  // K-block outer: its slices stay in L2
-                const bool pair = a.uq2[pr] != kNone;
-                const int rowA = a.up[pr] * a.m + m0, rowB1 = a.uq1[pr] * a.n + n0;
-                const int rowB2 = pair ? a.uq2[pr] * a.n + n0 : 0;
+                const bool pair = a.unq[pr] == 2;
+                const int rowA = a.up[pr] * a.m + m0, rowB1 = a.uq[pr] * a.n + n0;
+                const int rowB2 = pair ? rowB1 + a.n : 0;
                 const int ks1 = min(a.ksteps, (kbi + 1) * a.kb_steps);
                 for (int ks = kbi * a.kb_steps; ks < ks1; ++ks, ++it) {
                     const int s = it % kStages;
@@ -201,7 +184,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
                 fence_after();
                 const uint32_t d = tmem + (uint32_t)(b * 2 * kBN);
                 const int kbi = u / a.nunits, pr = u % a.nunits;  // K-block outer: its slices stay in L2
-                const bool pair = a.uq2[pr] != kNone;
+                const bool pair = a.unq[pr] == 2;
                 const int ks0 = kbi * a.kb_steps, ks1 = min(a.ksteps, (kbi + 1) * a.kb_steps);
                 for (int ks = ks0; ks < ks1; ++ks, ++it) {
                     const int s = it % kStages;
@@ -248,15 +231,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
                 }
                 fence_after();
                 const int pr = u % a.nunits;
-                const bool pair = a.uq2[pr] != kNone;
-                const float f1 = a.us1[pr], f2 = a.us2[pr];
+                const bool pair = a.unq[pr] == 2;
+                const float f1 = a.us[pr], f2 = f1 * a.uq_step;
                 const uint32_t acc = tmem + (uint32_t)(b * 2 * kBN) + lane_off + (uint32_t)(h * 64);
 #pragma unroll
                 for (int c = 0; c < 64; c += 16) {
                     uint32_t v[16];
 #pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        if (half == 1 && !pair) break;
+                    for (int half = 1; half >= 0; --half) {  // the smaller contribution first
+                        if (half == 1 && !pair) continue;
                         OO_TMEM_LD16(acc + half * kBN + c, v);
                         tmem_wait_ld();
                         const float f = half ? f2 : f1;  // a power of two: exact scale
@@ -309,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
 
 // ------------------------------------------------------------ CTA pairs
 // The same products on CTA pairs (cta_group::2, M = 256): a tile is 256 rows
-// x 128 columns, CTA r of the pair holding rows m0 + 128 r .. +127 of the
+// x TN = 128 columns, CTA r of the pair holding rows m0 + 128 r .. +127 of the
 // tile and its own accumulators and running sums.  A two-product unit
 // (p, q1) + (p, q2) is one M = 256, N = 256 MMA whose B operand is B_q1's
 // tile in rank 0's shared memory and B_q2's in rank 1's, so an SM stages
@@ -332,26 +315,42 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
 // 2048 444 -> 356 us, 1024 118 -> 105 us with the splits.  A unit's epilogue takes
 // about as long as a K-block of 1024 terms' MMAs, so K-blocks are balanced
 // (eq::shape): 1000 x 777 x 1300 in blocks of 1024 + 320 159 us, 704 + 640
-// 144 us with both.  What binds now at n = 4096 is the tensor rate, 0.93 of
+// 144 us with both (wide tiles).  What binds now at n = 4096 is the tensor rate, 0.93 of
 // 1.9 PFLOP/s over the products' 3.85 PFLOP, under the power limit.
+// Narrow tiles, TN = 64: a unit is up to four slices of B against one of A,
+// beside each other in the same 256 accumulator columns, so that A_p's 16 KB
+// still come with up to 16 KB of B for 512 clocks of MMA a K step, and half
+// the columns need half the time: 1000 x 777 x 1300 is 28 wide tiles on 76
+// CTA pairs, 144 us with the splits, and 52 narrow ones, 92 us; 1024^3 105 ->
+// 72 us.  (64-column tiles of two-product units would stage 24 KB for 256
+// clocks of MMA, more than the 65 bytes a clock that one SM gets from L2.)
 constexpr int kStagesPair = 6;
 constexpr uint32_t kStageBytesPair = 2 * kTile;  // A_p and this CTA's B tile
-constexpr uint32_t kIdescPair2 = idesc_bf16(2 * kBM, 2 * kBN);
-constexpr uint32_t kIdescOne2 = idesc_bf16(2 * kBM, kBN);
 
 struct EqPairMaps {
-    CUtensorMap a, b, bh;  // bh: B slices in 64-row boxes (one-product units)
+    CUtensorMap a, b, bh;  // B slices in boxes of a tile's columns and of half as many
 };
 
+// running sums += eight accumulator columns, scaled by f
+__device__ __forceinline__ void add8(float *Sh, float *Sl, const uint32_t (&d)[8], float f) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        eq::add_scaled(Sh[j], Sl[j], __uint_as_float(d[j]), f);
+        eq::renormalise(Sh[j], Sl[j]);
+    }
+}
+
+template <int TN>
 __device__ __forceinline__ void eq_tile_pair(const EqArgs &a, int t, int &m0, int &n0) {
     const int per_group = (kGroupM / 2) * a.n_tiles;
     const int g = t / per_group, r = t % per_group;
     const int rows = min(kGroupM / 2, a.m_tiles - g * (kGroupM / 2));
     m0 = (g * (kGroupM / 2) + r % rows) * 2 * kBM;
-    n0 = (r / rows) * kBN;
+    n0 = (r / rows) * TN;
 }
 
 // a.m_tiles counts 256-row slabs here
+template <int TN>
 __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __grid_constant__ EqPairMaps maps,
                                                                       const __grid_constant__ EqArgs a) {
     extern __shared__ __align__(1024) unsigned char esm_raw[];
@@ -404,15 +403,20 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
         bool ok = true;
         for (int t = cid; ok && t < tiles; t += ncl) {
             int m0, n0;
-            eq_tile_pair(a, t, m0, n0);
+            eq_tile_pair<TN>(a, t, m0, n0);
             for (int kbi = 0; ok && kbi < a.nkb; ++kbi)  // K-block outer: its slices stay in L2
                 for (int pr = 0; ok && pr < a.nunits; ++pr) {
-                    const bool pair = a.uq2[pr] != kNone;
                     const int rowA = a.up[pr] * a.m + m0 + (int)rank * kBM;
-                    const int rowB = pair ? (rank ? a.uq2[pr] : a.uq1[pr]) * a.n + n0
-                                          : a.uq1[pr] * a.n + n0 + (int)rank * (kBN / 2);
-                    const uint32_t tx = pair ? 2 * 2 * kTile : 2 * (kTile + kTile / 2);
-                    const CUtensorMap *mb = pair ? &maps.b : &maps.bh;
+                    // this CTA's B rows: half tiles c .. c + nq - 1 of the unit's 2 nq, in one
+                    // or two boxes (nq = 3: a whole tile and half of the middle one)
+                    const int nq = a.unq[pr], c = (int)rank * nq;
+                    const int rowB = (a.uq[pr] + (c >> 1)) * a.n + n0 + (c & 1) * (TN / 2);
+                    const bool half1 = nq == 1 || (c & 1) != 0;
+                    const CUtensorMap *mb = half1 ? &maps.bh : &maps.b;
+                    const int rowB2 = (a.uq[pr] + (c >> 1) + 1) * a.n + n0;  // nq > 2
+                    const CUtensorMap *mb2 = nq == 3 && !half1 ? &maps.bh : &maps.b;
+                    const uint32_t off2 = kTile + (half1 ? TN / 2 : TN) * kBK * 2;
+                    const uint32_t tx = 2 * kTile + nq * TN * kBK * 2;
                     const int ks1 = min(a.ksteps, (kbi + 1) * a.kb_steps);
                     for (int ks = kbi * a.kb_steps; ks < ks1; ++ks) {
                         if (loaded >= kStagesPair && !warp_wait<true>(empty0 + s * 8, phase, abort_flag, a.err, 1u)) {
@@ -423,6 +427,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
                         if (leader) bar_expect_tx_if(el, full_here + s * 8, tx);
                         tma_2d_pair_if(el, st, &maps.a, ks * kBK, rowA, fb);
                         tma_2d_pair_if(el, st + kTile, mb, ks * kBK, rowB, fb);
+                        if (TN < kBN && nq > 2) tma_2d_pair_if(el, st + off2, mb2, ks * kBK, rowB2, fb);
                         ++loaded;
                         if (++s == kStagesPair) {
                             s = 0;
@@ -450,7 +455,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
                     }
                     fence_after();
                     const uint32_t d = tmem + (uint32_t)(b * 2 * kBN);
-                    const uint32_t idesc = a.uq2[pr] != kNone ? kIdescPair2 : kIdescOne2;
+                    const uint32_t idesc = idesc_bf16(2 * kBM, a.unq[pr] * TN);
                     const int steps = min(a.ksteps, (kbi + 1) * a.kb_steps) - kbi * a.kb_steps;
                     uint32_t acc = 0;
                     for (int ks = 0; ks < steps; ++ks) {
@@ -482,15 +487,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
         const int q = warp & 3;
         const int h = (warp - 2) >> 2;
         const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-        float Sh[64], Sl[64];
+        constexpr int NC = TN / 2;  // columns of a warp
+        float Sh[NC], Sl[NC];
         int gu = 0;
         bool ok = true;
         for (int t = cid; ok && t < tiles; t += ncl) {
             int m0, n0;
-            eq_tile_pair(a, t, m0, n0);
+            eq_tile_pair<TN>(a, t, m0, n0);
             m0 += (int)rank * kBM;
 #pragma unroll
-            for (int j = 0; j < 64; ++j) Sh[j] = Sl[j] = 0.0f;
+            for (int j = 0; j < NC; ++j) Sh[j] = Sl[j] = 0.0f;
             for (int u = 0; u < units; ++u, ++gu) {
                 const int b = gu & 1;
                 if (!bar_wait_cluster(su32(&tfull[b]), (gu >> 1) & 1, abort_flag, a.err, 4u)) {
@@ -499,24 +505,22 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
                 }
                 fence_after();
                 const int pr = u % a.nunits;
-                const bool pair = a.uq2[pr] != kNone;
-                const float f1 = a.us1[pr], f2 = a.us2[pr];
-                const uint32_t acc = tmem + (uint32_t)(b * 2 * kBN) + lane_off + (uint32_t)(h * 64);
+                const int nq = a.unq[pr];
+                const float f1 = a.us[pr], f2 = f1 * a.uq_step;  // powers of two: exact scales
+                const float f3 = f2 * a.uq_step, f4 = f3 * a.uq_step;
+                const uint32_t acc = tmem + (uint32_t)(b * 2 * kBN) + lane_off + (uint32_t)(h * NC);
 #pragma unroll
-                for (int c = 0; c < 64; c += 8) {
-                    uint32_t v[8], w[8];
+                for (int c = 0; c < NC; c += 8) {
+                    uint32_t v[8], w[8], x[8], y[8];
                     OO_TMEM_LD8(acc + c, v);
-                    if (pair) OO_TMEM_LD8(acc + kBN + c, w);
+                    if (nq > 1) OO_TMEM_LD8(acc + TN + c, w);
+                    if (TN < kBN && nq > 2) OO_TMEM_LD8(acc + 2 * TN + c, x);
+                    if (TN < kBN && nq > 3) OO_TMEM_LD8(acc + 3 * TN + c, y);
                     tmem_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {  // f1, f2: powers of two, exact scales
-                        eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), f1);
-                        eq::renormalise(Sh[c + j], Sl[c + j]);
-                        if (pair) {
-                            eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(w[j]), f2);
-                            eq::renormalise(Sh[c + j], Sl[c + j]);
-                        }
-                    }
+                    if (TN < kBN && nq > 3) add8(Sh + c, Sl + c, y, f4);  // smallest first
+                    if (TN < kBN && nq > 2) add8(Sh + c, Sl + c, x, f3);
+                    if (nq > 1) add8(Sh + c, Sl + c, w, f2);
+                    add8(Sh + c, Sl + c, v, f1);
                 }
                 fence_before();
                 __syncwarp();
@@ -527,11 +531,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
                         bar_arrive_remote(map_to_rank(su32(&tempty[b]), 0));
                 }
             }
-            const int row0 = m0 + q * 32, c0 = n0 + h * 64, ncols = min(64, a.n - c0);
+            const int row0 = m0 + q * 32, c0 = n0 + h * NC, ncols = min(NC, a.n - c0);
             if (ok && row0 < a.m && ncols > 0) {
-                // scales: lane l holds row row0 + l's and columns c0 + l's and c0 + 32 + l's
+                // scales: lane l holds row row0 + l's and columns c0 + l's (and c0 + 32 + l's)
                 const int ea = row0 + lane < a.m ? a.ea[row0 + lane] : 0;
-                const int eb[2] = {lane < ncols ? a.eb[c0 + lane] : 0, 32 + lane < ncols ? a.eb[c0 + 32 + lane] : 0};
+                int eb[NC / 32];
+#pragma unroll
+                for (int i = 0; i < NC / 32; ++i) eb[i] = 32 * i + lane < ncols ? a.eb[c0 + 32 * i + lane] : 0;
                 eq::store_columns(Sh, Sl, out + (warp - 2) * eq::kOutBytes, a.C, a.ldc, row0, c0,
                                   min(32, a.m - row0), ncols, ea, eb);
             }
@@ -693,6 +699,7 @@ constexpr size_t kSmemEqPair = 1024 + (size_t)kStagesPair * kStageBytesPair + kE
 static_assert(kSmemEqPair <= 232448, "pair kernel exceeds the shared memory of a CTA");
 
 // 2-CTA clusters of the pair kernel that fit on the device at once (cached)
+template <int TN>
 int eq_pair_clusters() {
     int dev = 0;
     OO_CUDA_TRY(cudaGetDevice(&dev));
@@ -700,7 +707,7 @@ int eq_pair_clusters() {
     int ncl = dev < 64 ? max_clusters[dev].load() : 0;
     if (ncl > 0) return ncl;
     static std::atomic<uint64_t> attr{0};
-    set_smem_limit_once((const void *)gemm_fp64eq_pair_kernel, kSmemEqPair, attr);
+    set_smem_limit_once((const void *)gemm_fp64eq_pair_kernel<TN>, kSmemEqPair, attr);
     int sms = 148;
     OO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     cudaLaunchAttribute at[1];
@@ -714,7 +721,7 @@ int eq_pair_clusters() {
     cfg.dynamicSmemBytes = kSmemEqPair;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    OO_CUDA_TRY(cudaOccupancyMaxActiveClusters(&ncl, (const void *)gemm_fp64eq_pair_kernel, &cfg));
+    OO_CUDA_TRY(cudaOccupancyMaxActiveClusters(&ncl, (const void *)gemm_fp64eq_pair_kernel<TN>, &cfg));
     OO_REQUIRE(ncl >= 1, OO_ECUDA, "no 2-CTA cluster of the FP64-equivalent kernel fits on this device");
     if (dev < 64) max_clusters[dev].store(ncl);
     return ncl;
@@ -924,6 +931,41 @@ __global__ void __launch_bounds__(256) eq_group_split_cols_kernel(const eq::GSpl
     const int4 jb = jobs[blockIdx.x];
     eq::split_cols_job(gs[jb.y], jb.z, t, red);
 }
+void set_units(EqArgs &a, const EqShape &e, int most) {
+    const std::vector<eq::PairUnit> U = eq::pair_units(e, most);
+    OO_REQUIRE((int)U.size() <= kMaxUnits, OO_EINVAL, "too many product groups");
+    a.nunits = (int)U.size();
+    a.uq_step = std::ldexp(1.0f, -e.beta);
+    for (size_t i = 0; i < U.size(); ++i) {
+        a.up[i] = (unsigned char)U[i].p;
+        a.uq[i] = (unsigned char)U[i].q;
+        a.unq[i] = (unsigned char)U[i].nq;
+        a.us[i] = std::ldexp(1.0f, -e.beta * (U[i].p + U[i].q + 2));
+    }
+}
+
+template <int TN>
+void launch_pair(EqArgs &a, const EqShape &e, __nv_bfloat16 *As, __nv_bfloat16 *Bs, int kp, int clusters,
+                 cudaStream_t s) {
+    set_units(a, e, 2 * kBN / TN);
+    EqPairMaps pm;
+    map_bf16(&pm.a, As, (long long)e.slices * a.m, kp, kBM);
+    map_bf16(&pm.b, Bs, (long long)e.slices * a.n, kp, TN);
+    map_bf16(&pm.bh, Bs, (long long)e.slices * a.n, kp, TN / 2);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(2 * clusters));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemEqPair;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    OO_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_fp64eq_pair_kernel<TN>, (const EqPairMaps)pm, (const EqArgs)a));
+}
 }  // namespace
 
 void eq_group_split_jobs(int scheme, int problem, int m, int n, std::vector<int4> (&jobs)[6]) {
@@ -1010,9 +1052,6 @@ void launch_gemm_fp64eq(int m, int n, int k, const double *A, long long lda, con
         eq_split_cols_t_kernel<<<grid, 256, 0, s>>>(B, ldb, k, n, kp, e.beta, e.slices, mxo, eb, Bs);
         OO_CUDA_TRY(cudaGetLastError());
     }
-    EqMaps maps;
-    map_bf16(&maps.a, As, (long long)e.slices * m, kp, kBM);
-    map_bf16(&maps.b, Bs, (long long)e.slices * n, kp, kBN);
     EqArgs ga{};
     ga.m = m;
     ga.n = n;
@@ -1026,40 +1065,30 @@ void launch_gemm_fp64eq(int m, int n, int k, const double *A, long long lda, con
     ga.ea = ea;
     ga.eb = eb;
     ga.err = err;
-    const std::vector<EqUnit> U = eq_units(e);
-    OO_REQUIRE((int)U.size() <= kMaxUnits, OO_EINVAL, "too many product groups");
-    ga.nunits = (int)U.size();
-    for (size_t i = 0; i < U.size(); ++i) {
-        ga.up[i] = (unsigned char)U[i].p;
-        ga.uq1[i] = (unsigned char)U[i].q1;
-        ga.uq2[i] = (unsigned char)U[i].q2;
-        ga.us1[i] = std::ldexp(1.0f, -e.beta * (U[i].p + U[i].q1 + 2));
-        ga.us2[i] = U[i].q2 == kNone ? 0.0f : std::ldexp(1.0f, -e.beta * (U[i].p + U[i].q2 + 2));
-    }
     if (pair) {
-        EqPairMaps pm;
-        map_bf16(&pm.a, As, (long long)e.slices * m, kp, kBM);
-        map_bf16(&pm.b, Bs, (long long)e.slices * n, kp, kBN);
-        map_bf16(&pm.bh, Bs, (long long)e.slices * n, kp, kBN / 2);
-        ga.m_tiles = (m + 2 * kBM - 1) / (2 * kBM);  // 256-row slabs
-        const long long ptiles = (long long)ga.m_tiles * ga.n_tiles;
-        OO_REQUIRE(ptiles < (1ll << 31), OO_EINVAL, "too many tiles");
-        const int ncl = eq_pair_clusters();
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)(2 * std::min<long long>(ptiles, ncl)));
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = kSmemEqPair;
-        cfg.stream = s;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        OO_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_fp64eq_pair_kernel, (const EqPairMaps)pm, (const EqArgs)ga));
+        const int slabs = (m + 2 * kBM - 1) / (2 * kBM), n128 = (n + kBN - 1) / kBN, n64 = (n + 63) / 64;
+        ga.m_tiles = slabs;
+        const long long t128 = (long long)slabs * n128, t64 = (long long)slabs * n64;
+        OO_REQUIRE(t64 < (1ll << 31), OO_EINVAL, "too many tiles");
+        const int ncl = std::min(eq_pair_clusters<128>(), eq_pair_clusters<64>());
+        // A narrow tile costs 0.57 of a wide one (a K step of all products 4,314 against
+        // 7,656 clocks by staged bytes and MMA rate): narrow where that makes the waves
+        // shorter.  1000 x 777 x 1300: 52 of 76 pairs for 28, 92 us for 144; 300 x 4000 x
+        // 1000 would take two waves for one, and 2048^3 four for two, 2.28 times a wave.
+        const long long w128 = (t128 + ncl - 1) / ncl, w64 = (t64 + ncl - 1) / ncl;
+        if (57 * w64 < 100 * w128) {
+            ga.n_tiles = n64;
+            launch_pair<64>(ga, e, As, Bs, kp, (int)std::min<long long>(t64, ncl), s);
+        } else {
+            ga.n_tiles = n128;
+            launch_pair<128>(ga, e, As, Bs, kp, (int)std::min<long long>(t128, ncl), s);
+        }
         return;
     }
+    EqMaps maps;
+    map_bf16(&maps.a, As, (long long)e.slices * m, kp, kBM);
+    map_bf16(&maps.b, Bs, (long long)e.slices * n, kp, kBN);
+    set_units(ga, e, 2);
     static std::atomic<uint64_t> attr{0};
     set_smem_limit_once((const void *)gemm_fp64eq_kernel, smem_eq(), attr);
     const long long tiles = (long long)ga.m_tiles * ga.n_tiles;

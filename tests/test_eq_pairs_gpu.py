@@ -14,7 +14,8 @@ import torch
 pytestmark = pytest.mark.gpu
 
 SHAPES = [(1, 1, 513), (7, 9, 577), (127, 129, 1024), (129, 127, 1025), (256, 8, 1088), (257, 255, 1300),
-          (300, 33, 2048), (64, 300, 2049), (513, 261, 2113)]
+          (300, 33, 2048), (64, 300, 2049), (513, 261, 2113),
+          (2001, 1101, 577)]  # the last in wide tiles (one wave of CTA pairs), the others in narrow ones
 
 
 @pytest.mark.parametrize("ea,eb", [(0, 0), (-600, -455), (500, 480)])
