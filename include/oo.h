@@ -323,8 +323,8 @@ oo_status oo_inject_wait_timeout(oo_ctx *ctx, int what);
  *   OO_OPT_GEMM_PAIR        1 (default) the split-BF16 products of
  *                           oo_gemm_f64 / oo_gemm_f64_dev run on CTA pairs
  *                           (256-row tiles, each SM of a pair loading half
- *                           of the tile's B columns), the tile width (160,
- *                           192, 224 or 256 columns) chosen per problem;
+ *                           of the tile's B columns), the tile width (64 to
+ *                           256 columns, in steps of 32) chosen per problem;
  *                           160, 192, 224 or 256: CTA pairs with that tile
  *                           width; 0: single CTAs (128 x 128 tiles).  All
  *                           form the same products in the same order, so

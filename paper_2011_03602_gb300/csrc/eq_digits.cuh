@@ -172,30 +172,34 @@ __device__ __forceinline__ void renormalise(float &Sh, float &Sl) { ff::fast_two
 
 // (h + l) 2^S as a double, rounded once: the high part's bits and the low
 // part as an integer in units of the double's last place (ff::to_double's case
-// analysis took twice the instructions).  Zero, results near the ends of the
-// range and the flag scales of non-finite rows and columns take the general
-// conversion.
-__device__ __forceinline__ double scaled_value(float h, float l, int S) {
+// analysis took twice the instructions).  Returns whether that holds: zero,
+// results near the ends of the range and the flag scales of non-finite rows
+// and columns take general_value.
+__device__ __forceinline__ bool scaled_value(float h, float l, int S, double &v) {
     float s, e;
     ff::two_sum(h, l, s, e);
     const unsigned b = __float_as_uint(s), m = b & 0x7fffffu;
     const int es = (int)((b >> 23) & 0xffu), ed = es - 127 + 1023 + S;
-    if ((unsigned)(es - 64) > 126u || (unsigned)(ed - 2) > 2043u) return tc::nan_or_scaled(ff::to_double(h, l), S);
     // the last place is half as large below a power of two
     const int below = m == 0 && (int)(__float_as_uint(e) ^ b) < 0;
     int t = __float2int_rn(__fmul_rn(e, __uint_as_float((unsigned)(306 + below - es) << 23)));  // |t| <= 2^28
     if (b >> 31) t = -t;
-    const unsigned long long v = ((unsigned long long)(unsigned)ed << 52) + ((unsigned long long)m << 29) +
+    const unsigned long long x = ((unsigned long long)(unsigned)ed << 52) + ((unsigned long long)m << 29) +
                                  (unsigned long long)(long long)t;
-    return __longlong_as_double((long long)(v | ((unsigned long long)(b >> 31) << 63)));
+    v = __longlong_as_double((long long)(x | ((unsigned long long)(b >> 31) << 63)));
+    return (unsigned)(es - 64) <= 126u && (unsigned)(ed - 2) <= 2043u;
+}
+__device__ __forceinline__ double general_value(float h, float l, int S) {
+    return tc::nan_or_scaled(ff::to_double(h, l), S);
 }
 
 // An epilogue warp's sums -- lane l holds row row0 + l, columns c0 + j -- to C
 // through `out`, 32 rows x 8 columns of float pairs of the warp's own shared
 // memory (kOutBytes), so that 8-byte stores go out as 64-byte row segments and
-// the conversion is a loop, not unrolled over the columns.  With a row per
-// lane and the unrolled conversion a 256 x 128 tile of the pair scheme took
-// 122,000 clocks here, most of them instruction fetches and store replays.
+// the conversion is a loop, not unrolled over the columns, of four independent
+// values at a time.  With a row per lane and the unrolled conversion a 256 x
+// 128 tile of the pair scheme took 122,000 clocks here, most of them
+// instruction fetches and store replays.
 // ea: row l's scale; eb: columns l and 32 + l's; nrows, ncols: those that exist.
 constexpr uint32_t kOutBytes = 32 * 8 * 8;
 template <int NC>
@@ -214,10 +218,31 @@ __device__ __forceinline__ void store_columns(const float (&Sh)[NC], const float
         const bool col_ok = c + col < ncols;
         double *dst = C + (long long)(row0 + (lane >> 3)) * ldc + c0 + c + col;
 #pragma unroll 1
-        for (int r = lane >> 3; r < 32; r += 4, dst += 4 * ldc) {
-            const float2 v = out[r * 8 + (col ^ (r & 7))];
-            const int sa = __shfl_sync(0xffffffffu, ea, r);
-            if (col_ok && r < nrows) *dst = scaled_value(v.x, v.y, sa + sb);
+        for (int r = lane >> 3; r < 32; r += 16, dst += 16 * ldc) {
+            float2 w[4];
+            int S[4];
+            double v[4];
+            bool fast = true;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                w[i] = out[(r + 4 * i) * 8 + (col ^ ((r + 4 * i) & 7))];
+                S[i] = __shfl_sync(0xffffffffu, ea, r + 4 * i) + sb;
+                fast &= scaled_value(w[i].x, w[i].y, S[i], v[i]) || !col_ok || r + 4 * i >= nrows;
+            }
+            if (fast) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (col_ok && r + 4 * i < nrows) dst[4 * i * ldc] = v[i];
+            } else {
+#pragma unroll 1
+                for (int i = 0; i < 4; ++i) {
+                    const float2 x = out[(r + 4 * i) * 8 + (col ^ ((r + 4 * i) & 7))];
+                    const int Si = i == 0 ? S[0] : i == 1 ? S[1] : i == 2 ? S[2] : S[3];
+                    double y;
+                    if (!scaled_value(x.x, x.y, Si, y)) y = general_value(x.x, x.y, Si);
+                    if (col_ok && r + 4 * i < nrows) dst[4 * i * ldc] = y;
+                }
+            }
         }
         __syncwarp();
     }

@@ -38,6 +38,7 @@
 
 #include "ff.cuh"
 #include "oo_internal.h"
+#include "eq_digits.cuh"
 #include "tc.cuh"
 
 namespace oo {
@@ -47,7 +48,7 @@ namespace {
 constexpr int kBM = 128, kBN = 128, kBK = 64, kStages = 3;
 constexpr int kGemmThreads = 384;  // producer, MMA issuer, 2 idle, 8 epilogue warps
 constexpr int kEpiWarps = 8;
-constexpr uint32_t kStageOut = kEpiWarps * 32 * 16 * 8;  // per epilogue warp: 32 rows x 16 FP64 staging
+constexpr uint32_t kStageOut = kEpiWarps * 32 * 16 * 8;  // per epilogue warp: 32 rows x 16 columns of two floats
 constexpr uint32_t kTileA = kBM * kBK * 2;   // 16 KB
 constexpr uint32_t kTileB = kBN * kBK * 2;   // 16 KB
 constexpr uint32_t kStageBytes = 2 * kTileA + 2 * kTileB;  // 64 KB
@@ -66,7 +67,7 @@ struct GemmArgs {
     int m, n, k, kp;        // kp: padded K of the split operands (a multiple of kstage)
     int kstage;             // K values per pipeline stage: 64 (BF16) or 32 (TF32)
     int m_tiles, n_tiles;
-    int nw;                 // pair kernel: tile width (columns; a multiple of 32, 160 .. 256)
+    int nw;                 // pair kernel: tile width (columns; a multiple of 32, 64 .. 256)
     double *C;
     long long ldc;
     const int *ea;          // per-row scale exponents of A (power of two)
@@ -140,74 +141,100 @@ struct GroupSrc {
     }
 };
 
-// f * 2^S as a double by integer operations (exact; the FP64 pipe only for
-// zeros, subnormals and results outside the normal range); NaN where the
-// row's and column's scales flag a non-finite input (see nan_or_scaled)
-__device__ __forceinline__ double nan_or_widened(float f, int S) {
-    if (S > 4096) return __longlong_as_double(0x7ff8000000000000ll);
+// f * 2^S as a double by integer operations, exact; returns whether that
+// holds: zeros, subnormals, results outside the normal range and the flag
+// scales of non-finite rows and columns take widened_general
+__device__ __forceinline__ bool widened(float f, int S, double &v) {
     const unsigned b = __float_as_uint(f);
-    const int e = (int)((b >> 23) & 0xffu);
-    const int ne = e - 127 + 1023 + S;
-    if (e == 0 || e == 0xff || ne <= 0 || ne >= 0x7ff) return ldexp((double)f, S);
-    return __longlong_as_double((long long)(((unsigned long long)(b & 0x80000000u) << 32) |
-                                            ((unsigned long long)ne << 52) |
-                                            ((unsigned long long)(b & 0x7fffffu) << 29)));
+    const int e = (int)((b >> 23) & 0xffu), ne = e - 127 + 1023 + S;
+    v = __longlong_as_double((long long)(((unsigned long long)(b & 0x80000000u) << 32) |
+                                         ((unsigned long long)(unsigned)ne << 52) |
+                                         ((unsigned long long)(b & 0x7fffffu) << 29)));
+    return (unsigned)(e - 1) < 254u && (unsigned)(ne - 1) < 0x7feu;
+}
+__device__ __forceinline__ double widened_general(float f, int S) {
+    return S > 4096 ? __longlong_as_double(0x7ff8000000000000ll) : ldexp((double)f, S);
 }
 
 // Epilogue of one tile for one warp: TMEM lane quarter q holds rows
-// m0 + 32 q .. +31 of the tile; the warp takes tile columns hcol .. cend - 1
-// (cend - hcol a multiple of 16 or cut by the problem's last column), in at
-// most NCH 32-column chunks.  MERGED: one FP32 accumulator at d (the
+// m0 + 32 q .. +31 of the tile; the warp takes tile columns hcol .. cend - 1,
+// at most 32 NCH, in blocks of 16.  MERGED: one FP32 accumulator at d (the
 // split-BF16 products); else D_hh at d and D_x at d + 128, summed exactly
-// (the split-TF32 pair).  Each thread widens its row's values; 16-column
-// blocks go through a per-warp shared-memory transpose (XOR-swizzled: no
-// bank conflicts) so every global store writes two whole 128-byte row
-// segments.  sa: the row's scale exponent; e[c]: that of column
-// hcol + 32 c + lane.
+// (the split-TF32 pair).  A block goes through the warp's shared memory as it
+// was accumulated (XOR-swizzled: no bank conflicts) and is widened on the way
+// out, in a loop over rows whose every store writes two whole 128-byte row
+// segments.  (Widened on the way in, unrolled over the columns, the general
+// case was there 32 times, and a tile's store spent most of its time fetching
+// instructions; one value after another cost 6,400 clocks a block of 16
+// columns, each a chain of a shuffle, a load and branches.)  sa: the row's scale exponent; e[c]: that of
+// column hcol + 32 c + lane.
 template <int NCH, bool MERGED>
 __device__ __forceinline__ void store_tile_quarter(const TileJob &jb, uint32_t d, int q, int hcol, int cend, int lane,
-                                                   double *stg, int sa, const int (&e)[NCH]) {
-    const int n0 = jb.n0, row0 = jb.m0 + q * 32;
-    const int ncols = cend;  // columns of the tile this warp stores end here
-    const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+                                                   unsigned char *stg, int sa, const int (&e)[NCH]) {
+    const int row0 = jb.m0 + q * 32, nrows = min(32, jb.m - row0), cl = lane & 15;
+    const uint32_t acc = d + ((uint32_t)(q * 32) << 16);
+    float *s1 = reinterpret_cast<float *>(stg);
+    float2 *s2 = reinterpret_cast<float2 *>(stg);
 #pragma unroll 1
-    for (int cc = 0; cc < NCH; ++cc) {
-        const int c = hcol + cc * 32;
-        if (c >= ncols) break;
-        uint32_t h[32], x[32];
-        OO_TMEM_LD32(d + lane_off + c, h);
-        if constexpr (!MERGED) OO_TMEM_LD32(d + 128 + lane_off + c, x);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    for (int c = hcol, i = 0; c < cend; c += 16, ++i) {
+        uint32_t h[16], x[16];
+        OO_TMEM_LD16(acc + c, h);
+        if constexpr (!MERGED) OO_TMEM_LD16(acc + 128 + c, x);
+        tmem_wait_ld();
         int ecur = e[0];
 #pragma unroll
-        for (int i = 1; i < NCH; ++i)
-            if (cc == i) ecur = e[i];
+        for (int n = 1; n < NCH; ++n)
+            if (i >> 1 == n) ecur = e[n];
+        const int sb = __shfl_sync(0xffffffffu, ecur, (i & 1) * 16 + cl);
 #pragma unroll
-        for (int sub = 0; sub < 2; ++sub) {
-            if (c + sub * 16 >= ncols) break;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int t2 = sub * 16 + j;
-                const int sb = __shfl_sync(0xffffffffu, ecur, t2);
-                double v;
-                if constexpr (MERGED) {
-                    v = nan_or_widened(__uint_as_float(h[t2]), sa + sb);
-                } else {
-                    // exact two-sum of the partial products, widened and
-                    // scaled without the (slow) FP64 pipe
-                    v = nan_or_scaled(ff::to_double(__uint_as_float(h[t2]), __uint_as_float(x[t2])), sa + sb);
-                }
-                stg[lane * 16 + (j ^ (lane & 15))] = v;
-            }
-            __syncwarp();
-            const int cl = lane & 15, col = c + sub * 16 + cl;
-#pragma unroll 4
-            for (int r = lane >> 4; r < 32; r += 2) {
-                const double v = stg[r * 16 + (cl ^ (r & 15))];
-                if (row0 + r < jb.m && col < ncols) jb.C[(long long)(row0 + r) * jb.ldc + n0 + col] = v;
-            }
-            __syncwarp();
+        for (int j = 0; j < 16; ++j) {
+            if constexpr (MERGED)
+                s1[lane * 16 + (j ^ (lane >> 1))] = __uint_as_float(h[j]);
+            else
+                s2[lane * 16 + (j ^ (lane & 15))] = make_float2(__uint_as_float(h[j]), __uint_as_float(x[j]));
         }
+        __syncwarp();
+        const bool col_ok = c + cl < cend;
+        double *dst = jb.C + (long long)(row0 + (lane >> 4)) * jb.ldc + jb.n0 + c + cl;
+#pragma unroll 1
+        for (int r0 = lane >> 4; r0 < 32; r0 += 16, dst += 16 * jb.ldc) {  // eight independent values at a time
+            double v[8];
+            int S[8];
+            bool fast = true;
+#pragma unroll
+            for (int n = 0; n < 8; ++n) {
+                const int r = r0 + 2 * n;
+                S[n] = __shfl_sync(0xffffffffu, sa, r) + sb;
+                bool ok;
+                if constexpr (MERGED) {
+                    ok = widened(s1[r * 16 + (cl ^ (r >> 1))], S[n], v[n]);
+                } else {
+                    const float2 w = s2[r * 16 + (cl ^ (r & 15))];
+                    ok = eq::scaled_value(w.x, w.y, S[n], v[n]);
+                }
+                fast &= ok || !col_ok || r >= nrows;
+            }
+            if (fast) {
+#pragma unroll
+                for (int n = 0; n < 8; ++n)
+                    if (col_ok && r0 + 2 * n < nrows) dst[2 * n * jb.ldc] = v[n];
+            } else {
+#pragma unroll
+                for (int n = 0; n < 8; ++n) {
+                    const int r = r0 + 2 * n;
+                    if (!col_ok || r >= nrows) continue;
+                    if constexpr (MERGED) {
+                        const float f = s1[r * 16 + (cl ^ (r >> 1))];
+                        dst[2 * n * jb.ldc] = widened(f, S[n], v[n]) ? v[n] : widened_general(f, S[n]);
+                    } else {
+                        const float2 w = s2[r * 16 + (cl ^ (r & 15))];
+                        dst[2 * n * jb.ldc] =
+                            eq::scaled_value(w.x, w.y, S[n], v[n]) ? v[n] : eq::general_value(w.x, w.y, S[n]);
+                    }
+                }
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -219,7 +246,7 @@ __device__ __forceinline__ void gemm_body(const Src &src, unsigned *err) {
     extern __shared__ __align__(1024) unsigned char gsm_raw[];
     unsigned char *gsm = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(gsm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    double *stg_all = reinterpret_cast<double *>(gsm + kStages * kStageBytes);  // epilogue store staging
+    unsigned char *stg_all = gsm + kStages * kStageBytes;  // epilogue store staging
     uint64_t *bars = reinterpret_cast<uint64_t *>(gsm + kStages * kStageBytes + kStageOut);
     uint64_t *full = bars, *empty = bars + kStages;
     uint64_t *tfull = bars + 2 * kStages, *tempty = bars + 2 * kStages + 2;
@@ -344,7 +371,7 @@ __device__ __forceinline__ void gemm_body(const Src &src, unsigned *err) {
         // 32 (w & 3) .. +31 of the tile, and column half (w - 4) >> 2;
         // quarters with no valid row are skipped.
         const int q = warp & 3, hcol = ((warp - 4) >> 2) * 64;
-        double *stg = stg_all + (size_t)(warp - 4) * 32 * 16;
+        unsigned char *stg = stg_all + (warp - 4) * (kStageOut / kEpiWarps);
         int lt = 0;
         for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++lt) {
             const int b = lt & 1;
@@ -412,17 +439,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_group_kernel(const __gri
 
 // ------------------------------------------------- CTA-pair split3 kernel
 // The split-BF16 product on CTA pairs (cta_group::2).  A unit is a 256 x W
-// tile of C (W = a.nw, 160 .. 256 columns, chosen per problem so that the
+// tile of C (W = a.nw, 64 .. 256 columns, chosen per problem so that the
 // units fill the resident clusters' waves: n = 4096 takes W = 224, 304
 // units = 4 waves of 76 pairs, where W = 256 leaves the fourth wave a
-// third full); CTA r of the pair loads rows m0 + 128 r .. +127 of A1 and
+// third full, and small products narrow tiles, which occupy more SMs); CTA r of the pair loads rows m0 + 128 r .. +127 of A1 and
 // A2 and rows n0 + r W/2 .. +W/2-1 of B1 and B2 (its half of the tile's
 // columns).  Rank 0 issues M = 256, N = W MMAs into both CTAs' TMEM (each
 // holds its 128 rows x W columns, double-buffered); the commits arrive on
 // both CTAs' barriers; each CTA's epilogue stores its own rows and reports
-// to rank 0 that its accumulator buffer is free.  Wide N matters: measured
-// on GB300, N = 128 instructions (either tile shape) kept the tensor pipe
-// ~64 % busy at most, N = 256 ones ~97 %.  Every output element sees the
+// to rank 0 that its accumulator buffer is free.  Producer and MMA issuer run
+// as whole warps and the store widens eight independent values at a time: n =
+// 4096 317 -> 292 us with the split, 1000 x 776 x 1300 68 -> 37 us at W = 160
+// and 31 us at W = 64, which the issuer's own instructions ruled out before.
+// Every output element sees the
 // same products in the same K order as in gemm_split3_kernel, so the two
 // kernels give the same bits.
 constexpr int kStagesP = 3;
@@ -447,7 +476,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_split3_pair_kernel(const
     extern __shared__ __align__(1024) unsigned char gsm_raw[];
     unsigned char *gsm = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(gsm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    double *stg_all = reinterpret_cast<double *>(gsm + kStagesP * kStageBytesP);
+    unsigned char *stg_all = gsm + kStagesP * kStageBytesP;
     uint64_t *bars = reinterpret_cast<uint64_t *>(gsm + kStagesP * kStageBytesP + kStageOut);
     uint64_t *full = bars, *empty = bars + kStagesP;
     uint64_t *tfull = bars + 2 * kStagesP, *tempty = tfull + 2;
@@ -455,7 +484,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_split3_pair_kernel(const
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     unsigned *err = a.err;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const bool leader = rank == 0;
     const int cid = (int)(blockIdx.x >> 1), ncl = (int)(gridDim.x >> 1);
@@ -484,77 +513,86 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_split3_pair_kernel(const
     __syncthreads();
     cluster_sync_all();  // both CTAs' barriers and TMEM exist before either uses the other's
     fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     int loaded = 0, tiles_mma = 0;
-    if (warp == 0 && lane == 0) {
-        // ---------------------------------------------------- TMA producer (both CTAs)
-        int it = 0;
+    if (warp == 0) {
+        // ---------------------------------------------------- TMA producer (both CTAs, whole warp)
+        const uint32_t el = elect_one();
+        const uint32_t sm0 = su32(gsm), empty0 = su32(empty);
+        const uint32_t full_here = su32(full), full0 = map_to_rank(full_here, 0);
+        int s = 0;
+        uint32_t phase = 1;  // the ring's first use needs no wait
         bool ok = true;
         for (int u = cid; ok && u < units; u += ncl) {
             int mp, n0;
             pair_coords(a, u, mp, n0);
             const int ma = mp + (int)rank * kBM, nb = n0 + (int)rank * half;
-            for (int ks = 0; ks < ksteps; ++ks, ++it) {
-                const int s = it % kStagesP;
-                const uint32_t use = it / kStagesP;
-                if (use > 0 && !bar_wait_cluster(su32(&empty[s]), (use - 1) & 1, abort_flag, err, 1u)) {
+            for (int ks = 0; ks < ksteps; ++ks) {
+                if (loaded >= kStagesP && !warp_wait<true>(empty0 + s * 8, phase, abort_flag, err, 1u)) {
                     ok = false;
                     break;
                 }
-                unsigned char *st = gsm + (size_t)s * kStageBytesP;
-                if (leader) bar_expect_tx(su32(&full[s]), stage_tx);
-                const uint32_t fb = map_to_rank(su32(&full[s]), 0);
+                const uint32_t st = sm0 + s * kStageBytesP, fb = full0 + s * 8;
                 const int k0 = ks * kBK;
-                tma_2d_pair(su32(st), &maps.a1, k0, ma, fb);
-                tma_2d_pair(su32(st + kTileA), &maps.a2, k0, ma, fb);
-                tma_2d_pair(su32(st + 2 * kTileA), &maps.b1, k0, nb, fb);
-                tma_2d_pair(su32(st + 2 * kTileA + kTileB), &maps.b2, k0, nb, fb);
+                if (leader) bar_expect_tx_if(el, full_here + s * 8, stage_tx);
+                tma_2d_pair_if(el, st, &maps.a1, k0, ma, fb);
+                tma_2d_pair_if(el, st + 2 * kTileA, &maps.b1, k0, nb, fb);
+                tma_2d_pair_if(el, st + 2 * kTileA + kTileB, &maps.b2, k0, nb, fb);
+                tma_2d_pair_if(el, st + kTileA, &maps.a2, k0, ma, fb);
                 ++loaded;
+                if (++s == kStagesP) {
+                    s = 0;
+                    phase ^= 1;
+                }
             }
         }
-    } else if (warp == 1 && lane == 0 && leader) {
-        // ---------------------------------------------------- MMA issuer (rank 0)
+    } else if (warp == 1 && leader) {
+        // ---------------------------------------------------- MMA issuer (rank 0, whole warp)
+        const uint32_t el = elect_one();
         const uint32_t idesc = idesc_bf16(2 * kBM, a.nw);
-        int it = 0, lt = 0;
+        const uint64_t da0 = sdesc_sw128(su32(gsm)), db0 = sdesc_sw128(su32(gsm) + 2 * kTileA);
+        const uint32_t full0 = su32(full), empty0 = su32(empty), tfull0 = su32(tfull), tempty0 = su32(tempty);
+        int s = 0, lt = 0;
+        uint32_t phase = 0;
         bool ok = true;
         for (int u = cid; ok && u < units; u += ncl, ++lt) {
             const int b = lt & 1;
             const uint32_t buse = lt >> 1;
-            if (buse > 0 && !bar_wait_cluster(su32(&tempty[b]), (buse - 1) & 1, abort_flag, err, 2u)) break;
+            if (buse > 0 && !warp_wait<true>(tempty0 + b * 8, (buse - 1) & 1, abort_flag, err, 2u)) break;
             fence_after();
             const uint32_t d = tmem + (uint32_t)(b * 256);
-            for (int ks = 0; ks < ksteps; ++ks, ++it) {
-                const int s = it % kStagesP;
-                const uint32_t use = it / kStagesP;
-                if (!bar_wait_cluster(su32(&full[s]), use & 1, abort_flag, err, 2u)) {
+            uint32_t acc = 0;
+            for (int ks = 0; ks < ksteps; ++ks) {
+                if (!warp_wait<true>(full0 + s * 8, phase, abort_flag, err, 2u)) {
                     ok = false;
                     break;
                 }
                 fence_after();
-                const uint32_t base = su32(gsm + (size_t)s * kStageBytesP);
-                const uint32_t a1 = base, a2 = base + kTileA, b1 = base + 2 * kTileA, b2 = b1 + kTileB;
+                const uint64_t a1 = da0 + (uint64_t)(s * (int)(kStageBytesP >> 4)), a2 = a1 + (kTileA >> 4);
+                const uint64_t b1 = db0 + (uint64_t)(s * (int)(kStageBytesP >> 4)), b2 = b1 + (kTileB >> 4);
 #pragma unroll
-                for (int kk = 0; kk < kBK / 16; ++kk) {
-                    const uint32_t off = kk * 32;
-                    const uint32_t acc = (ks == 0 && kk == 0) ? 0u : 1u;
-                    mma_bf16_pair(d, sdesc_sw128(a1 + off), sdesc_sw128(b1 + off), idesc, acc);
-                    mma_bf16_pair(d, sdesc_sw128(a1 + off), sdesc_sw128(b2 + off), idesc, 1u);
-                    mma_bf16_pair(d, sdesc_sw128(a2 + off), sdesc_sw128(b1 + off), idesc, 1u);
+                for (int kk = 0; kk < kBK / 16; ++kk) {  // 32 bytes of each row per MMA
+                    mma_bf16_pair_if(el, d, a1 + kk * 2, b1 + kk * 2, idesc, acc);
+                    acc = 1;
+                    mma_bf16_pair_if(el, d, a1 + kk * 2, b2 + kk * 2, idesc, 1u);
+                    mma_bf16_pair_if(el, d, a2 + kk * 2, b1 + kk * 2, idesc, 1u);
                 }
-                mma_commit_pair(su32(&empty[s]), 3);  // stage s free in both CTAs
+                mma_commit_pair_if(el, empty0 + s * 8, 3);  // stage s free in both CTAs
+                if (++s == kStagesP) {
+                    s = 0;
+                    phase ^= 1;
+                }
             }
             if (!ok) break;
-            mma_commit_pair(su32(&tfull[b]), 3);  // both halves of the accumulator complete
+            mma_commit_pair_if(el, tfull0 + b * 8, 3);  // both halves of the accumulator complete
             ++tiles_mma;
         }
     } else if (warp >= 4) {
         // ---------------------------------------------------- epilogue (both CTAs)
-        // warp-halves take tile columns [0, 128) and [128, W): chunk starts
-        // stay multiples of 32
-        const int q = warp & 3, hsel = (warp - 4) >> 2, hcol = hsel * 128;
-        const int hend = hsel ? a.nw : min(128, a.nw);
-        double *stg = stg_all + (size_t)(warp - 4) * 32 * 16;
+        // a warp of each lane quarter takes half of the tile's columns (a multiple of 16)
+        const int q = warp & 3, hcol = ((warp - 4) >> 2) * half, hend = hcol + half;
+        unsigned char *stg = stg_all + (warp - 4) * (kStageOut / kEpiWarps);
         int lt = 0;
         for (int u = cid; u < units; u += ncl, ++lt) {
             const int b = lt & 1;
@@ -1151,17 +1189,20 @@ int pair_clusters() {
     return ncl;
 }
 
-// Tile width of the pair kernel for an m x n product: the width among 256,
-// 224, 192 and 160 columns with the fewest column-waves (waves of units over
-// the resident clusters x width), the widest on a tie.  Narrower MMAs lose
-// tensor throughput (N = 128 ran at ~64 %), so 160 is the floor.
-int pair_tile_width(int m, int n, int ncl) {
+// Tile width of the pair kernel for an m x n x k product: the least of waves x
+// K steps x (56 + w) + 15 w over w = 64, 96 .. 256 columns, the widest on a tie.
+// A K step of a tile w wide took 0.40, 0.55, 0.72, 0.95 us at w = 64, 128, 192,
+// 256 in full waves (the fixed part: operand loads and instruction issue), the
+// last wave's store about as long as 15 K steps' share of a column.  1000 x 776
+// x 1300: w = 64 30.8 us, 160 36.8; 2048^3: 128 73.8, 256 76.1; 4096^3: 224
+// 291.9, 256 318.5, 128 319.2.
+int pair_tile_width(int m, int n, int kp, int ncl) {
     const long long slabs = (m + 2 * kBM - 1) / (2 * kBM);
     int best = kBNP;
     long long best_cost = -1;
-    for (int w = kBNP; w >= 160; w -= 32) {
+    for (int w = kBNP; w >= 64; w -= 32) {
         const long long units = slabs * ((n + w - 1) / w);
-        const long long cost = (units + ncl - 1) / ncl * w;
+        const long long cost = (units + ncl - 1) / ncl * (kp / kBK) * (56 + w) + 15 * w;
         if (best_cost < 0 || cost < best_cost) {
             best = w;
             best_cost = cost;
@@ -1256,8 +1297,9 @@ void launch_gemm_split3(int m, int n, int k, const double *A, long long lda, con
     int ncl = 0, nw = kBN;
     if (pair) {
         ncl = pair_clusters();
-        nw = pair == 1 ? pair_tile_width(m, n, ncl) : pair;
-        OO_REQUIRE(nw >= 160 && nw <= kBNP && nw % 32 == 0, OO_EINVAL, "pair tile width must be 160, 192, 224 or 256");
+        nw = pair == 1 ? pair_tile_width(m, n, kp, ncl) : pair;
+        OO_REQUIRE(pair == 1 || (nw >= 160 && nw <= kBNP && nw % 32 == 0), OO_EINVAL,
+                   "pair tile width must be 160, 192, 224 or 256");
     }
     // B tiles: half of a pair tile's columns per CTA, else 128 columns
     map_bf16(&maps.b1, B1, n, kp, pair ? nw / 2 : kBN);

@@ -267,7 +267,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
                     for (int j = 0; j < 64; ++j) {
                         const int sb = __shfl_sync(0xffffffffu, j < 32 ? e0 : e1, j & 31);
                         if (row_ok && c0 + j < a.n)
-                            crow[j] = eq::scaled_value(Sh[j], Sl[j], sa + sb);
+                        {
+                            double v;
+                            if (!eq::scaled_value(Sh[j], Sl[j], sa + sb, v)) v = eq::general_value(Sh[j], Sl[j], sa + sb);
+                            crow[j] = v;
+                        }
                     }
                 }
             }
