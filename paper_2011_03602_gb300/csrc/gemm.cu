@@ -156,6 +156,9 @@ __device__ __forceinline__ double widened_general(float f, int S) {
     return S > 4096 ? __longlong_as_double(0x7ff8000000000000ll) : ldexp((double)f, S);
 }
 
+// largest biased exponent of a row or column -> its scale exponent
+__device__ __forceinline__ int max_to_scale(int mx) { return mx == 0 ? 0 : mx - 1023 + 1; }
+
 // Epilogue of one tile for one warp: TMEM lane quarter q holds rows
 // m0 + 32 q .. +31 of the tile; the warp takes tile columns hcol .. cend - 1,
 // at most 32 NCH, in blocks of 16.  MERGED: one FP32 accumulator at d (the
@@ -381,8 +384,12 @@ __device__ __forceinline__ void gemm_body(const Src &src, unsigned *err) {
             const int n0 = jb.n0, row0 = jb.m0 + q * 32;
             const int ncols = jb.n - n0;  // valid columns of the tile (may exceed 128)
             const int sa = row0 + lane < jb.m ? jb.ea[row0 + lane] : 0;
-            const int e[2] = {hcol + lane < ncols ? jb.eb[n0 + hcol + lane] : 0,
-                              hcol + 32 + lane < ncols ? jb.eb[n0 + hcol + 32 + lane] : 0};
+            int e[2] = {hcol + lane < ncols ? jb.eb[n0 + hcol + lane] : 0,
+                        hcol + 32 + lane < ncols ? jb.eb[n0 + hcol + 32 + lane] : 0};
+            if constexpr (TF32) {  // column maxima
+                e[0] = max_to_scale(e[0]);
+                e[1] = max_to_scale(e[1]);
+            }
             if (!bar_wait(su32(&tfull[b]), (lt >> 1) & 1, abort_flag, err, 4u)) break;
             fence_after();
             if (row0 < jb.m)
@@ -658,27 +665,6 @@ __device__ __forceinline__ int bf16_col_scale(int mx) {
     if (u >= -20 && u < 40) return 0;
     return mx - 1023 + 1;
 }
-// per-column maxima of B (k x n): grid.x over column blocks of 32, grid.y over k chunks
-__global__ void col_maxexp_kernel(const double *B, long long ldb, int k, int n, int rows_per, int *e) {
-    const int col = blockIdx.x * 32 + threadIdx.x;
-    const int r0 = blockIdx.y * rows_per, r1 = min(k, r0 + rows_per);
-    if (col >= n) return;
-    int mx = 0;
-#pragma unroll 8
-    for (int l = r0 + threadIdx.y; l < r1; l += blockDim.y) {
-        mx = max(mx, biased_exp_or_flag((unsigned long long)__double_as_longlong(B[(long long)l * ldb + col])));
-    }
-    if (mx > 0) atomicMax(e + col, mx);
-}
-__global__ void exp_to_scale_kernel(int *e, int count) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) e[i] = e[i] == 0 ? 0 : e[i] - 1023 + 1;
-}
-// the same for the columns of B in the split-BF16 pattern (bf16_col_scale)
-__global__ void exp_to_bf16_col_scale_kernel(int *e, int count) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) e[i] = bf16_col_scale(e[i]);
-}
 
 // x * 2^-S -> (hi, lo) BF16 pair with hi + lo = x * 2^-S to ~16 bits
 __device__ __forceinline__ void split_bf16(double x, int S, __nv_bfloat16 &hi, __nv_bfloat16 &lo) {
@@ -730,60 +716,6 @@ __device__ __forceinline__ void split_row_warp(const double *src, int k, int kp,
     }
 }
 
-// A (m x k, lda) -> per-row scale ea and A1, A2 (m x kp); one warp per row
-__global__ void split_rows_fused_kernel(const double *A, long long lda, int m, int k, int kp, int *ea,
-                                        __nv_bfloat16 *A1, __nv_bfloat16 *A2) {
-    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (row >= m) return;
-    split_row_warp(A + (long long)row * lda, k, kp, ea + row, A1 + (long long)row * kp, A2 + (long long)row * kp);
-}
-
-// Same, one 256-thread CTA per row with 16-byte loads (lda even, A 16-byte
-// aligned): the second read of the row hits L1 and each thread keeps eight
-// loads in flight in the exponent pass.
-__global__ void __launch_bounds__(256) split_rows_v2_kernel(const double *A, long long lda, int m, int k, int kp,
-                                                          int *ea, __nv_bfloat16 *A1, __nv_bfloat16 *A2) {
-    const int row = blockIdx.x;
-    const double *base = A + (long long)row * lda;
-    const double2 *src = reinterpret_cast<const double2 *>(base);
-    const int k2 = k >> 1;
-    int mx = 0;
-    auto ex = [](double x) { return biased_exp_or_flag((unsigned long long)__double_as_longlong(x)); };
-#pragma unroll 8
-    for (int l2 = threadIdx.x; l2 < k2; l2 += 256) {
-        const double2 v = src[l2];
-        mx = max(mx, max(ex(v.x), ex(v.y)));
-    }
-    if ((k & 1) && threadIdx.x == 0) mx = max(mx, ex(base[k - 1]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    __shared__ int red[8];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    mx = red[0];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) mx = max(mx, red[w]);
-    const int S = mx == 0 ? 0 : mx - 1023 + 1;
-    if (threadIdx.x == 0) ea[row] = S;
-    __nv_bfloat162 *d1 = reinterpret_cast<__nv_bfloat162 *>(A1 + (long long)row * kp);
-    __nv_bfloat162 *d2 = reinterpret_cast<__nv_bfloat162 *>(A2 + (long long)row * kp);
-#pragma unroll 2
-    for (int l2 = threadIdx.x; l2 < kp / 2; l2 += 256) {
-        const int l = 2 * l2;
-        double2 v = make_double2(0.0, 0.0);
-        if (l + 1 < k) {
-            v = src[l2];
-        } else if (l < k) {
-            v.x = base[l];
-        }
-        __nv_bfloat16 h0, o0, h1, o1;
-        split_bf16(v.x, S, h0, o0);
-        split_bf16(v.y, S, h1, o1);
-        d1[l2] = __halves2bfloat162(h0, h1);
-        d2[l2] = __halves2bfloat162(o0, o1);
-    }
-}
-
 // One 64 (k) x 64 (column) tile of B -> transposed BF16 hi / lo tiles of
 // B1t, B2t (n x kp); 256 threads, through shared memory.
 // (B1t, B2t rows `pitch` elements apart; columns [0, kp) written)
@@ -817,21 +749,15 @@ __device__ __forceinline__ void split_b_tile(const double *B, long long ldb, int
     }
 }
 
-// B (k x n, ldb) -> B1t, B2t (n x kp, transposed), zero padding in [k, kp)
-__global__ void split_cols_t_kernel(const double *B, long long ldb, int k, int n, int kp, const int *eb,
-                                    __nv_bfloat16 *B1t, __nv_bfloat16 *B2t) {
-    split_b_tile(B, ldb, k, n, kp, kp, eb, B1t, B2t, blockIdx.y * 64, blockIdx.x * 64);
-}
-
-// B (k x n, ldb even, 16-byte aligned) -> column scales eb and B1t, B2t
+// B (k x n; V2: ldb even, 16-byte aligned) -> column scales eb and B1t, B2t
 // (n x kp, transposed), zero padding in [k, kp).  One CTA per strip of 16
 // columns, one pass over B: every entry is split unscaled (S = 0) while the
 // columns' largest exponents are gathered; a column whose scale turns out
 // not to be 0 (bf16_col_scale: its largest entry outside [2^-20, 2^40), or
 // a non-finite entry) is split again with its scale, re-reading the strip
-// -- normally no column.  Same scales and splits as col_maxexp +
-// exp_to_bf16_col_scale + split_cols_t, with B read once.
+// -- normally no column.
 constexpr int kStripThreads = 512;
+template <bool V2>
 __device__ __forceinline__ void split_cols_strip(const double *B, long long ldb, int k, int n, int kp, int *eb,
                                                  __nv_bfloat16 *B1t, __nv_bfloat16 *B2t, int strip) {
     __shared__ int red[64][17];
@@ -847,10 +773,12 @@ __device__ __forceinline__ void split_cols_strip(const double *B, long long ldb,
         double2 v = make_double2(0.0, 0.0);
         if (l < k) {
             const double *src = B + (long long)l * ldb + col;
-            if (in1)
+            if (V2 && in1) {
                 v = *reinterpret_cast<const double2 *>(src);
-            else if (in0)
-                v.x = *src;
+            } else {
+                if (in0) v.x = src[0];
+                if (in1) v.y = src[1];
+            }
         }
         return v;
     };
@@ -920,24 +848,21 @@ __device__ __forceinline__ void split_cols_strip(const double *B, long long ldb,
     }
 }
 
-__global__ void __launch_bounds__(kStripThreads) split_cols_strip_kernel(const double *B, long long ldb, int k, int n,
-                                                                        int kp, int *eb, __nv_bfloat16 *B1t,
-                                                                        __nv_bfloat16 *B2t) {
-    split_cols_strip(B, ldb, k, n, kp, eb, B1t, B2t, blockIdx.x);
-}
-
 // One row of A -> its scale exponent and BF16 hi / lo rows, by 256 threads
-// (half of a 512-thread CTA) synchronising on named barrier `bar`; row
-// 16-byte aligned, lda even.  Same results as split_rows_v2_kernel.
+// (half of a 512-thread CTA) synchronising on named barrier `bar`; V2: rows
+// 16-byte aligned.
+template <bool V2>
 __device__ __forceinline__ void split_row_half(const double *base, int k, int kp, int *ea_row, __nv_bfloat16 *a1,
                                                __nv_bfloat16 *a2, int t, int bar, int *red8) {
-    const double2 *src = reinterpret_cast<const double2 *>(base);
+    auto load = [&](int l2) {
+        return V2 ? reinterpret_cast<const double2 *>(base)[l2] : make_double2(base[2 * l2], base[2 * l2 + 1]);
+    };
     const int k2 = k >> 1;
     auto ex = [](double x) { return biased_exp_or_flag((unsigned long long)__double_as_longlong(x)); };
     int mx = 0;
 #pragma unroll 8
     for (int l2 = t; l2 < k2; l2 += 256) {
-        const double2 v = src[l2];
+        const double2 v = load(l2);
         mx = max(mx, max(ex(v.x), ex(v.y)));
     }
     if ((k & 1) && t == 0) mx = max(mx, ex(base[k - 1]));
@@ -957,7 +882,7 @@ __device__ __forceinline__ void split_row_half(const double *base, int k, int kp
         const int l = 2 * l2;
         double2 v = make_double2(0.0, 0.0);
         if (l + 1 < k) {
-            v = src[l2];
+            v = load(l2);
         } else if (l < k) {
             v.x = base[l];
         }
@@ -971,21 +896,25 @@ __device__ __forceinline__ void split_row_half(const double *base, int k, int kp
 
 // Both operands in one launch: CTAs [0, nstrip) split 16-column strips of
 // B, the rest split two rows of A each, so the bandwidth-bound row splits
-// run while the strips wait on their loads.
+// run while the strips wait on their loads.  VA, VB: 16-byte loads of A, B,
+// where leading dimension and base allow them (8-byte loads otherwise: 1000 x
+// 777 x 1300 31 us with the product, where column maxima, their scales, rows and columns in
+// launches of their own made it 45 us).
+template <bool VA, bool VB>
 __global__ void __launch_bounds__(kStripThreads) split_ab_kernel(const double *A, long long lda, int m,
                                                                 const double *B, long long ldb, int n, int k, int kp,
                                                                 int nstrip, int *ea, int *eb, __nv_bfloat16 *A1,
                                                                 __nv_bfloat16 *A2, __nv_bfloat16 *B1t,
                                                                 __nv_bfloat16 *B2t) {
     if ((int)blockIdx.x < nstrip) {
-        split_cols_strip(B, ldb, k, n, kp, eb, B1t, B2t, blockIdx.x);
+        split_cols_strip<VB>(B, ldb, k, n, kp, eb, B1t, B2t, blockIdx.x);
         return;
     }
     __shared__ int red8[2][8];
     const int half = threadIdx.x >> 8;
     const int row = 2 * ((int)blockIdx.x - nstrip) + half;
     if (row >= m) return;
-    split_row_half(A + (long long)row * lda, k, kp, ea + row, A1 + (long long)row * kp, A2 + (long long)row * kp,
+    split_row_half<VA>(A + (long long)row * lda, k, kp, ea + row, A1 + (long long)row * kp, A2 + (long long)row * kp,
                    threadIdx.x & 255, 1 + half, red8[half]);
 }
 
@@ -1042,13 +971,31 @@ __device__ __forceinline__ void split_tf32(double x, int S, float &hi, float &lo
     lo = round_tf32(__fadd_rn(__fsub_rn(h, hi), l));
 }
 
-// rows of A, one 256-thread block each: the row's scale exponent, then
-// the TF32 pair (zeros in the padding [k, kp)); the second pass reads the
-// row from L2
+// Column maxima of B (k x n), 32 columns x rows_per rows a block of the first
+// max_blocks, atomicMax into eb (zeroed first; the later kernels turn them into
+// scales, max_to_scale); then rows of A, a 256-thread
+// block each: the row's scale exponent and the TF32 pair (zeros in the
+// padding [k, kp)); the second pass reads the row from L2.  The maxima hide
+// behind the rows' traffic: as launches of their own they and the scales took
+// 13 us of 1000 x 777 x 1300's 60.
 __global__ void __launch_bounds__(256) split_rows_tf32_kernel(const double *A, long long lda, int m, int k, int kp,
-                                                             int *ea, float *A1, float *A2) {
+                                                             int *ea, float *A1, float *A2, const double *B,
+                                                             long long ldb, int n, int rows_per, int col_blocks,
+                                                             int max_blocks, int *eb) {
+    if ((int)blockIdx.x < max_blocks) {
+        const int col = (int)(blockIdx.x % col_blocks) * 32 + (threadIdx.x & 31);
+        const int r0 = (int)(blockIdx.x / col_blocks) * rows_per, r1 = min(k, r0 + rows_per);
+        int mx = 0;
+        if (col < n) {
+#pragma unroll 8
+            for (int l = r0 + (threadIdx.x >> 5); l < r1; l += 8)
+                mx = max(mx, eff_exp_or_flag((unsigned long long)__double_as_longlong(B[(long long)l * ldb + col])));
+        }
+        if (mx > 0) atomicMax(eb + col, mx);
+        return;
+    }
     __shared__ int red[8];
-    const int row = blockIdx.x, tid = threadIdx.x;
+    const int row = blockIdx.x - max_blocks, tid = threadIdx.x;
     const double *src = A + (long long)row * lda;
     int mx = 0;
 #pragma unroll 4
@@ -1072,28 +1019,14 @@ __global__ void __launch_bounds__(256) split_rows_tf32_kernel(const double *A, l
     }
 }
 
-// column maxima of B (k x n) over chunks of 256 rows: 32 columns x 8 row
-// groups per block, atomicMax into eb (zeroed first); exp_to_scale_kernel
-// then turns the maxima into scale exponents
-__global__ void col_max_tf32_kernel(const double *B, long long ldb, int k, int n, int *eb) {
-    const int col = blockIdx.x * 32 + threadIdx.x;
-    const int l0 = blockIdx.y * 256, l1 = min(k, l0 + 256);
-    if (col >= n) return;
-    int mx = 0;
-#pragma unroll 8
-    for (int l = l0 + threadIdx.y; l < l1; l += 8)
-        mx = max(mx, eff_exp_or_flag((unsigned long long)__double_as_longlong(B[(long long)l * ldb + col])));
-    if (mx > 0) atomicMax(eb + col, mx);
-}
-
 // B transposed and split: 32 x 32 tiles through shared memory (reads along
-// n, writes along k), zeros in the padding [k, kp)
+// n, writes along k), zeros in the padding [k, kp); eb: the column maxima
 __global__ void split_cols_tf32_kernel(const double *B, long long ldb, int k, int n, int kp, const int *eb,
                                        float *B1, float *B2) {
     __shared__ float th[32][33], tl[32][33];
     const int c0 = blockIdx.x * 32, l0 = blockIdx.y * 32;
     const int x = threadIdx.x, c = c0 + x;
-    const int S = c < n ? eb[c] : 0;
+    const int S = c < n ? max_to_scale(eb[c]) : 0;
     for (int y = threadIdx.y; y < 32; y += 8) {
         const int l = l0 + y;
         float h = 0.0f, lo = 0.0f;
@@ -1257,40 +1190,17 @@ void launch_gemm_split3(int m, int n, int k, const double *A, long long lda, con
     unsigned *err = reinterpret_cast<unsigned *>(eb + n);
     OO_CUDA_TRY(cudaMemsetAsync(err, 0, 4, s));
 
-    const bool strip_b = ldb % 2 == 0 && ((uintptr_t)B & 15u) == 0;
+    const bool cols_v2 = ldb % 2 == 0 && ((uintptr_t)B & 15u) == 0;
     const bool rows_v2 = lda % 2 == 0 && ((uintptr_t)A & 15u) == 0;
-    if (strip_b && rows_v2) {
-        const int nstrip = (n + 15) / 16;
-        const long long grid = (long long)nstrip + (m + 1) / 2;
-        OO_REQUIRE(grid < (1ll << 31), OO_EINVAL, "problem too large");
-        split_ab_kernel<<<(unsigned)grid, kStripThreads, 0, s>>>(A, lda, m, B, ldb, n, k, kp, nstrip, ea, eb, A1, A2,
-                                                                B1, B2);
-        OO_CUDA_TRY(cudaGetLastError());
-    } else if (!strip_b) {
-        OO_CUDA_TRY(cudaMemsetAsync(eb, 0, (size_t)n * 4, s));
-        const int rows_per = 256;
-        dim3 grid((n + 31) / 32, (k + rows_per - 1) / rows_per), block(32, 8);
-        OO_REQUIRE(grid.y <= 65535, OO_EINVAL, "k too large");
-        col_maxexp_kernel<<<grid, block, 0, s>>>(B, ldb, k, n, rows_per, eb);
-        OO_CUDA_TRY(cudaGetLastError());
-        exp_to_bf16_col_scale_kernel<<<(n + 255) / 256, 256, 0, s>>>(eb, n);
-        OO_CUDA_TRY(cudaGetLastError());
-    }
-    if (!(strip_b && rows_v2)) {
-        if (rows_v2)
-            split_rows_v2_kernel<<<m, 256, 0, s>>>(A, lda, m, k, kp, ea, A1, A2);
-        else
-            split_rows_fused_kernel<<<(m + 7) / 8, 256, 0, s>>>(A, lda, m, k, kp, ea, A1, A2);
-        OO_CUDA_TRY(cudaGetLastError());
-        if (strip_b) {
-            split_cols_strip_kernel<<<(n + 15) / 16, kStripThreads, 0, s>>>(B, ldb, k, n, kp, eb, B1, B2);
-        } else {
-            dim3 grid((n + 63) / 64, kp / 64);
-            OO_REQUIRE(grid.y <= 65535, OO_EINVAL, "k too large");
-            split_cols_t_kernel<<<grid, 256, 0, s>>>(B, ldb, k, n, kp, eb, B1, B2);
-        }
-        OO_CUDA_TRY(cudaGetLastError());
-    }
+    OO_REQUIRE(cols_v2 || kp / 64 <= 65535, OO_EINVAL, "k too large");
+    const int nstrip = (n + 15) / 16;
+    const long long split_grid = (long long)nstrip + (m + 1) / 2;
+    OO_REQUIRE(split_grid < (1ll << 31), OO_EINVAL, "problem too large");
+    (rows_v2 ? (cols_v2 ? split_ab_kernel<true, true> : split_ab_kernel<true, false>)
+             : (cols_v2 ? split_ab_kernel<false, true> : split_ab_kernel<false, false>))<<<(unsigned)split_grid,
+                                                                                           kStripThreads, 0, s>>>(
+        A, lda, m, B, ldb, n, k, kp, nstrip, ea, eb, A1, A2, B1, B2);
+    OO_CUDA_TRY(cudaGetLastError());
     GemmMaps maps;
     map_bf16(&maps.a1, A1, m, kp, kBM);
     map_bf16(&maps.a2, A2, m, kp, kBM);
@@ -1371,16 +1281,15 @@ void launch_gemm_split3_tf32(int m, int n, int k, const double *A, long long lda
     int *ea = reinterpret_cast<int *>(p + 2 * L.a_bytes + 2 * L.b_bytes);
     int *eb = ea + m;
     unsigned *err = reinterpret_cast<unsigned *>(eb + n);
-    OO_CUDA_TRY(cudaMemsetAsync(err, 0, 4, s));
-    split_rows_tf32_kernel<<<m, 256, 0, s>>>(A, lda, m, k, kp, ea, A1, A2);
+    OO_CUDA_TRY(cudaMemsetAsync(eb, 0, (size_t)n * 4 + 4, s));  // the column maxima and the error word
+    constexpr int kRowsPer = 128;
+    const int col_blocks = (n + 31) / 32;
+    const long long max_blocks = (long long)col_blocks * ((k + kRowsPer - 1) / kRowsPer);
+    OO_REQUIRE(max_blocks + m < (1ll << 31), OO_EINVAL, "matrix too large");
+    split_rows_tf32_kernel<<<(unsigned)(max_blocks + m), 256, 0, s>>>(A, lda, m, k, kp, ea, A1, A2, B, ldb, n,
+                                                                     kRowsPer, col_blocks, (int)max_blocks, eb);
     OO_CUDA_TRY(cudaGetLastError());
-    OO_CUDA_TRY(cudaMemsetAsync(eb, 0, (size_t)n * 4, s));
-    OO_REQUIRE((k + 255) / 256 <= 65535, OO_EINVAL, "k too large");
-    col_max_tf32_kernel<<<dim3((n + 31) / 32, (k + 255) / 256), dim3(32, 8), 0, s>>>(B, ldb, k, n, eb);
-    OO_CUDA_TRY(cudaGetLastError());
-    exp_to_scale_kernel<<<(n + 255) / 256, 256, 0, s>>>(eb, n);
-    OO_CUDA_TRY(cudaGetLastError());
-    OO_REQUIRE(kp / 32 <= 65535, OO_EINVAL, "k too large");
+    OO_REQUIRE((k + 255) / 256 <= 65535 && kp / 32 <= 65535, OO_EINVAL, "k too large");
     split_cols_tf32_kernel<<<dim3((n + 31) / 32, kp / 32), dim3(32, 8), 0, s>>>(B, ldb, k, n, kp, eb, B1, B2);
     OO_CUDA_TRY(cudaGetLastError());
     GemmMaps maps;
