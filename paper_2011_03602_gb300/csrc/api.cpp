@@ -12,6 +12,7 @@ struct oo_ctx {
     Ctx c;
     // cached stencil launch state for oo_stencil_dev (keyed by its arguments)
     StencilPlan *user_plan = nullptr;
+    void *user_scratch = nullptr;  // its scratch: partial residuals, counter, error word; for any grid
     std::vector<const void *> user_key;
     int gemm_prec = -1;  // precision pattern of the last GEMM launch
 };
@@ -145,6 +146,7 @@ void oo_destroy(oo_ctx *ctx) {
     }
     if (ctx->c.stream) cudaStreamSynchronize(ctx->c.stream);
     stencil_plan_destroy(ctx->user_plan);
+    if (ctx->user_scratch) cudaFree(ctx->user_scratch);
     jacobi_work_free(ctx->c.jw);
     for (auto &kv : ctx->c.fft_plans) fft_plan_destroy(kv.second);
     ctx->c.fft_scratch.release();
@@ -268,12 +270,17 @@ oo_status oo_stencil_dev(oo_ctx *ctx, int I, int J, int K, int pitch, const floa
         const int want = ctx->c.stencil_variant_for(I, J, K);
         key.push_back(reinterpret_cast<const void *>((intptr_t)want));
         if (!ctx->user_plan || ctx->user_key != key) {
-            if (ctx->user_plan) {
-                OO_CUDA_TRY(cudaStreamSynchronize(ctx->c.stream));
-                stencil_plan_destroy(ctx->user_plan);
-                ctx->user_plan = nullptr;
-            }
-            ctx->user_plan = stencil_plan_create(JacobiDims{I, J, K, pitch}, coef, p, wrk2, ctx->c.num_sms, want);
+            // Other arrays or another grid: new tensor maps over the context's
+            // scratch, which the stream orders behind the last sweep's use of it.
+            // A plan with scratch of its own waited for that sweep to free it and
+            // allocated again: 88 us for 150 x 131 x 270 where the sweep takes 70.
+            const JacobiDims d{I, J, K, pitch};
+            const size_t bytes = stencil_scratch_bytes(d, ctx->c.num_sms);
+            if (!ctx->user_scratch) OO_CUDA_TRY(cudaMalloc(&ctx->user_scratch, bytes));
+            StencilPlan *np = stencil_plan_create_ext(d, coef, p, wrk2, ctx->c.num_sms, ctx->user_scratch, bytes,
+                                                      ctx->c.stream, want);
+            stencil_plan_destroy(ctx->user_plan);
+            ctx->user_plan = np;
             ctx->user_key = key;
         }
         const bool inject = ctx->c.inject_wait == OO_INJECT_STENCIL_LOAD;
