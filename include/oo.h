@@ -252,9 +252,7 @@ oo_status oo_stencil_check(oo_ctx *ctx);
  * Every call shares the array and clears its counter and error word first,
  * so calls that overlap on the GPU (other streams, other contexts on the
  * same device) race and must not be issued.  The tile variant and work
- * split are oo_stencil_dev's (same wrk2 bits; the same residual bits while
- * that split fits the array, else the residual is summed over fewer
- * i-segments and agrees to about 1e-12 relative).  Grids whose tiles
+ * split are oo_stencil_dev's (same wrk2 and residual bits).  Grids whose tiles
  * alone need more than 65536 partial slots (ceil((K-1)/TK) *
  * ceil((J-2)/TJ) * consumer warps; TK x TJ = 128 x 8 with 16 warps by
  * default for K > 65) are rejected with OO_EINVAL.  Arguments and layout as
@@ -295,8 +293,8 @@ oo_status oo_tune_stencil(oo_ctx *ctx, int I, int J, int K, int *variant, double
  *                           issues its first p-tile copy, so the consumer
  *                           warps' bounded wait (about one second) runs out;
  *   OO_INJECT_FUSED_BARRIER the next fused-iteration launch (small grids,
- *                           all iteration nests on the GPU) waits at its first
- *                           grid barrier for one block more than it launched.
+ *                           all iteration nests on the GPU) waits in its first
+ *                           iteration for one block more than it launched.
  *   OO_INJECT_SERVE_STALL   the device-resident serving loop started next
  *                           (oo_serve_start_resident) gives the first request
  *                           it admits a work entry whose dependency never
@@ -685,11 +683,13 @@ typedef struct {
 typedef struct oo_batch oo_batch;
 oo_status oo_batch_create(oo_ctx *ctx, const oo_req *reqs, int n_req, oo_batch **out);
 /* mode 0: grouped persistent kernels (GEMM split passes + one tensor-core
- *         kernel over every split-BF16 tile, one split launch + one
- *         tensor-core kernel over every FP64-equivalent tile; FFT maxima
- *         pass + three item launches), the GEMM and FFT groups on forked
+ *         kernel over every split-BF16 tile; row and column split launches
+ *         per accumulation scheme + a tensor-core kernel over every
+ *         FP64-equivalent tile of the level schemes and one of the pair
+ *         scheme; three FFT item launches), the GEMM and FFT groups on forked
  *         streams;
- * mode 1: the same, captured into a CUDA graph on first use and replayed;
+ * mode 1: the same, captured into a CUDA graph on first use (which runs the
+ *         launches themselves unless the batch has run before) and replayed;
  * mode 2: one library call per request (oo_gemm_f64_dev / oo_fft_c128_dev).
  * Asynchronous on the context's stream.                                  */
 oo_status oo_batch_run(oo_batch *b, int mode);
