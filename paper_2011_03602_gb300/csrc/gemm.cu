@@ -19,12 +19,13 @@
 // FP64 oracle, not claimed to be FP64.
 //
 // Kernels: persistent, warp-specialised.  gemm_split3_pair_kernel (the
-// default) runs 256 x 256 output tiles on CTA pairs (cta_group::2, M = 256,
-// N = 256 MMAs, each SM holding half of the tile's B columns);
+// default) runs 256 x W output tiles (W = 64 .. 256) on CTA pairs
+// (cta_group::2, M = 256, N = W MMAs, each SM holding half of the tile's B
+// columns);
 // gemm_split3_kernel and the grouped kernel run 128 x 128 tiles on single
 // CTAs (M = 128, N = 128).  Warp 0 issues TMA loads of the four BF16 operand
 // tiles (128B-swizzled, K-major) into a 3-stage ring, warp 1 allocates 512
-// TMEM columns (two accumulator buffers) and one of its threads issues
+// TMEM columns (two accumulator buffers) and an elected lane of it issues
 // tcgen05.mma (K = 16, kind::f16, BF16 x BF16 -> FP32) and tcgen05.commit
 // to release stages; eight epilogue warps (4-11, two per TMEM lane quarter)
 // read finished accumulators with tcgen05.ld and write FP64 C while the
@@ -898,8 +899,8 @@ __device__ __forceinline__ void split_row_half(const double *base, int k, int kp
 // B, the rest split two rows of A each, so the bandwidth-bound row splits
 // run while the strips wait on their loads.  VA, VB: 16-byte loads of A, B,
 // where leading dimension and base allow them (8-byte loads otherwise: 1000 x
-// 777 x 1300 31 us with the product, where column maxima, their scales, rows and columns in
-// launches of their own made it 45 us).
+// 777 x 1300 31 us with the product, 45 us where column maxima, their scales,
+// rows and columns had launches of their own).
 template <bool VA, bool VB>
 __global__ void __launch_bounds__(kStripThreads) split_ab_kernel(const double *A, long long lda, int m,
                                                                 const double *B, long long ldb, int n, int k, int kp,

@@ -935,6 +935,8 @@ __global__ void __launch_bounds__(256) eq_group_split_cols_kernel(const eq::GSpl
     const int4 jb = jobs[blockIdx.x];
     eq::split_cols_job(gs[jb.y], jb.z, t, red);
 }
+
+// the pair scheme's units and scales, up to `most` slices of B a unit
 void set_units(EqArgs &a, const EqShape &e, int most) {
     const std::vector<eq::PairUnit> U = eq::pair_units(e, most);
     OO_REQUIRE((int)U.size() <= kMaxUnits, OO_EINVAL, "too many product groups");
@@ -970,6 +972,7 @@ void launch_pair(EqArgs &a, const EqShape &e, __nv_bfloat16 *As, __nv_bfloat16 *
     cfg.numAttrs = 1;
     OO_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_fp64eq_pair_kernel<TN>, (const EqPairMaps)pm, (const EqArgs)a));
 }
+
 }  // namespace
 
 void eq_group_split_jobs(int scheme, int problem, int m, int n, std::vector<int4> (&jobs)[6]) {
