@@ -283,6 +283,7 @@ __device__ __forceinline__ void gemm_body(const Src &src, unsigned *err) {
     __syncthreads();
     fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    wait_previous();
 
     int loaded = 0;          // producer: stages issued
     int tiles_mma = 0;       // MMA issuer: tiles whose accumulation was issued
@@ -522,6 +523,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_split3_pair_kernel(const
     cluster_sync_all();  // both CTAs' barriers and TMEM exist before either uses the other's
     fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    wait_previous();
 
     int loaded = 0, tiles_mma = 0;
     if (warp == 0) {
@@ -907,6 +909,7 @@ __global__ void __launch_bounds__(kStripThreads) split_ab_kernel(const double *A
                                                                 int nstrip, int *ea, int *eb, __nv_bfloat16 *A1,
                                                                 __nv_bfloat16 *A2, __nv_bfloat16 *B1t,
                                                                 __nv_bfloat16 *B2t) {
+    next_may_start();
     if ((int)blockIdx.x < nstrip) {
         split_cols_strip<VB>(B, ldb, k, n, kp, eb, B1t, B2t, blockIdx.x);
         return;
@@ -1025,6 +1028,7 @@ __global__ void __launch_bounds__(256) split_rows_tf32_kernel(const double *A, l
 __global__ void split_cols_tf32_kernel(const double *B, long long ldb, int k, int n, int kp, const int *eb,
                                        float *B1, float *B2) {
     __shared__ float th[32][33], tl[32][33];
+    next_may_start();
     const int c0 = blockIdx.x * 32, l0 = blockIdx.y * 32;
     const int x = threadIdx.x, c = c0 + x;
     const int S = c < n ? max_to_scale(eb[c]) : 0;
@@ -1152,18 +1156,19 @@ void launch_split3_pair(const GemmMaps &maps, GemmArgs ga, int nw, int ncl, cuda
     ga.n_tiles = (ga.n + nw - 1) / nw;              // nw-column panels
     const long long units = (long long)ga.m_tiles * ga.n_tiles;
     OO_REQUIRE(units < (1ll << 31), OO_EINVAL, "too many tiles");
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1] = programmatic();
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(2 * std::min<long long>(units, ncl)));
     cfg.blockDim = dim3(kGemmThreads);
     cfg.dynamicSmemBytes = kSmemPair;
     cfg.stream = s;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     OO_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_split3_pair_kernel, maps, (const GemmArgs)ga));
 }
 
@@ -1240,8 +1245,7 @@ void launch_gemm_split3(int m, int n, int k, const double *A, long long lda, con
     cudaGetDevice(&dev2);
     cudaDeviceGetAttribute(&sms2, cudaDevAttrMultiProcessorCount, dev2);
     const int grid = (int)std::min<long long>(tiles, sms2);
-    gemm_split3_kernel<<<grid, kGemmThreads, smem_gemm(), s>>>(maps, ga);
-    OO_CUDA_TRY(cudaGetLastError());
+    launch_behind(gemm_split3_kernel, grid, kGemmThreads, smem_gemm(), s, maps, ga);
 }
 
 // ------------------------------------------------------- TF32 pattern
@@ -1319,8 +1323,7 @@ void launch_gemm_split3_tf32(int m, int n, int k, const double *A, long long lda
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int grid = (int)std::min<long long>(tiles, sms);
-    gemm_split3_tf32_kernel<<<grid, kGemmThreads, smem_gemm(), s>>>(maps, ga);
-    OO_CUDA_TRY(cudaGetLastError());
+    launch_behind(gemm_split3_tf32_kernel, grid, kGemmThreads, smem_gemm(), s, maps, ga);
 }
 
 // ------------------------------------------------------------ group plans

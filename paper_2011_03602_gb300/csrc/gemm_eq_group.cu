@@ -662,6 +662,7 @@ __device__ __forceinline__ void eq_levels_body(const LvMaps &maps, unsigned *err
     __syncthreads();
     fence_after();
     pp.tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    wait_previous();
     int st = 0, kc = 0, tile = 0, last_w = 0;
     if (warp == 0) {
         const uint32_t el = elect_one();
@@ -1271,8 +1272,7 @@ void launch_gemm_eq_tiles(int m, int n, int k, const void *As, const void *Bs, c
     static std::atomic<uint64_t> attr{0};
     set_smem_limit_once((const void *)eq_levels_single_kernel, kLvSmem, attr);
     const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, num_sms));
-    eq_levels_single_kernel<<<grid, kLvThreads, kLvSmem, s>>>(maps, err, P);
-    OO_CUDA_TRY(cudaGetLastError());
+    launch_behind(eq_levels_single_kernel, grid, kLvThreads, kLvSmem, s, maps, err, P);
 }
 
 // ---------------------------------------------------------- the autotuner

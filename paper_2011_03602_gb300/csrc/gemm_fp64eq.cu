@@ -395,6 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
     cluster_sync_all();  // both CTAs' barriers and TMEM exist before either uses the other's
     fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    wait_previous();
 
     int loaded = 0, units_mma = 0;
     if (warp == 0) {
@@ -674,6 +675,7 @@ __global__ void __launch_bounds__(256) eq_split_rows_kernel(const double *A, lon
 __global__ void eq_split_cols_t_kernel(const double *B, long long ldb, int k, int n, int kp, int beta, int s,
                                        const int *mxo, int *eb, __nv_bfloat16 *Bs) {
     __shared__ double t[64][65];
+    next_may_start();
     const int c0 = blockIdx.x * 64, l0 = blockIdx.y * 64;
     const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
     if (l0 == 0 && ty == 0 && c0 + tx < n) eb[c0 + tx] = mxo[c0 + tx] == 0 ? 0 : mxo[c0 + tx] - 1022;
@@ -906,6 +908,7 @@ __global__ void __launch_bounds__(256) eq_level_split_kernel(const __grid_consta
                                                             unsigned *err) {
     extern __shared__ __align__(16) double lv_t[];
     __shared__ int red[256];
+    next_may_start();
     if (blockIdx.x == 0 && threadIdx.x == 0) *err = 0;  // of the product kernel that follows
     if ((int)blockIdx.x < row_blocks)
         LevelSplit<BETA, S>::rows(G, blockIdx.x * 32);
@@ -958,18 +961,19 @@ void launch_pair(EqArgs &a, const EqShape &e, __nv_bfloat16 *As, __nv_bfloat16 *
     map_bf16(&pm.a, As, (long long)e.slices * a.m, kp, kBM);
     map_bf16(&pm.b, Bs, (long long)e.slices * a.n, kp, TN);
     map_bf16(&pm.bh, Bs, (long long)e.slices * a.n, kp, TN / 2);
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1] = programmatic();
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(2 * clusters));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemEqPair;
     cfg.stream = s;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     OO_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_fp64eq_pair_kernel<TN>, (const EqPairMaps)pm, (const EqArgs)a));
 }
 

@@ -303,6 +303,36 @@ __device__ __forceinline__ void mma_commit_pair_if(uint32_t el, uint32_t bar, ui
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// Programmatic launch of a product kernel behind its split kernel: the split's
+// CTAs let it start (next_may_start) and it sets up its barriers and tensor
+// memory while they end; before it reads anything they wrote it waits for
+// all of the split (wait_previous; both do nothing in ordinary launches).  256^3
+// FP64-equivalent 24.6 -> 22.5 us, split-BF16 16.5 -> 12.6, split-TF32 26.9 -> 24.8;
+// 1024^3 70 -> 66, 26 -> 22, 42 -> 40.
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("fence.proxy.async.global;" ::: "memory");  // TMA reads what it stored
+}
+inline cudaLaunchAttribute programmatic() {
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    return a;
+}
+template <class... P, class... A>
+void launch_behind(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s, const A &...args) {
+    cudaLaunchAttribute at[1] = {programmatic()};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    OO_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+}
+
 // Non-finite inputs of the matrix products.  The exponent passes over A's
 // rows and B's columns report a row / column holding a NaN or an infinity
 // as this biased exponent (above every finite one), so its scale exponent
