@@ -99,8 +99,11 @@ __global__ void __launch_bounds__(T, 2 * (kFftThreads / T)) fft_pass_kernel(FftA
     // The stage table goes after the data (the 4096-point one is read in
     // place): copied when the data's loads are in flight, one latency instead of
     // two, but here in the full CTAs of the four-step passes, which have no
-    // registers for both (2^22 in 212 us with the spills that costs).
-    constexpr bool kTableFirst = MODE != 0 && T == kFftThreads;
+    // registers for both (2^22 in 212 us with the spills that costs), and in the
+    // second pass, which copies it while the first ends (launched
+    // programmatically behind it: 2^22 206.2 -> 202.3 us, 64 x 2^14 50.7 -> 49.8).
+    constexpr bool kTableFirst = MODE == 2 || (MODE == 1 && T == kFftThreads);
+    if (MODE == 1) asm volatile("griddepcontrol.launch_dependents;");
     const float4 *stw = a.tw;
     if (twiddles_staged(log2L)) {
         float4 *t_s = fsmem + kSlots;
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(T, 2 * (kFftThreads / T)) fft_pass_kernel(FftA
             if (MODE == 1) return ((q & (C - 1)) << log2L) + (q >> (31 - __clz(C)));
             return q;
         };
+        if (MODE == 2) asm volatile("griddepcontrol.wait;" ::: "memory");  // for all of the first pass
         double2 raw[kPer];
 #pragma unroll
         for (int r = 0; r < kPer; ++r) {
@@ -482,8 +486,17 @@ void launch_fft(const FftPlan *p, int batch, int dir, const double *in, double *
         set_smem_limit_once(p.fn, kFftSmemMax, *p.limit_set);
         const long long C = (long long)(T * kFftPer) >> log2L;
         void *args[] = {&a};
-        OO_CUDA_TRY(cudaLaunchKernel(p.fn, dim3((unsigned)((columns + C - 1) / C)), dim3(T), args,
-                                     fft_smem_bytes(log2L, T * kFftPer), s));
+        cudaLaunchAttribute at[1]{};
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)((columns + C - 1) / C));
+        cfg.blockDim = dim3(T);
+        cfg.dynamicSmemBytes = fft_smem_bytes(log2L, T * kFftPer);
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = mode == 2 ? 1 : 0;
+        OO_CUDA_TRY(cudaLaunchKernelExC(&cfg, p.fn, args));
     };
     if (!four_step) {
         a.in_d = in;
