@@ -472,7 +472,7 @@ __device__ __forceinline__ bool fused_wait(const unsigned *words, int lo, int hi
 __global__ void __launch_bounds__(kFusedThreads + 64, 1) jacobi_fused_kernel(FusedArgs a) {
     extern __shared__ float coef_s[];            // [NCOEF][cap]
     __shared__ float2 ss_s[2][kFusedThreads];    // each thread's residual, of an even / odd iteration
-    __shared__ int ok_s;
+    __shared__ int ok_s[2];                      // the exchange warp's verdict on an even / odd iteration
     constexpr int kAll = kFusedThreads + 64, kSync = kFusedThreads + 32;
     const int J = a.J, Ji = J - 2, Ki = a.K - 2;
     const long long nint = (long long)(a.I - 2) * Ji * Ki;
@@ -483,15 +483,18 @@ __global__ void __launch_bounds__(kFusedThreads + 64, 1) jacobi_fused_kernel(Fus
     const int lane = threadIdx.x & 31;
 
     // Barrier 1: iteration `it` of this CTA is stored (every warp).  Barrier 2:
-    // the neighbours' is too, or ok_s is false (all but the residual warp).
-    // After a failure barrier 1 is passed once more, where the residual warp
-    // reads ok_s.
+    // the neighbours' is too, or ok_s[it & 1] is false (all but the residual
+    // warp).  After a failure barrier 1 is passed once more, behind which the
+    // residual warp reads that verdict.  It reads iteration it - 1's while the
+    // exchange warp may be writing iteration it's, hence the two slots: with
+    // one, a residual warp that saw the later verdict left a barrier early, and
+    // the others waited for it there for ever.
     if (threadIdx.x >= kSync) {
         // ------------------------------------------------ residual warp
         bool ok = true;
         for (int it = 0; it < a.iters; ++it) {
             bar_named<kAll>(1);
-            if (it > 0 && !ok_s) return;
+            if (it > 0 && !ok_s[(it - 1) & 1]) return;
             if (!ok) continue;
             double v = 0.0;
 #pragma unroll 4
@@ -530,7 +533,7 @@ __global__ void __launch_bounds__(kFusedThreads + 64, 1) jacobi_fused_kernel(Fus
             bar_named<kAll>(1);
             if (lane == 0) st_release(a.done + b * kFusedLine, it + 1);
             const bool ok = fused_wait(a.done, lo, it == 0 ? hi + (int)a.wait_extra : hi, it + 1, a.err);
-            if (lane == 0) ok_s = ok;
+            if (lane == 0) ok_s[it & 1] = ok;
             bar_named<kSync>(2);
             if (!ok) {
                 if (it + 1 < a.iters) bar_named<kAll>(1);
@@ -594,7 +597,7 @@ __global__ void __launch_bounds__(kFusedThreads + 64, 1) jacobi_fused_kernel(Fus
         ss_s[it & 1][tid] = make_float2(RH, RL);
         bar_named<kAll>(1);
         bar_named<kSync>(2);
-        if (!ok_s) {
+        if (!ok_s[it & 1]) {
             if (it + 1 < a.iters) bar_named<kAll>(1);
             return;
         }
