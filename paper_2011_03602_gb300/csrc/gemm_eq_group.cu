@@ -267,7 +267,8 @@ __device__ __forceinline__ bool mma_tile(const GArgs &a, const Pipe &pp, const G
 // One epilogue warp (of eight: lane quarter q = warp & 3, column half h):
 // add every finished unit of one tile, scaled by its power of two, into a
 // float-float running sum (Sh, Sl) of this row's columns, then write FP64
-// C; false when the pipeline aborted
+// C; false when the pipeline aborted.  LEVELS: the tile may be of a level scheme
+template <bool LEVELS>
 __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, const GProb &P, const int4 td, int &gu,
                                               float (&Sh)[64], float (&Sl)[64]) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -280,7 +281,7 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
     const int ncols = min(cpw, P.n - td.z - cw0);
     const bool active = row0 < P.m && ncols > 0;  // warp-uniform
     const int units = P.nkb * S.nunits;
-    const bool levels = P.scheme >= kTabLevel7;
+    const bool levels = LEVELS && P.scheme >= kTabLevel7;
 #pragma unroll
     for (int j = 0; j < 64; ++j) Sh[j] = Sl[j] = 0.0f;
     for (int uu = 0; uu < units; ++uu, ++gu) {
@@ -288,32 +289,27 @@ __device__ __forceinline__ bool epilogue_tile(const GArgs &a, const Pipe &pp, co
         if (!bar_wait(su32(&pp.tfull[b]), (gu >> 1) & 1, pp.abort_flag, a.err, 4u)) return false;
         fence_after();
         const int u = uu % S.nunits;
-        // powers of two, exact scales; the pair scheme adds the right half first (eq::pair_units)
-        const bool swap = !levels && S.usR[u] != 0.0f;
-        const float f1 = swap ? S.usR[u] : S.usL[u], f2 = swap ? S.usL[u] : S.usR[u];
+        const float fL = S.usL[u], fR = S.usR[u];  // powers of two, exact scales; fR 0: no right half
         if (active) {
             const uint32_t acc = pp.tmem + (uint32_t)(b * 256) + lane_off + (uint32_t)cw0;
-            const uint32_t acc1 = acc + (swap ? td.w : 0), acc2 = acc + (swap ? 0 : td.w);
 #pragma unroll
-            for (int c = 0; c < 64; c += 16) {
-                if (c < ncols) {
-                    uint32_t v[16];
-                    OO_TMEM_LD16(acc1 + c, v);
-                    tmem_wait_ld();
+            for (int c = 0; c < 64; c += 8) {
+                if (c >= ncols) continue;
+                uint32_t v[8], w[8];
+                OO_TMEM_LD8(acc + c, v);
+                if (!LEVELS || fR != 0.0f) OO_TMEM_LD8(acc + (uint32_t)td.w + c, w);  // (unread without a right half)
+                tmem_wait_ld();
+                if (levels) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), f1);
-                        if (!levels) eq::renormalise(Sh[c + j], Sl[c + j]);
+                    for (int j = 0; j < 8; ++j) eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), fL);
+                    if (fR != 0.0f) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(w[j]), fR);
                     }
-                    if (f2 != 0.0f) {
-                        OO_TMEM_LD16(acc2 + c, v);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), f2);
-                            if (!levels) eq::renormalise(Sh[c + j], Sl[c + j]);
-                        }
-                    }
+                } else if (fR != 0.0f) {
+                    eq::add_two8(Sh + c, Sl + c, w, fR, v, fL);
+                } else {
+                    eq::add_one8(Sh + c, Sl + c, v, fL);
                 }
             }
         }
@@ -382,7 +378,7 @@ __device__ __forceinline__ void eq_tiles_body(const GMaps &maps, const GArgs &a,
         int gu = 0;
         for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
             const int4 td = src.tile(t);
-            if (!epilogue_tile(a, pp, src.prob(td.x), td, gu, Sh, Sl)) break;
+            if (!epilogue_tile<false>(a, pp, src.prob(td.x), td, gu, Sh, Sl)) break;
         }
     }
     pipe_teardown(pp, loaded, units_mma);
@@ -877,7 +873,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_tiles_kernel(const __gri
             if (td.x == kTileStop) break;
             if (td.x < 0) continue;
             const ResTileDesc &D = r.desc[td.x];
-            if (!epilogue_tile(a, pp, D.P, td, gu, Sh, Sl)) break;
+            if (!epilogue_tile<true>(a, pp, D.P, td, gu, Sh, Sl)) break;
             __syncwarp();
             if (lane == 0) {
                 __threadfence();

@@ -235,20 +235,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
                 const float f1 = a.us[pr], f2 = f1 * a.uq_step;
                 const uint32_t acc = tmem + (uint32_t)(b * 2 * kBN) + lane_off + (uint32_t)(h * 64);
 #pragma unroll
-                for (int c = 0; c < 64; c += 16) {
-                    uint32_t v[16];
-#pragma unroll
-                    for (int half = 1; half >= 0; --half) {  // the smaller contribution first
-                        if (half == 1 && !pair) continue;
-                        OO_TMEM_LD16(acc + half * kBN + c, v);
-                        tmem_wait_ld();
-                        const float f = half ? f2 : f1;  // a power of two: exact scale
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            eq::add_scaled(Sh[c + j], Sl[c + j], __uint_as_float(v[j]), f);
-                            eq::renormalise(Sh[c + j], Sl[c + j]);
-                        }
-                    }
+                for (int c = 0; c < 64; c += 8) {
+                    uint32_t v[8], w[8];
+                    OO_TMEM_LD8(acc + c, v);
+                    if (pair) OO_TMEM_LD8(acc + kBN + c, w);
+                    tmem_wait_ld();
+                    if (pair)
+                        eq::add_two8(Sh + c, Sl + c, w, f2, v, f1);  // powers of two: exact scales
+                    else
+                        eq::add_one8(Sh + c, Sl + c, v, f1);
                 }
                 fence_before();
                 __syncwarp();
@@ -312,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
 // and 1050 while the epilogue ran, for 512 clocks of MMA; n = 4096 took 2.92
 // ms in this kernel, 2.29 ms so (3.13 -> 2.56 ms with the splits).
 // The epilogue: C is stored through shared memory (eq::store_columns) and a
-// running sum costs 10 operations a product, the power-of-two scale folded
+// running sum costs 8 operations a product, the power-of-two scale folded
 // into them.  With a row of C per lane and the conversion unrolled over the
 // columns the store took 122,000 clocks a tile, in which the tensor cores did
 // two units of the next tile and then waited: n = 4096 2.50 -> 2.18 ms, n =
@@ -334,15 +329,6 @@ constexpr uint32_t kStageBytesPair = 2 * kTile;  // A_p and this CTA's B tile
 struct EqPairMaps {
     CUtensorMap a, b, bh;  // B slices in boxes of a tile's columns and of half as many
 };
-
-// running sums += eight accumulator columns, scaled by f
-__device__ __forceinline__ void add8(float *Sh, float *Sl, const uint32_t (&d)[8], float f) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        eq::add_scaled(Sh[j], Sl[j], __uint_as_float(d[j]), f);
-        eq::renormalise(Sh[j], Sl[j]);
-    }
-}
 
 template <int TN>
 __device__ __forceinline__ void eq_tile_pair(const EqArgs &a, int t, int &m0, int &n0) {
@@ -522,10 +508,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_pair_kernel(const __g
                     if (TN < kBN && nq > 2) OO_TMEM_LD8(acc + 2 * TN + c, x);
                     if (TN < kBN && nq > 3) OO_TMEM_LD8(acc + 3 * TN + c, y);
                     tmem_wait_ld();
-                    if (TN < kBN && nq > 3) add8(Sh + c, Sl + c, y, f4);  // smallest first
-                    if (TN < kBN && nq > 2) add8(Sh + c, Sl + c, x, f3);
-                    if (nq > 1) add8(Sh + c, Sl + c, w, f2);
-                    add8(Sh + c, Sl + c, v, f1);
+                    if (TN < kBN && nq > 3)  // smallest first
+                        eq::add_two8(Sh + c, Sl + c, y, f4, x, f3);
+                    else if (TN < kBN && nq > 2)
+                        eq::add_one8(Sh + c, Sl + c, x, f3);
+                    if (nq > 1)
+                        eq::add_two8(Sh + c, Sl + c, w, f2, v, f1);
+                    else
+                        eq::add_one8(Sh + c, Sl + c, v, f1);
                 }
                 fence_before();
                 __syncwarp();
