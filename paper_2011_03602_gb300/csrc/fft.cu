@@ -480,8 +480,8 @@ void launch_fft(const FftPlan *p, int batch, int dir, const double *in, double *
     a.n = n;
     a.batch = batch;
     a.inverse = dir > 0 ? 1 : 0;
-    auto pass = [&](int mode, int log2L, long long columns) {
-        const int T = fft_threads(mode, log2L, columns, num_sms());
+    const int sms = num_sms();
+    auto pass = [&](int mode, int log2L, long long columns, int T, size_t smem) {
         const FftPass p = fft_pass(mode, fft_padded(log2L), T);
         set_smem_limit_once(p.fn, kFftSmemMax, *p.limit_set);
         const long long C = (long long)(T * kFftPer) >> log2L;
@@ -492,7 +492,7 @@ void launch_fft(const FftPlan *p, int batch, int dir, const double *in, double *
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)((columns + C - 1) / C));
         cfg.blockDim = dim3(T);
-        cfg.dynamicSmemBytes = fft_smem_bytes(log2L, T * kFftPer);
+        cfg.dynamicSmemBytes = smem;
         cfg.stream = s;
         cfg.attrs = at;
         cfg.numAttrs = mode == 2 ? 1 : 0;
@@ -502,17 +502,29 @@ void launch_fft(const FftPlan *p, int batch, int dir, const double *in, double *
         a.in_d = in;
         a.out_d = out;
         a.tw = p->tw_single;
-        pass(0, p->log2n, batch);
+        const int T = fft_threads(0, p->log2n, batch, sms);
+        pass(0, p->log2n, batch, T, fft_smem_bytes(p->log2n, T * kFftPer));
         return;
     }
+    const long long cols1 = (long long)batch << p->log2n2, cols2 = (long long)batch << p->log2n1;
+    const int T1 = fft_threads(1, p->log2n1, cols1, sms), T2 = fft_threads(2, p->log2n2, cols2, sms);
+    size_t smem1 = fft_smem_bytes(p->log2n1, T1 * kFftPer), smem2 = fft_smem_bytes(p->log2n2, T2 * kFftPer);
+    // Both passes of small CTAs ask for the same shared memory.  Asking for a
+    // little more in the second (lengths 2^odd) can make the SMs split L1 and
+    // shared memory differently for it, and an SM does that only when it is
+    // empty, so that the second pass's early CTAs held the first up: 2^13 x 48
+    // 37.0 us, 25.9 so; 2^17 x 4 41.4 and 33.0.  From one and a half full CTAs per
+    // SM on, the larger first pass loses as much (2^17 x 7 47.0 and 47.2, x 8 49.3
+    // and 50.4).
+    if (T1 == T2 && T1 < kFftThreads && 2 * (n * batch / kFftElems) < 3ll * sms) smem1 = smem2 = std::max(smem1, smem2);
     a.tw_hi = p->tw_hi;
     a.tw_lo = p->tw_lo;
     a.in_d = in;
     a.tw = p->tw_n1;
-    pass(1, p->log2n1, (long long)batch << p->log2n2);
+    pass(1, p->log2n1, cols1, T1, smem1);
     a.out_d = out;
     a.tw = p->tw_n2;
-    pass(2, p->log2n2, (long long)batch << p->log2n1);
+    pass(2, p->log2n2, cols2, T2, smem2);
 }
 
 // ------------------------------------------------------------ group plans
