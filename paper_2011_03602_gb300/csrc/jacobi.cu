@@ -669,7 +669,9 @@ struct StencilArgs {
     int I, J, K, pitch;
     int n_kt;
     int whole, n_col, seg, i_cut, tail;  // work split (Runs)
+    int seg_q, seg_r, tail_q, tail_r;    // i_cut by seg, planes above the cut by tail: quotients and remainders
     float omega;
+    int chained;        // a face pass is the predecessor: coefficients may be loaded before it has ended
     float *wrk2;
     double *partials;   // consumer warps x CTAs
     unsigned *counter;  // CTAs finished (reset by the last one)
@@ -706,10 +708,24 @@ struct Tile {
 // all tile planes per CTA 336 / 48.9 us (its CTAs are at unrelated planes, p
 // is read 2.5 times from HBM); this split 303 / 47.6 us.
 // next(): the runs of planes of one column that CTA b marches through, in order.
+// QUICK: the same with short divisions, for the producer, whose first copies
+// wait for them (64-bit ones and the coefficient ring before p took 12 % of a
+// small sweep: 24 x 107 x 111 16.6 us, 14.6 so); in the consumers, which wait for
+// the copies, they cost the main loop registers (257 x 257 x 513 299 -> 303 us).
+template <bool QUICK>
 struct Runs {
+    using Pos = std::conditional_t<QUICK, int, long long>;
     int step, b;
-    long long pos, end;     // a tail CTA's range of tile planes above the cut
+    Pos pos, end;           // a tail CTA's range of tile planes above the cut
     __device__ __forceinline__ explicit Runs(int b_) : step(0), b(b_), pos(0), end(0) {}
+    // x / n, rounded down, for 0 <= x < 2^21: the quotient of x + 1/2 is at least
+    // 1 / 2n away from every integer, more than its error
+    static __device__ __forceinline__ int quot(int x, int n) { return (int)__fdividef((float)x + 0.5f, (float)n); }
+    // x t / n, rounded down, x = q n + r (t and n at most the CTAs)
+    static __device__ __forceinline__ Pos part(long long x, int q, int r, int t, int n) {
+        if (QUICK) return t * q + quot(t * r, n);
+        return (Pos)(x * t / n);
+    }
     __device__ __forceinline__ bool next(const StencilArgs &a, int TK, int TJ, int &k0, int &j0, int &ib, int &ie) {
         const int span = a.I - 2;
         int col, i0, i1;
@@ -719,27 +735,33 @@ struct Runs {
             i1 = span;
         } else if (b < a.seg * a.n_col) {
             if (step > a.whole) return false;
-            const int s = b / a.n_col;
-            col = b % a.n_col;
-            i0 = (int)((long long)a.i_cut * s / a.seg);
-            i1 = (int)((long long)a.i_cut * (s + 1) / a.seg);
+            const int s = QUICK ? quot(b, a.n_col) : b / a.n_col;
+            col = QUICK ? b - s * a.n_col : b % a.n_col;
+            i0 = (int)part(a.i_cut, a.seg_q, a.seg_r, s, a.seg);
+            i1 = (int)part(a.i_cut, a.seg_q, a.seg_r, s + 1, a.seg);
         } else {
             const int t = b - a.seg * a.n_col, h = span - a.i_cut;
             if (step == a.whole) {
                 if (t >= a.tail) return false;
-                pos = (long long)a.n_col * h * t / a.tail;
-                end = (long long)a.n_col * h * (t + 1) / a.tail;
+                pos = part((long long)a.n_col * h, a.tail_q, a.tail_r, t, a.tail);
+                end = part((long long)a.n_col * h, a.tail_q, a.tail_r, t + 1, a.tail);
             }
             if (pos >= end) return false;
             col = (int)(pos / h);
             i0 = a.i_cut + (int)(pos % h);
-            i1 = (int)min((long long)span, i0 + end - pos);
+            i1 = (int)min((Pos)span, i0 + end - pos);
             pos += i1 - i0;
         }
         if (step >= a.whole) col += a.whole * (int)gridDim.x;
         ++step;
-        k0 = col % a.n_kt * TK;
-        j0 = 1 + col / a.n_kt * TJ;
+        if (QUICK && a.whole == 0) {  // fewer columns than CTAs
+            const int jt = quot(col, a.n_kt);
+            k0 = (col - jt * a.n_kt) * TK;
+            j0 = 1 + jt * TJ;
+        } else {
+            k0 = col % a.n_kt * TK;
+            j0 = 1 + col / a.n_kt * TJ;
+        }
         ib = 1 + i0;
         ie = 1 + i1;
         return true;
@@ -810,15 +832,20 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
                 return true;
             };
             // A sweep launched to overlap its predecessor's end (launch_stencil,
-            // `chained`) may fill its coefficient ring -- no launch writes those
-            // arrays then -- before it waits for the predecessor's p.
-            Runs runs(blockIdx.x);
+            // a later turn) fills its coefficient ring -- no launch writes those
+            // arrays then -- before it waits for the predecessor's p.  Any other
+            // sweep has nothing to wait for and asks for p first, which the
+            // consumers need first.
+            Runs<true> runs(blockIdx.x);
             int k0, j0, ib, ie;
             bool more = runs.next(a, TK, TJ, k0, j0, ib, ie);
-            for (int i = ib; more && i < ie && i < ib + DC; ++i) load_coef(k0, j0, i);
-            uint32_t ahead = cfill;  // coefficient planes of this run already loaded
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            asm volatile("fence.proxy.async.global;" ::: "memory");
+            uint32_t ahead = 0;  // coefficient planes of this run already loaded
+            if (a.chained) {
+                for (int i = ib; more && i < ie && i < ib + DC; ++i) load_coef(k0, j0, i);
+                ahead = cfill;
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                asm volatile("fence.proxy.async.global;" ::: "memory");
+            }
             for (; ok && more; more = runs.next(a, TK, TJ, k0, j0, ib, ie), ahead = 0) {
                 for (int q = ib - 1; q <= ie; ++q) {
                     {
@@ -907,7 +934,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB)
         uint32_t cuse = 0, pseq = 0;
         bool ok = true;
         double racc = 0.0;           // this thread's ss^2 sum, run after run
-        Runs runs(blockIdx.x);
+        Runs<false> runs(blockIdx.x);
         int k0, j0, ib, ie;
         while (ok && runs.next(a, TK, TJ, k0, j0, ib, ie)) {
             const int j = j0 + r, kb = k0 + PPT * cg;
@@ -1249,6 +1276,15 @@ void fill_stencil_plan(StencilPlan *sp, const JacobiDims &d, const float *const 
         }
         if (std::ceil((double)span / a.seg) + kRunStart <= best) a.tail = 0, a.i_cut = span;
     }
+    // equal segments only: as few as are no longer, whose CTAs read fewer halo planes
+    // (17 x 33 x 357: 8 segments of two planes 13.2 us, 12 of one or two 14.1)
+    if (a.n_col && a.tail == 0) {
+        const int longest = (span + a.seg - 1) / a.seg;
+        a.seg = (span + longest - 1) / longest;
+    }
+    if (a.seg > 0) a.seg_q = a.i_cut / a.seg, a.seg_r = a.i_cut % a.seg;
+    const long long above = (long long)a.n_col * (span - a.i_cut);
+    if (a.tail > 0) a.tail_q = (int)(above / a.tail), a.tail_r = (int)(above % a.tail);
     sp->grid = a.whole ? G : a.seg * a.n_col + a.tail;
     a.wrk2 = wrk2;
 }
@@ -1331,19 +1367,17 @@ void stencil_plan_destroy(StencilPlan *sp) {
     delete sp;
 }
 
-void launch_stencil(StencilPlan *sp, float omega, double *res_dev, cudaStream_t s, bool inject_timeout, bool flip,
-                    bool chained) {
-    sp->args.omega = omega;
-    sp->args.res = res_dev;
-    if (!flip) {
-        variant(sp->variant).launch(sp->grid, sp->maps, sp->args, s, inject_timeout, chained);
-        return;
-    }
+void launch_stencil(StencilPlan *sp, float omega, double *res_dev, cudaStream_t s, bool inject_timeout, int turn) {
     StencilMaps maps = sp->maps;
     StencilArgs args = sp->args;
-    maps.p = sp->p_flip;
-    args.wrk2 = sp->out_flip;
-    variant(sp->variant).launch(sp->grid, maps, args, s, inject_timeout, chained);
+    args.omega = omega;
+    args.res = res_dev;
+    args.chained = turn > 0;
+    if (turn > 0 && (turn & 1)) {
+        maps.p = sp->p_flip;
+        args.wrk2 = sp->out_flip;
+    }
+    variant(sp->variant).launch(sp->grid, maps, args, s, inject_timeout, args.chained);
 }
 
 const unsigned *stencil_plan_err_ptr(const StencilPlan *sp) { return sp->args.err; }

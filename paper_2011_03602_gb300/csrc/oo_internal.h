@@ -378,13 +378,13 @@ void stencil_plan_destroy(StencilPlan *sp);
 // inject_timeout: fault injection for tests -- the producer never issues the
 // first p-tile fill, so the consumers' bounded wait runs out (~1 s) and the
 // sweep reports an error bit instead of a result
-// flip: the sweep reads the plan's wrk2 and writes its p (whose memory must
-// be the caller's to write)
-// chained: the launch before it on s is a launch_bc_faces whose sweep, like
-// this one, finds its coefficients unchanged; the sweep may then set itself
-// up and load coefficients while its predecessor ends
+// turn: -1 a sweep by itself; 0, 1, ... the iteration of a run in which p and
+// wrk2 (whose memory must be the caller's to write) exchange roles and a
+// launch_bc_faces follows each sweep: odd turns read wrk2 and write p, and a
+// turn after the first, whose coefficients are the last one's, may set itself
+// up and load coefficients while the face pass before it ends
 void launch_stencil(StencilPlan *sp, float omega, double *res_dev, cudaStream_t s, bool inject_timeout = false,
-                    bool flip = false, bool chained = false);
+                    int turn = -1);
 // All iterations of the all-GPU iteration nests in one cooperative launch
 // (small grids): ctl is jacobi_fused_ctl_bytes() of device scratch, whose
 // first word is nonzero afterwards if a bounded wait ran out.  Both

@@ -265,8 +265,7 @@ void run_pattern(Ctx &c, uint64_t gene, int hoist, const oo_jacobi &prob, float 
                     // applies to the next stencil sweep launched
                     const bool inject = c.inject_wait == OO_INJECT_STENCIL_LOAD;
                     if (inject) c.inject_wait = OO_INJECT_NONE;
-                    launch_stencil(w.splan, prob.omega, w.res_dev + it, s, inject, exchange && (it & 1),
-                                   exchange && it > 0);
+                    launch_stencil(w.splan, prob.omega, w.res_dev + it, s, inject, exchange ? it : -1);
                     if (!stencil_on_gpu) {
                         // a pipeline wait that ran out would repeat in every
                         // sweep: check the first one before queueing the rest

@@ -197,7 +197,7 @@ void start(Server &S, SReq &q) {
         const float *p_dev = a[VAR_P];
         for (int it = 0; it < r.iters; ++it) {
             float *out = a[it & 1 ? VAR_P : VAR_WRK2];
-            launch_stencil(q.splan, r.omega, res + it, s, false, it & 1, it > 0);
+            launch_stencil(q.splan, r.omega, res + it, s, false, it);
             launch_bc_faces(d, out, s);  // N4 + N5
             p_dev = out;
         }
