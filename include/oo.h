@@ -232,8 +232,9 @@ oo_status oo_stencil_dev(oo_ctx *ctx, int I, int J, int K, int pitch,
                          const float *const *coef, const float *p, float omega,
                          float *wrk2, double *res_dev);
 /* After oo_stencil_dev sweeps: synchronise the context's stream and report
- * OO_ETIMEOUT if a bounded pipeline wait of the last plan's sweeps ran out
- * (their wrk2 / residual are then incomplete); the error word is cleared. */
+ * OO_ETIMEOUT if a bounded pipeline wait of any sweep since the last check
+ * ran out, on whichever arrays (that sweep's wrk2 / residual are then
+ * incomplete); the error word is cleared.                                */
 oo_status oo_stencil_check(oo_ctx *ctx);
 
 /* The same stencil sweep as oo_stencil_dev, for callers that cannot

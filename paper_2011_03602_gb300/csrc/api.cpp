@@ -271,14 +271,17 @@ oo_status oo_stencil_dev(oo_ctx *ctx, int I, int J, int K, int pitch, const floa
         key.push_back(reinterpret_cast<const void *>((intptr_t)want));
         if (!ctx->user_plan || ctx->user_key != key) {
             // Other arrays or another grid: new tensor maps over the context's
-            // scratch, which the stream orders behind the last sweep's use of it.
+            // scratch, which the stream orders behind the last sweep's use of it and
+            // whose error word keeps any sweep's time-out until oo_stencil_check.
             // A plan with scratch of its own waited for that sweep to free it and
             // allocated again: 88 us for 150 x 131 x 270 where the sweep takes 70.
             const JacobiDims d{I, J, K, pitch};
             const size_t bytes = stencil_scratch_bytes(d, ctx->c.num_sms);
-            if (!ctx->user_scratch) OO_CUDA_TRY(cudaMalloc(&ctx->user_scratch, bytes));
-            StencilPlan *np = stencil_plan_create_ext(d, coef, p, wrk2, ctx->c.num_sms, ctx->user_scratch, bytes,
-                                                      ctx->c.stream, want);
+            if (!ctx->user_scratch) {
+                OO_CUDA_TRY(cudaMalloc(&ctx->user_scratch, bytes));
+                stencil_scratch_clear(ctx->user_scratch, ctx->c.stream);
+            }
+            StencilPlan *np = stencil_plan_create_ext(d, coef, p, wrk2, ctx->c.num_sms, ctx->user_scratch, bytes, want);
             stencil_plan_destroy(ctx->user_plan);
             ctx->user_plan = np;
             ctx->user_key = key;

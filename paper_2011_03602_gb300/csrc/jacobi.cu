@@ -1288,26 +1288,29 @@ void fill_stencil_plan(StencilPlan *sp, const JacobiDims &d, const float *const 
     sp->grid = a.whole ? G : a.seg * a.n_col + a.tail;
     a.wrk2 = wrk2;
 }
+// Scratch: counter and error word in the first 256 bytes, whatever the grid, so
+// that plans which share it (oo_stencil_dev) leave each other's alone; then the
+// partial residuals.
+constexpr size_t kScratchHead = 256;
 void attach_scratch(StencilPlan *sp, void *scratch) {
     StencilArgs &a = sp->args;
     sp->scratch = scratch;
-    a.partials = reinterpret_cast<double *>(scratch);
-    a.counter = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(scratch) +
-                                             (size_t)sp->grid * kMaxConsumerWarps * 8);
+    a.counter = static_cast<unsigned *>(scratch);
     a.err = a.counter + 1;
+    a.partials = reinterpret_cast<double *>(static_cast<char *>(scratch) + kScratchHead);
 }
 size_t plan_scratch_bytes(const StencilPlan *sp) {
-    return (size_t)sp->grid * kMaxConsumerWarps * 8 + 256;
+    return kScratchHead + (size_t)sp->grid * kMaxConsumerWarps * 8;
 }
 }  // namespace
 
 size_t stencil_scratch_bytes(const JacobiDims &d, int num_sms) {
     (void)d;
-    return (size_t)num_sms * kMaxCtasPerSm * kMaxConsumerWarps * 8 + 256;  // of any tile variant
+    return kScratchHead + (size_t)num_sms * kMaxCtasPerSm * kMaxConsumerWarps * 8;  // of any tile variant
 }
 
 StencilPlan *stencil_plan_create_ext(const JacobiDims &d, const float *const coef[NCOEF], const float *p, float *wrk2,
-                                     int num_sms, void *scratch, size_t scratch_bytes, cudaStream_t s, int variant) {
+                                     int num_sms, void *scratch, size_t scratch_bytes, int variant) {
     OO_REQUIRE(d.I >= 3 && d.J >= 3 && d.K >= 3, OO_EINVAL, "grid must be at least 3 x 3 x 3");
     OO_REQUIRE(d.pitch >= d.K && d.pitch % 4 == 0, OO_EINVAL, "pitch must be >= K and a multiple of 4");
     OO_REQUIRE(((uintptr_t)wrk2 & 15u) == 0 && ((uintptr_t)scratch & 15u) == 0, OO_EINVAL,
@@ -1319,7 +1322,6 @@ StencilPlan *stencil_plan_create_ext(const JacobiDims &d, const float *const coe
         OO_REQUIRE(plan_scratch_bytes(sp) <= scratch_bytes, OO_EINVAL, "stencil scratch too small");
         attach_scratch(sp, scratch);
         sp->own_scratch = false;
-        OO_CUDA_TRY(cudaMemsetAsync(sp->args.counter, 0, 8, s));
     } catch (...) {
         delete sp;
         throw;
@@ -1340,7 +1342,7 @@ StencilPlan *stencil_plan_create(const JacobiDims &d, const float *const coef[NC
         void *scr = nullptr;
         OO_CUDA_TRY(cudaMalloc(&scr, bytes));
         attach_scratch(sp, scr);
-        OO_CUDA_TRY(cudaMemset(sp->scratch, 0, bytes));
+        OO_CUDA_TRY(cudaMemset(sp->scratch, 0, kScratchHead));
     } catch (...) {
         if (sp->scratch) cudaFree(sp->scratch);
         delete sp;
@@ -1381,6 +1383,8 @@ void launch_stencil(StencilPlan *sp, float omega, double *res_dev, cudaStream_t 
 }
 
 const unsigned *stencil_plan_err_ptr(const StencilPlan *sp) { return sp->args.err; }
+
+void stencil_scratch_clear(void *scratch, cudaStream_t s) { OO_CUDA_TRY(cudaMemsetAsync(scratch, 0, kScratchHead, s)); }
 
 unsigned stencil_plan_check(StencilPlan *sp, cudaStream_t s) {
     unsigned e = 0;

@@ -367,12 +367,14 @@ int stencil_plan_variant(const StencilPlan *sp);
 int stencil_variant_count();
 // the variant a plan takes when none is chosen (by row length)
 int stencil_default_variant(const JacobiDims &d);
-// A plan whose scratch (partial residuals, counter, error word) lives in
-// caller-provided device memory of at least stencil_scratch_bytes(d, sms).
+// A plan whose scratch (counter, error word, partial residuals) lives in
+// caller-provided device memory of at least stencil_scratch_bytes(d, sms),
+// cleared once (stencil_scratch_clear): a sweep leaves the counter at zero, and
+// plans that share the memory share its error word.
 StencilPlan *stencil_plan_create_ext(const JacobiDims &d, const float *const coef[NCOEF], const float *p, float *wrk2,
-                                     int num_sms, void *scratch, size_t scratch_bytes, cudaStream_t s,
-                                     int variant = -1);
+                                     int num_sms, void *scratch, size_t scratch_bytes, int variant = -1);
 size_t stencil_scratch_bytes(const JacobiDims &d, int num_sms);
+void stencil_scratch_clear(void *scratch, cudaStream_t s);
 void stencil_plan_destroy(StencilPlan *sp);
 // One stencil sweep; the residual (FP64) lands in *res_dev.
 // inject_timeout: fault injection for tests -- the producer never issues the
@@ -398,7 +400,7 @@ float *launch_jacobi_fused(const JacobiDims &d, const float *const coef[NCOEF], 
                            bool inject_timeout = false);
 // Device address of the plan's error word (0 = fine).
 const unsigned *stencil_plan_err_ptr(const StencilPlan *sp);
-// Reads and clears the device-side error word of the plan (0 = fine).
+// Reads and clears the device-side error word of the plan's scratch (0 = fine).
 unsigned stencil_plan_check(StencilPlan *sp, cudaStream_t s);
 
 // Host nests (host_nests.cpp), on unpadded I x J x K arrays.
