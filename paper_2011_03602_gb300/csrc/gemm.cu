@@ -752,6 +752,33 @@ __device__ __forceinline__ void split_b_tile(const double *B, long long ldb, int
     }
 }
 
+// The split of B where one CTA per strip of columns would walk a long inner
+// dimension alone (launch_gemm_split3): the columns' largest exponents (eb,
+// zeroed first; blocks of 32 columns x kMaxRows rows), their scales, then 64 x
+// 64 tiles.  Same scales and splits as split_cols_strip.
+constexpr int kMaxRows = 256;
+__global__ void __launch_bounds__(256) col_maxexp_kernel(const double *B, long long ldb, int k, int n, int col_blocks,
+                                                       int *eb) {
+    const int col = (int)(blockIdx.x % col_blocks) * 32 + (threadIdx.x & 31);
+    const int r0 = (int)(blockIdx.x / col_blocks) * kMaxRows, r1 = min(k, r0 + kMaxRows);
+    if (col >= n) return;
+    int mx = 0;
+#pragma unroll 8
+    for (int l = r0 + (threadIdx.x >> 5); l < r1; l += 8)
+        mx = max(mx, biased_exp_or_flag((unsigned long long)__double_as_longlong(B[(long long)l * ldb + col])));
+    if (mx > 0) atomicMax(eb + col, mx);
+}
+__global__ void col_scale_kernel(int *eb, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) eb[i] = bf16_col_scale(eb[i]);
+}
+__global__ void __launch_bounds__(256) split_cols_tiles_kernel(const double *B, long long ldb, int k, int n, int kp,
+                                                             int col_tiles, const int *eb, __nv_bfloat16 *B1t,
+                                                             __nv_bfloat16 *B2t) {
+    split_b_tile(B, ldb, k, n, kp, kp, eb, B1t, B2t, (int)(blockIdx.x / col_tiles) * 64,
+                 (int)(blockIdx.x % col_tiles) * 64);
+}
+
 // B (k x n; V2: ldb even, 16-byte aligned) -> column scales eb and B1t, B2t
 // (n x kp, transposed), zero padding in [k, kp).  One CTA per strip of 16
 // columns, one pass over B: every entry is split unscaled (S = 0) while the
@@ -1199,7 +1226,22 @@ void launch_gemm_split3(int m, int n, int k, const double *A, long long lda, con
     const bool cols_v2 = ldb % 2 == 0 && ((uintptr_t)B & 15u) == 0;
     const bool rows_v2 = lda % 2 == 0 && ((uintptr_t)A & 15u) == 0;
     OO_REQUIRE(cols_v2 || kp / 64 <= 65535, OO_EINVAL, "k too large");
-    const int nstrip = (n + 15) / 16;
+    // One CTA a strip walks 64 rows at a time with 8-byte loads (odd ldb): a long
+    // inner dimension and few strips take the tiles instead.  16 x 17 x 65536 681 us
+    // in strips, 380 so, 16 x 17 x 16384 178 and 116, 1000 x 257 x 16384 218 and 202;
+    // 16 x 1025 x 16384 203 and 210, 1000 x 257 x 4096 56 and 61.
+    const bool tiles_b = !cols_v2 && n <= 512 && k >= 16384;
+    const int nstrip = tiles_b ? 0 : (n + 15) / 16;
+    if (tiles_b) {
+        OO_CUDA_TRY(cudaMemsetAsync(eb, 0, (size_t)n * 4, s));
+        const int mb = (n + 31) / 32, tb = (n + 63) / 64;
+        col_maxexp_kernel<<<mb * ((k + kMaxRows - 1) / kMaxRows), 256, 0, s>>>(B, ldb, k, n, mb, eb);
+        OO_CUDA_TRY(cudaGetLastError());
+        col_scale_kernel<<<(n + 255) / 256, 256, 0, s>>>(eb, n);
+        OO_CUDA_TRY(cudaGetLastError());
+        split_cols_tiles_kernel<<<tb * (kp / 64), 256, 0, s>>>(B, ldb, k, n, kp, tb, eb, B1, B2);
+        OO_CUDA_TRY(cudaGetLastError());
+    }
     const long long split_grid = (long long)nstrip + (m + 1) / 2;
     OO_REQUIRE(split_grid < (1ll << 31), OO_EINVAL, "problem too large");
     (rows_v2 ? (cols_v2 ? split_ab_kernel<true, true> : split_ab_kernel<true, false>)
