@@ -465,7 +465,9 @@ oo_status oo_gemm_scheme(int k, int *scheme, int *per_accumulator);
  * oo_tune_gemm_tiles: the autotuner.  For every bucket it times each width
  * on a synthetic group of products drawn in the bucket (one warm-up and
  * three timed launches, CUDA events on the context's stream), keeps the
- * fastest in the context's table and writes it to widths (may be NULL);
+ * fastest in the context's table and writes it to widths (may be NULL); for
+ * k <= 512 widths 64 and 128 are one launch, timed once, and the built-in
+ * table decides between them;
  * ms (may be NULL) receives OO_TILE_NBUCKETS x OO_TILE_KBUCKETS x 3 mean
  * launch times (widths 32, 64, 128).  Batches created afterwards use the
  * table.  Synchronous; allocates device memory for the trial.

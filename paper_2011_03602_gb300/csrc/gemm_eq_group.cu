@@ -1004,10 +1004,11 @@ double tile_cost(const eq::Shape &e, int ksteps, int width) {
 
 // The accumulation scheme of an FP64-equivalent product with inner
 // dimension k: a fixed rule, so a problem gives the same bits alone and in a
-// batch.  Measured on GB300 (grouped products of the batched workload):
-// levels with 7-bit digits up to one 128-deep K-block, levels with 6-bit
-// digits up to 512, the pair scheme beyond (long K: tensor-bound, fewer
-// products win).
+// batch: levels with 7-bit digits up to one 128-deep K-block, levels with 6-bit
+// digits up to 512, the pair scheme beyond (28 products for 36).  The line at
+// 512 was measured on grouped products with both schemes in the unit-based
+// roles (k in 513 .. 1024: 2.48 ms pairs, 2.59 ms levels); the level kernel,
+// 2.8 times as fast up to 512, takes one K-block and has not run beyond it.
 int eq_scheme_for(int k) {
     if (k <= 128) return eq::kSchemeLevel7;
     if (k <= 512) return eq::kSchemeLevel6;
@@ -1016,7 +1017,9 @@ int eq_scheme_for(int k) {
 
 // The built-in tile widths: the autotuner's choices on GB300, written by
 // paper_2011_03602_gb300/tune_gemm_tiles.py (rows n <= 32 .. > 512, columns
-// k <= 64 .. > 512).
+// k <= 64 .. > 512), with every tile in the unit-based roles, which the
+// resident loop and the pair scheme run.  The level kernel runs widths above 64
+// as 64 (level_width).
 int eq_default_width(int nb, int kb) {
     static const int table[OO_TILE_NBUCKETS][OO_TILE_KBUCKETS] = {
 #include "eq_tile_table.inc"
@@ -1275,7 +1278,8 @@ void launch_gemm_eq_tiles(int m, int n, int k, const void *As, const void *Bs, c
 // For every (n, k) bucket: a fixed synthetic group of products drawn in the
 // bucket (m log-uniform in [16, 512], n and k uniform in the bucket's range;
 // zero inputs, the work does not depend on the values), timed with every
-// tile width; the fastest width is kept in the context's table.
+// tile width that has a launch of its own; the fastest is kept in the context's
+// table.
 void tune_gemm_tiles(Ctx &c, double *ms_out) {
     static const int nlo[OO_TILE_NBUCKETS] = {16, 33, 65, 129, 257, 513};
     static const int nhi[OO_TILE_NBUCKETS] = {32, 64, 128, 256, 512, 1024};
@@ -1325,7 +1329,12 @@ void tune_gemm_tiles(Ctx &c, double *ms_out) {
                 }
                 float best = 0.f;
                 int best_w = 128;
-                for (int wi = 0; wi < 3; ++wi) {
+                // the level kernel runs 128-wide entries as 64-wide ones: one launch, timed
+                // once; between the two the built-in table decides, which the
+                // resident loop's tiles were measured with
+                const bool level = eq_scheme_for(khi[kb]) != eq::kSchemePairs;
+                double *ms_at = ms_out ? ms_out + (nb * OO_TILE_KBUCKETS + kb) * 3 : nullptr;
+                for (int wi = 0; wi < (level ? 2 : 3); ++wi) {
                     std::array<int, OO_TILE_NBUCKETS * OO_TILE_KBUCKETS> tab;
                     tab.fill(widths[wi]);
                     g = eq_group_create(v, c.num_sms, tab.data());
@@ -1341,12 +1350,14 @@ void tune_gemm_tiles(Ctx &c, double *ms_out) {
                     OO_REQUIRE(eq_group_check(g, s) == 0, OO_ETIMEOUT, "pipeline wait ran out while tuning");
                     eq_group_destroy(g);
                     g = nullptr;
-                    if (ms_out) ms_out[(nb * OO_TILE_KBUCKETS + kb) * 3 + wi] = ms;
+                    if (ms_at) ms_at[wi] = ms;
                     if (wi == 0 || ms < best) {
                         best = ms;
                         best_w = widths[wi];
                     }
                 }
+                if (level && ms_at) ms_at[2] = ms_at[1];
+                if (level && best_w == 64) best_w = std::max(64, eq_default_width(nb, kb));
                 OO_CUDA_TRY(cudaStreamSynchronize(s));
                 OO_CUDA_TRY(cudaFree(buf));
                 buf = nullptr;
