@@ -253,10 +253,11 @@ oo_status oo_stencil_check(oo_ctx *ctx);
  * Every call shares the array and clears its counter and error word first,
  * so calls that overlap on the GPU (other streams, other contexts on the
  * same device) race and must not be issued.  The tile variant and work
- * split are oo_stencil_dev's (same wrk2 and residual bits).  Grids whose tiles
- * alone need more than 65536 partial slots (ceil((K-1)/TK) *
- * ceil((J-2)/TJ) * consumer warps; TK x TJ = 128 x 8 with 16 warps by
- * default for K > 65) are rejected with OO_EINVAL.  Arguments and layout as
+ * split are oo_stencil_dev's (same wrk2 and residual bits).  Grids for which
+ * ceil((K-1)/TK) * ceil((J-2)/TJ) * W exceeds 65536 are rejected with
+ * OO_EINVAL, TK x TJ and W being the chosen or tuned variant's tile and
+ * consumer warps, and 128 x 8 and 16 (64 x 8 and 8 for K <= 65) where none is
+ * chosen, whatever tile the default rule then runs.  Arguments and layout as
  * for oo_stencil_dev; asynchronous on the context's stream.  A bounded
  * pipeline wait that runs out is reported by oo_stencil_noalloc_check, not
  * by this call.                                                          */

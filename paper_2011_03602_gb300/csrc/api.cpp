@@ -276,7 +276,7 @@ oo_status oo_stencil_dev(oo_ctx *ctx, int I, int J, int K, int pitch, const floa
             // A plan with scratch of its own waited for that sweep to free it and
             // allocated again: 88 us for 150 x 131 x 270 where the sweep takes 70.
             const JacobiDims d{I, J, K, pitch};
-            const size_t bytes = stencil_scratch_bytes(d, ctx->c.num_sms);
+            const size_t bytes = stencil_scratch_bytes(ctx->c.num_sms);
             if (!ctx->user_scratch) {
                 OO_CUDA_TRY(cudaMalloc(&ctx->user_scratch, bytes));
                 stencil_scratch_clear(ctx->user_scratch, ctx->c.stream);

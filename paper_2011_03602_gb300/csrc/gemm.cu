@@ -1225,7 +1225,7 @@ void launch_gemm_split3(int m, int n, int k, const double *A, long long lda, con
 
     const bool cols_v2 = ldb % 2 == 0 && ((uintptr_t)B & 15u) == 0;
     const bool rows_v2 = lda % 2 == 0 && ((uintptr_t)A & 15u) == 0;
-    OO_REQUIRE(cols_v2 || kp / 64 <= 65535, OO_EINVAL, "k too large");
+    OO_REQUIRE(cols_v2 || kp / 64 <= 65535, OO_EINVAL, "k too large");  // the entry's limit, no launch's
     // One CTA a strip walks 64 rows at a time with 8-byte loads (odd ldb): a long
     // inner dimension and few strips take the tiles instead.  16 x 17 x 65536 681 us
     // in strips, 380 so, 16 x 17 x 16384 178 and 116, 1000 x 257 x 16384 218 and 202;
@@ -1336,7 +1336,7 @@ void launch_gemm_split3_tf32(int m, int n, int k, const double *A, long long lda
     split_rows_tf32_kernel<<<(unsigned)(max_blocks + m), 256, 0, s>>>(A, lda, m, k, kp, ea, A1, A2, B, ldb, n,
                                                                      kRowsPer, col_blocks, (int)max_blocks, eb);
     OO_CUDA_TRY(cudaGetLastError());
-    OO_REQUIRE((k + 255) / 256 <= 65535 && kp / 32 <= 65535, OO_EINVAL, "k too large");
+    OO_REQUIRE(kp / 32 <= 65535, OO_EINVAL, "k too large");
     split_cols_tf32_kernel<<<dim3((n + 31) / 32, kp / 32), dim3(32, 8), 0, s>>>(B, ldb, k, n, kp, eb, B1, B2);
     OO_CUDA_TRY(cudaGetLastError());
     GemmMaps maps;

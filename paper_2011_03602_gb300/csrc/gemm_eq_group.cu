@@ -995,9 +995,7 @@ int bucket_k(int k) {
 // relative cost of a tile, for ordering the work list (largest first)
 double tile_cost(const eq::Shape &e, int ksteps, int width) {
     if (e.scheme != eq::kSchemePairs) return (double)width * (ksteps * (double)e.nprod * 2.0 + 110.0);
-    return (double)width * ((double)ksteps * e.nprod + 8.0 * e.nkb * (e.scheme == eq::kSchemePairs
-                                                                        ? (e.nprod + e.slices) / 2.0
-                                                                        : (e.levels + 1) / 2.0));
+    return (double)width * ((double)ksteps * e.nprod + 8.0 * e.nkb * (e.nprod + e.slices) / 2.0);
 }
 
 }  // namespace

@@ -1304,9 +1304,8 @@ size_t plan_scratch_bytes(const StencilPlan *sp) {
 }
 }  // namespace
 
-size_t stencil_scratch_bytes(const JacobiDims &d, int num_sms) {
-    (void)d;
-    return kScratchHead + (size_t)num_sms * kMaxCtasPerSm * kMaxConsumerWarps * 8;  // of any tile variant
+size_t stencil_scratch_bytes(int num_sms) {
+    return kScratchHead + (size_t)num_sms * kMaxCtasPerSm * kMaxConsumerWarps * 8;
 }
 
 StencilPlan *stencil_plan_create_ext(const JacobiDims &d, const float *const coef[NCOEF], const float *p, float *wrk2,
@@ -1450,8 +1449,10 @@ extern "C" oo_status oo_stencil_noalloc_dev(oo_ctx *ctx, int I, int J, int K, in
         OO_CUDA_TRY(cudaSetDevice(c.device));
         // the plan lives on the host stack: tile variant and work split as
         // oo_stencil_dev chooses them (the context's option or tuned choice,
-        // else the default rule).  Grids beyond the documented limit are
-        // refused, though a sweep needs few of the static array's slots.
+        // else the default rule).  The sizes it takes are the interface's, by
+        // tile counts that a sweep's scratch no longer depends on: `shape` and
+        // the variant counted for an untuned grid are part of that limit, not
+        // what the sweep runs.
         {
             static const int shape[kNumVariants][3] = {  // tile_k, tile_j, consumer warps the limit counts
                 {128, 8, 8}, {128, 8, 16}, {128, 4, 8}, {64, 8, 4}, {64, 8, 8}};
@@ -1460,8 +1461,8 @@ extern "C" oo_status oo_stencil_noalloc_dev(oo_ctx *ctx, int I, int J, int K, in
             const long long cols = (long long)((K - 1 + shape[v][0] - 1) / shape[v][0]) *
                                    ((J - 2 + shape[v][1] - 1) / shape[v][1]);
             OO_REQUIRE(cols * shape[v][2] <= kStaticPartials, OO_EINVAL,
-                       "grid too large for the static scratch: ceil((K-1)/tile_k) * ceil((J-2)/tile_j) * consumer "
-                       "warps must be <= " + std::to_string(kStaticPartials));
+                       "grid too large for the allocation-free sweep: ceil((K-1)/tile_k) * ceil((J-2)/tile_j) * "
+                       "consumer warps must be <= " + std::to_string(kStaticPartials));
         }
         StencilPlan sp;
         sp.variant = c.stencil_variant_for(I, J, K);

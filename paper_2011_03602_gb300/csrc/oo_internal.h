@@ -368,12 +368,12 @@ int stencil_variant_count();
 // the variant a plan takes when none is chosen (by row length)
 int stencil_default_variant(const JacobiDims &d);
 // A plan whose scratch (counter, error word, partial residuals) lives in
-// caller-provided device memory of at least stencil_scratch_bytes(d, sms),
+// caller-provided device memory of at least stencil_scratch_bytes(sms),
 // cleared once (stencil_scratch_clear): a sweep leaves the counter at zero, and
 // plans that share the memory share its error word.
 StencilPlan *stencil_plan_create_ext(const JacobiDims &d, const float *const coef[NCOEF], const float *p, float *wrk2,
                                      int num_sms, void *scratch, size_t scratch_bytes, int variant = -1);
-size_t stencil_scratch_bytes(const JacobiDims &d, int num_sms);
+size_t stencil_scratch_bytes(int num_sms);  // for any grid and tile variant
 void stencil_scratch_clear(void *scratch, cudaStream_t s);
 void stencil_plan_destroy(StencilPlan *sp);
 // One stencil sweep; the residual (FP64) lands in *res_dev.

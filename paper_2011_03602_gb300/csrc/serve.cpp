@@ -107,7 +107,7 @@ void plan_sizes(Server &S, SReq &q) {
         q.h_out = hput(jd.n_host() * 4);
         q.h_res = hput((size_t)std::max(1, r.iters) * 8);
         d = (size_t)NARR * up256(jd.n_dev() * 4) + up256((size_t)std::max(1, r.iters) * 8) +
-            up256(stencil_scratch_bytes(jd, S.c->num_sms));
+            up256(stencil_scratch_bytes(S.c->num_sms));
     }
     q.h_err = hput(16);
     q.h_bytes = h;
@@ -188,7 +188,7 @@ void start(Server &S, SReq &q) {
         // before oo_serve_start) applies here too
         stencil_scratch_clear(scr, s);
         q.splan = stencil_plan_create_ext(d, coef, a[VAR_P], a[VAR_WRK2], c.num_sms, scr,
-                                          stencil_scratch_bytes(d, c.num_sms),
+                                          stencil_scratch_bytes(c.num_sms),
                                           c.stencil_variant_for((int)r.m, (int)r.n, (int)r.k));
         // the offload pattern with every nest on the GPU and hoisted copies:
         // nothing crosses until the final p and res
