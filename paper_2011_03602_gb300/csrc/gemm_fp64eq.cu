@@ -101,6 +101,8 @@ __device__ __forceinline__ void eq_tile(const EqArgs &a, int t, int &m0, int &n0
     n0 = (r / rows) * kBN;
 }
 
+// Single CTAs (OO_OPT_GEMM_PAIR = 0): what the CTA-pair kernel's bits are
+// compared with, so its roles and its store stay plain.
 __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_constant__ EqMaps maps,
                                                                  const __grid_constant__ EqArgs a) {
     extern __shared__ __align__(1024) unsigned char esm_raw[];

@@ -271,7 +271,10 @@ __global__ void bc_k_kernel(float *p, int rows, int K, int pitch) {
 // chunks of the i / j face rows, then the two ends of every interior row.
 // Bound by launch latency (3 us alone), so it is launched to run beside the
 // sweep, whose interior stores it does not touch; it ends only after the
-// sweep has (griddepcontrol.wait), so what follows it follows both.
+// sweep has (griddepcontrol.wait), so what follows it follows both.  It may start
+// before the sweep before that one, which reads this array, has ended: that is
+// safe because the faces hold these very values already, from the setup or from
+// two turns ago (in the first turn no sweep has read the array).
 __global__ void bc_faces_kernel(float *p, int I, int J, int K, int pitch) {
     const unsigned chunks = (unsigned)(K + 3) / 4u;
     const unsigned face_rows = 2u * J + 2u * (I - 2);
@@ -383,9 +386,9 @@ void launch_bc_faces(const JacobiDims &d, float *p, cudaStream_t s) {
 // N4 / N5 boundary) in one cooperative launch, for grids small enough that
 // launches, not HBM, bound the separate kernels.
 //
-// What bounds it: at 33 x 33 x 65 an SM holds 400 points, less than one per
-// thread, so an iteration is one point's chain (about 280 float-float
-// instructions, 19 loads) plus one exchange between SMs.  So:
+// At 33 x 33 x 65 an SM holds 400 points, less than one per thread, so an
+// iteration is one point's chain (about 280 float-float instructions, 19 loads)
+// plus one exchange between SMs.  So:
 //   - CTA b (one per SM) owns the same contiguous range of interior points
 //     in every iteration; their coefficients are read once and stay in its
 //     shared memory (12 x 4 bytes a point, the points beyond it read theirs
@@ -403,9 +406,12 @@ void launch_bc_faces(const JacobiDims &d, float *p, cudaStream_t s) {
 //   - one warp publishes and waits, another sums the residual while the
 //     sixteen others compute: FP64 adds run at 1/59 of the FP32 rate, and
 //     512 threads reducing in FP64 take as long as the stencil itself.
-// Two grid barriers, a copy pass and the coefficients from L2 in every
-// iteration took 14.2 us at 33 x 33 x 65; this takes 3.4 us, of which about
-// 3 are the exchange (a single CTA's worth of points takes 3.2).
+// With two grid barriers, a copy pass and the coefficients from L2 in every
+// iteration 50 iterations at 33 x 33 x 65 took 758 us with the call; 195 us so.
+// An iteration takes 3.0 us there (from 2000 and 4000 of them), as it does for
+// one point in one CTA (3.0) and for 20 CTAs of 256 points (2.8): what binds is
+// the chain of an iteration, loads behind a fence, one point's arithmetic, two
+// barriers, a release and a poll through L2, not points or neighbours.
 // Waits are bounded: one that runs out sets the error word and every CTA
 // leaves at its next wait.
 namespace {
