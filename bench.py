@@ -6,7 +6,8 @@ transfers -- the configuration the GA search at scale runs on.  One step is
 one whole pattern run (setup nests + 200 x [stencil, copy-back, two boundary
 nests]).  Metric: effective HBM GB/s of the pattern = algorithmic bytes of
 all nests / step time (stencil 56 B, copy-back 8 B per interior point and
-iteration; setup 56 B per point; faces 4 B per face point and iteration).
+iteration; setup 56 B per point; faces 4 B per face point and iteration), a
+work rate: the library exchanges p and wrk2 in place of the copy-back.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
@@ -536,6 +537,8 @@ def run_gpu(args):
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
             "data": "synthetic",
             "config": bench_config(ws),
+            "value_counts": "a work rate: the bytes of all nests of the program, the copy-back nest's too, which "
+                            "the exchange of p and wrk2 does not move; the stencil's own bandwidth is in roofline",
             "roofline": {"bound": "hbm", "kernel": "stencil (nest N2)",
                          "achieved": round(achieved, 1), "peak": peak, "peak_source": peak_src,
                          "unit": "GB/s", "frac": round(achieved / peak, 4), "traffic": traffic,

@@ -316,15 +316,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp64eq_kernel(const __grid_c
 // 2048 444 -> 356 us, 1024 118 -> 105 us with the splits.  A unit's epilogue takes
 // about as long as a K-block of 1024 terms' MMAs, so K-blocks are balanced
 // (eq::shape): 1000 x 777 x 1300 in blocks of 1024 + 320 159 us, 704 + 640
-// 144 us with both (wide tiles).  What binds now at n = 4096 is the tensor rate, 0.93 of
-// 1.9 PFLOP/s over the products' 3.85 PFLOP, under the power limit.
+// 144 us with both (wide tiles).  What binds now at n = 4096 is the tensor rate, 0.91 of
+// 1.96 PFLOP/s over the products' 3.85 PFLOP with the splits, under the power limit.
 // Narrow tiles, TN = 64: a unit is up to four slices of B against one of A,
 // beside each other in the same 256 accumulator columns, so that A_p's 16 KB
 // still come with up to 16 KB of B for 512 clocks of MMA a K step, and half
 // the columns need half the time: 1000 x 777 x 1300 is 28 wide tiles on 76
-// CTA pairs, 144 us with the splits, and 52 narrow ones, 92 us; 1024^3 105 ->
-// 72 us.  (64-column tiles of two-product units would stage 24 KB for 256
-// clocks of MMA, more than the 65 bytes a clock that one SM gets from L2.)
+// CTA pairs, 144 us with the splits, and 52 narrow ones, 92 us (90 with two
+// products added at once); 1024^3 105 -> 72 us.  (64-column tiles of two-product
+// units would stage 24 KB for 256 clocks of MMA, more than the 65 bytes a clock
+// that one SM gets from L2.)
 constexpr int kStagesPair = 6;
 constexpr uint32_t kStageBytesPair = 2 * kTile;  // A_p and this CTA's B tile
 
