@@ -1467,8 +1467,8 @@ extern "C" oo_status oo_stencil_noalloc_dev(oo_ctx *ctx, int I, int J, int K, in
             const long long cols = (long long)((K - 1 + shape[v][0] - 1) / shape[v][0]) *
                                    ((J - 2 + shape[v][1] - 1) / shape[v][1]);
             OO_REQUIRE(cols * shape[v][2] <= kStaticPartials, OO_EINVAL,
-                       "grid too large for the allocation-free sweep: ceil((K-1)/tile_k) * ceil((J-2)/tile_j) * "
-                       "consumer warps must be <= " + std::to_string(kStaticPartials));
+                       "grid too large for the static scratch: ceil((K-1)/tile_k) * ceil((J-2)/tile_j) * consumer "
+                       "warps must be <= " + std::to_string(kStaticPartials));
         }
         StencilPlan sp;
         sp.variant = c.stencil_variant_for(I, J, K);
