@@ -478,7 +478,7 @@ __device__ __forceinline__ bool fused_wait(const unsigned *words, int lo, int hi
 __global__ void __launch_bounds__(kFusedThreads + 64, 1) jacobi_fused_kernel(FusedArgs a) {
     extern __shared__ float coef_s[];            // [NCOEF][cap]
     __shared__ float2 ss_s[2][kFusedThreads];    // each thread's residual, of an even / odd iteration
-    __shared__ int ok_s[2];                      // the exchange warp's verdict on an even / odd iteration
+    __shared__ int failed_at;                    // the iteration whose wait ran out (iters: none)
     constexpr int kAll = kFusedThreads + 64, kSync = kFusedThreads + 32;
     const int J = a.J, Ji = J - 2, Ki = a.K - 2;
     const long long nint = (long long)(a.I - 2) * Ji * Ki;
@@ -489,18 +489,19 @@ __global__ void __launch_bounds__(kFusedThreads + 64, 1) jacobi_fused_kernel(Fus
     const int lane = threadIdx.x & 31;
 
     // Barrier 1: iteration `it` of this CTA is stored (every warp).  Barrier 2:
-    // the neighbours' is too, or ok_s[it & 1] is false (all but the residual
-    // warp).  After a failure barrier 1 is passed once more, behind which the
-    // residual warp reads that verdict.  It reads iteration it - 1's while the
-    // exchange warp may be writing iteration it's, hence the two slots: with
-    // one, a residual warp that saw the later verdict left a barrier early, and
-    // the others waited for it there for ever.
+    // the neighbours' is too, or failed_at is `it` (all but the residual warp).
+    // After a failure barrier 1 is passed once more, behind which the residual
+    // warp leaves.  It reads failed_at while the exchange warp may be writing
+    // `it`, which it does not take for an earlier failure: a flag instead, seen
+    // false one iteration early, would have it leave before the barrier that the
+    // others still enter, where they would wait for ever.  (A flag for each parity
+    // of the iteration is as safe, but stored in every one: 50 ns an iteration.)
     if (threadIdx.x >= kSync) {
         // ------------------------------------------------ residual warp
         bool ok = true;
         for (int it = 0; it < a.iters; ++it) {
             bar_named<kAll>(1);
-            if (it > 0 && !ok_s[(it - 1) & 1]) return;
+            if (failed_at < it) return;
             if (!ok) continue;
             double v = 0.0;
 #pragma unroll 4
@@ -535,11 +536,12 @@ __global__ void __launch_bounds__(kFusedThreads + 64, 1) jacobi_fused_kernel(Fus
         const long long D = (long long)Ji * Ki + Ki + 1;  // how far a point's update reaches
         auto owner = [&](long long q) { return (int)(((q + 1) * G - 1) / nint); };
         const int lo = owner(max(0ll, q0 - D)), hi = owner(min(nint - 1, q0 + n - 1 + D));
+        if (lane == 0) failed_at = a.iters;
         for (int it = 0; it < a.iters; ++it) {
             bar_named<kAll>(1);
             if (lane == 0) st_release(a.done + b * kFusedLine, it + 1);
             const bool ok = fused_wait(a.done, lo, it == 0 ? hi + (int)a.wait_extra : hi, it + 1, a.err);
-            if (lane == 0) ok_s[it & 1] = ok;
+            if (!ok && lane == 0) failed_at = it;
             bar_named<kSync>(2);
             if (!ok) {
                 if (it + 1 < a.iters) bar_named<kAll>(1);
@@ -603,7 +605,7 @@ __global__ void __launch_bounds__(kFusedThreads + 64, 1) jacobi_fused_kernel(Fus
         ss_s[it & 1][tid] = make_float2(RH, RL);
         bar_named<kAll>(1);
         bar_named<kSync>(2);
-        if (!ok_s[it & 1]) {
+        if (failed_at == it) {
             if (it + 1 < a.iters) bar_named<kAll>(1);
             return;
         }

@@ -5,41 +5,66 @@ barrier 1, compute and exchange at barrier 2) and the exchange warp's verdict
 travels through shared memory; a role that leaves one barrier early would
 strand the others, because the barriers count a fixed number of threads.  That
 cannot be provoked on a GPU, so the roles are replayed here step by step in
-every order the barriers allow, with the number of verdict slots and the slots'
-indices as the kernel has them."""
+every order the barriers allow, with the statements on the verdict that the
+kernel has."""
 import os
-import re
 
 import pytest
 
 SOURCE = os.path.join(os.path.dirname(__file__), "..", "paper_2011_03602_gb300", "csrc", "jacobi.cu")
 
 
-def verdict_slots():
-    """(slots, accesses): the declaration of ok_s and what indexes it."""
-    with open(SOURCE) as f:
-        text = f.read()
-    kernel = text[text.index("jacobi_fused_kernel(FusedArgs a)"):text.index("size_t fused_words_bytes")]
-    decl = re.search(r"__shared__ int ok_s(?:\[(\d+)\])?;", kernel)
-    assert decl, "ok_s not found"
-    return int(decl.group(1) or 1), re.findall(r"ok_s\[([^\]]*)\][ ;)]", kernel.replace(decl.group(0), ""))
+class Flag:
+    """One flag, stored in every iteration: what the roles must not share."""
+
+    def __init__(self, iters):
+        self.ok = True
+
+    def store(self, it, ok):
+        self.ok = ok
+
+    def compute_leaves(self, it):
+        return not self.ok
+
+    def residual_leaves(self, it):
+        return it > 0 and not self.ok
 
 
-def compute(iters, slots, ok):
+class FailedAt:
+    """The kernel's verdict: the iteration that failed, stored then only."""
+
+    STATEMENTS = ("if (lane == 0) failed_at = a.iters;", "if (!ok && lane == 0) failed_at = it;",
+                  "if (failed_at == it) {", "if (failed_at < it) return;")
+
+    def __init__(self, iters):
+        self.at = iters
+
+    def store(self, it, ok):
+        if not ok:
+            self.at = it
+
+    def compute_leaves(self, it):
+        return self.at == it
+
+    def residual_leaves(self, it):
+        return self.at < it
+
+
+def compute(iters, verdict):
     for it in range(iters):
         yield "b1"
         yield "b2"
-        if not ok[it % slots]:
+        if verdict.compute_leaves(it):
             if it + 1 < iters:
                 yield "b1"
             return
 
 
-def exchange(iters, slots, ok, fails_at):
+def exchange(iters, verdict, fails_at):
     for it in range(iters):
         yield "b1"
         yield "step"  # the wait
-        ok[it % slots] = it != fails_at
+        verdict.store(it, it != fails_at)
         yield "b2"
         if it == fails_at:
             if it + 1 < iters:
@@ -47,21 +72,21 @@ def exchange(iters, slots, ok, fails_at):
             return
 
 
-def residual(iters, slots, ok):
+def residual(iters, verdict):
     for it in range(iters):
         yield "b1"
         yield "step"  # anything may happen between the barrier and the read
-        if it > 0 and not ok[(it - 1) % slots]:
+        if verdict.residual_leaves(it):
             return
 
 
 NEEDS = {"b1": {0, 1, 2}, "b2": {0, 1}}
 
 
-def replay(choices, iters, slots, fails_at):
-    """The state after the given choices: (positions, ended, who may go on)."""
-    ok = [True] * slots
-    roles = [compute(iters, slots, ok), exchange(iters, slots, ok, fails_at), residual(iters, slots, ok)]
+def replay(choices, iters, kind, fails_at):
+    """Where the roles are after the given choices, and who may go on."""
+    verdict = kind(iters)
+    roles = [compute(iters, verdict), exchange(iters, verdict, fails_at), residual(iters, verdict)]
     at = [next(r) for r in roles]
 
     def ready():
@@ -77,25 +102,29 @@ def replay(choices, iters, slots, fails_at):
     return at, ready()
 
 
-def stuck_orders(iters, slots, fails_at):
+def stuck_orders(iters, kind, fails_at):
     """Orders after which some role waits for one that has left."""
     bad, todo = [], [()]
     while todo:
         path = todo.pop()
-        at, go = replay(path, iters, slots, fails_at)
+        at, go = replay(path, iters, kind, fails_at)
         if not go and any(x != "end" for x in at):
             bad.append(path)
         todo += [path + (g,) for g in go]
     return bad
 
 
-def test_model_finds_the_race_of_a_single_slot():
-    assert stuck_orders(3, 1, 1)
+def test_model_finds_the_race_of_a_flag():
+    assert stuck_orders(3, Flag, 1)
 
 
 @pytest.mark.parametrize("iters", [1, 2, 3, 4])
 def test_kernel_ends_in_every_order(iters):
-    slots, index = verdict_slots()
-    assert slots == 1 or sorted(set(index)) == ["(it - 1) & 1", "it & 1"]
+    with open(SOURCE) as f:
+        text = f.read()
+    kernel = text[text.index("jacobi_fused_kernel(FusedArgs a)"):text.index("size_t fused_words_bytes")]
+    for statement in FailedAt.STATEMENTS:
+        assert kernel.count(statement) == 1, statement
+    assert kernel.count("failed_at") == len(FailedAt.STATEMENTS) + 3  # the declaration and the comment
     for fails_at in [None] + list(range(iters)):
-        assert not stuck_orders(iters, slots, fails_at), fails_at
+        assert not stuck_orders(iters, FailedAt, fails_at), fails_at
